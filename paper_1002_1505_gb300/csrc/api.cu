@@ -124,6 +124,7 @@ struct dda_ctx {
   double* d_nh = nullptr;             // far-field directions
   double2* d_F = nullptr;             // far-field sums
   double* d_fpart = nullptr;          // far-field partial sums
+  float2* d_ftab = nullptr;           // far-field phase tables (many directions)
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // cached solver graphs (complex64, complex128)
   // A captured iteration graph holds device pointers and launch parameters by value.  `gen`
   // changes whenever a device buffer is (re)allocated or the launch schedule or geometry
@@ -1864,15 +1865,15 @@ dda_status dda_cross_sections(dda_ctx* c, const void* p_dev, double* q_out, cons
       const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
       e = grow(c, &c->d_nh, sizeof(double) * nh.size());
       if (e.ok()) e = grow(c, &c->d_F, sizeof(double2) * (size_t)nrhs * ndir * 3);
-      if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * 6 * (size_t)nrhs * ndir * nblk);
+      const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
+      if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * dda::farfield_scratch(nrhs, ndir, c->n, box, nblk));
       double2* d_F = c->d_F;
       if (e.ok()) {
         e = cuda_ok(cudaMemcpy(c->d_nh, nh.data(), sizeof(double) * nh.size(), cudaMemcpyHostToDevice),
                     "direction upload");
-        const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
         if (e.ok())
-          e = dda::farfield(c->d_ijk, c->d_origin, c->d_nh, k, P, nrhs, ndir, c->n, box, d_F, (double2*)c->d_fpart,
-                            nblk, c->stream);
+          e = dda::farfield(c->d_ijk, c->d_map, c->d_origin, c->d_nh, k, P, nrhs, c->iorth, ndir, c->n, box, d_F,
+                            c->d_fpart, nblk, c->stream);
       }
       std::vector<double2> F((size_t)nrhs * ndir * 3);
       if (e.ok()) {
@@ -1975,14 +1976,14 @@ dda_status dda_periodic_scattering(dda_ctx* c, const void* p_dev, int n_spec, co
     const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
     e = grow(c, &c->d_nh, sizeof(double) * nh.size());
     if (e.ok()) e = grow(c, &c->d_F, sizeof(double2) * (size_t)nrhs * ndir * 3);
-    if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * 6 * (size_t)nrhs * ndir * nblk);
+    const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
+    if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * dda::farfield_scratch(nrhs, ndir, c->n, box, nblk));
     if (e.ok())
       e = cuda_ok(cudaMemcpy(c->d_nh, nh.data(), sizeof(double) * nh.size(), cudaMemcpyHostToDevice),
                   "direction upload");
-    const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
     if (e.ok())
-      e = dda::farfield(c->d_ijk, c->d_origin, c->d_nh, k, P, nrhs, ndir, c->n, box, c->d_F, (double2*)c->d_fpart,
-                        nblk, c->stream);
+      e = dda::farfield(c->d_ijk, c->d_map, c->d_origin, c->d_nh, k, P, nrhs, c->iorth, ndir, c->n, box, c->d_F,
+                        c->d_fpart, nblk, c->stream);
     std::vector<double2> F((size_t)nrhs * ndir * 3);
     if (e.ok()) {
       e = cuda_ok(cudaMemcpyAsync(F.data(), c->d_F, sizeof(double2) * F.size(), cudaMemcpyDeviceToHost, c->stream),
@@ -2216,11 +2217,8 @@ dda_status dda_angular_averages(dda_ctx* c, const void* p_dev, double eta, doubl
     const std::vector<ScaDir> dirs = scattering_directions(k * aeff, eta);
     const int ndir = (int)dirs.size();
     const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
-    const int nt = box[0] + box[1] + box[2];
-    const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
-    const int nchunk = (ndir + 7) / 8;
-    // RHS per pass: phase tables under ~256 MB
-    const int per = (int)std::max<int64_t>(1, std::min<int64_t>(nrhs, (256ll << 20) / ((int64_t)ndir * nt * 8)));
+    const dda::FarPlan plan = dda::far_many_plan(c->n, box, nrhs, c->iorth, ndir);
+    const int per = plan.per;
     std::vector<double> nl((size_t)ndir * 3);
     for (int d = 0; d < ndir; ++d) {
       const double t = dirs[d].theta, f = dirs[d].phi;
@@ -2228,14 +2226,10 @@ dda_status dda_angular_averages(dda_ctx* c, const void* p_dev, double eta, doubl
       nl[3 * d + 1] = std::sin(t) * std::cos(f);
       nl[3 * d + 2] = std::sin(t) * std::sin(f);
     }
-    float2* d_tab = nullptr;
-    double* d_part = nullptr;
-    double* d_nh = nullptr;
-    double2* d_F = nullptr;
-    e = dalloc((char**)&d_tab, sizeof(float2) * (size_t)per * ndir * nt);
-    if (e.ok()) e = dalloc((char**)&d_part, sizeof(double) * (size_t)per * nchunk * nblk * 48);
-    if (e.ok()) e = dalloc((char**)&d_nh, sizeof(double) * (size_t)per * ndir * 3);
-    if (e.ok()) e = dalloc((char**)&d_F, sizeof(double2) * (size_t)per * ndir * 3);
+    e = grow(c, &c->d_ftab, plan.tab_bytes);
+    if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * plan.part_doubles);
+    if (e.ok()) e = grow(c, &c->d_nh, sizeof(double) * (size_t)per * ndir * 3);
+    if (e.ok()) e = grow(c, &c->d_F, sizeof(double2) * (size_t)per * ndir * 3);
     std::vector<double> nh((size_t)per * ndir * 3);
     std::vector<double2> F((size_t)per * ndir * 3);
     for (int b0 = 0; b0 < nrhs && e.ok(); b0 += per) {
@@ -2247,16 +2241,16 @@ dda_status dda_angular_averages(dda_ctx* c, const void* p_dev, double eta, doubl
           for (int q = 0; q < 3; ++q)
             nh[((size_t)bb * ndir + d) * 3 + q] = nl[3 * d] * ax[q] + nl[3 * d + 1] * ax[3 + q] + nl[3 * d + 2] * ax[6 + q];
       }
-      if (cudaMemcpyAsync(d_nh, nh.data(), sizeof(double) * (size_t)nb * ndir * 3, cudaMemcpyHostToDevice, c->stream) !=
+      if (cudaMemcpyAsync(c->d_nh, nh.data(), sizeof(double) * (size_t)nb * ndir * 3, cudaMemcpyHostToDevice, c->stream) !=
           cudaSuccess) {
         e = Err::make(DDA_ECUDA, "direction upload failed");
         break;
       }
       const double2* P = (const double2*)p_dev + (size_t)b0 * 3 * c->n;
-      e = dda::farfield_many(c->d_ijk, c->d_origin, d_nh, k, P, nb, ndir, c->n, box, d_tab, d_part, nblk, d_F,
-                             c->stream);
+      e = dda::farfield_many(c->d_ijk, c->d_map, c->d_origin, c->d_nh, k, P, nb, ndir, c->n, box, plan, c->d_ftab,
+                             c->d_fpart, c->d_F, c->stream);
       if (!e.ok()) break;
-      if (cudaMemcpyAsync(F.data(), d_F, sizeof(double2) * (size_t)nb * ndir * 3, cudaMemcpyDeviceToHost, c->stream) !=
+      if (cudaMemcpyAsync(F.data(), c->d_F, sizeof(double2) * (size_t)nb * ndir * 3, cudaMemcpyDeviceToHost, c->stream) !=
               cudaSuccess ||
           cudaStreamSynchronize(c->stream) != cudaSuccess) {
         e = Err::make(DDA_ECUDA, "far-field sums failed");
@@ -2290,10 +2284,6 @@ dda_status dda_angular_averages(dda_ctx* c, const void* p_dev, double eta, doubl
         for (int q = 0; q < 3; ++q) o[3 + q] = csum > 0 ? gv[q] / csum : 0.0;
       }
     }
-    dfree(d_tab);
-    dfree(d_part);
-    dfree(d_nh);
-    dfree(d_F);
     if (!e.ok()) return fail(c, e);
     if (ndir_out) *ndir_out = ndir;
     return DDA_OK;

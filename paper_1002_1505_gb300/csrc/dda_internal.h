@@ -334,16 +334,28 @@ Err qsums_tensor(const double2* einc, const double2* iat, double kd, const doubl
                  double* out3, RedBuf rb, cudaStream_t st);
 Err qsums(const uint8_t* comp, const double2* einc /*[nrhs][3][N]*/, const double2* ia, int ncomp, double kd,
           const double2* p, int nrhs, int64_t n, double* out3, RedBuf rb, cudaStream_t st);
-// F[rhs][dir][3] = sum_j P_j exp(-i kd n_dir . r_j); ndirs directions per RHS (nhat given per RHS, TF)
-Err farfield(const int32_t* ijk, const double* origin3, const double* nhat /*[nrhs][ndir][3]*/, double kd,
-             const double2* p, int nrhs, int ndir, int64_t n, const int box[3], double2* out, double2* part, int nblk,
-             cudaStream_t st);
-// Far field F = sum_j P_j exp(-i k n.r_j) for many directions (nhat [nrhs][ndir][3] in TF) from
-// separable FP32 phase tables (tab: nrhs*ndir*(box sum) float2; part: nrhs*ceil(ndir/8)*nblk*48
-// doubles); out [nrhs][ndir][3].
-Err farfield_many(const int32_t* ijk, const double* origin3, const double* nhat, double kd, const double2* p,
-                  int nrhs, int ndir, int64_t n, const int box[3], float2* tab, double* part, int nblk, double2* out,
-                  cudaStream_t st);
+// F[rhs][dir][3] = sum_j P_j exp(-i kd n_dir . r_j), FP64; ndir directions per RHS (nhat
+// [nrhs][ndir][3] in TF, the same for the iorth RHS of an orientation); map: box -> site;
+// scratch: farfield_scratch doubles.
+size_t farfield_scratch(int nrhs, int ndir, int64_t n, const int box[3], int nblk);
+Err farfield(const int32_t* ijk, const int32_t* map, const double* origin3, const double* nhat, double kd,
+             const double2* p, int nrhs, int iorth, int ndir, int64_t n, const int box[3], double2* out,
+             double* scratch, int nblk, cudaStream_t st);
+// The same for many directions, from separable FP32 phase tables.  The plan says how the sum is
+// organised (box rows or sites), how many RHS a pass takes (a multiple of iorth for rows) and the
+// sizes of tab and part; out [nrhs][ndir][3].
+struct FarPlan {
+  bool rows = false;
+  int nb = 1;              // polarizations per direction set
+  int per = 1;             // RHS per pass
+  int nblk = 1;            // row or site blocks
+  int64_t ndp = 0;         // table pitch in directions
+  size_t tab_bytes = 0, part_doubles = 0;
+};
+FarPlan far_many_plan(int64_t n, const int box[3], int nrhs, int iorth, int ndir);
+Err farfield_many(const int32_t* ijk, const int32_t* map, const double* origin3, const double* nhat, double kd,
+                  const double2* p, int nrhs, int ndir, int64_t n, const int box[3], const FarPlan& f, float2* tab,
+                  double* part, double2* out, cudaStream_t st);
 // Far-field moments for the radiative torque: out[rhs][d][12] = g (3 complex) and
 // T[c][a] = sum_j (r_j - r_cm)_c P_ja exp(-i k n.r_j) (9 complex); shift = origin - r_cm.
 Err farfield_moments(const int32_t* ijk, const double* origin3, const double* nhat, double kd, const double2* p,

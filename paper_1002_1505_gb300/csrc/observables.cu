@@ -255,6 +255,246 @@ __global__ void k_far_many_fin(const double* __restrict__ part, int nblk, int nc
   }
 }
 
+// ------------------------------------------------------------------ far field by box rows
+// The same sums organised by the box's x rows.  With c the row's centre and sites paired as
+// x = c -+ delta, sum_x P e^{-ik n_x x} = e^{-ik n_x c} sum_u [P+ cos(phi_u) + i P- sin(phi_u)], where
+// P+- = P(c + delta_u) +- P(c - delta_u) does not depend on the direction: four real products per
+// pair, component and direction instead of eight, and the y, z and centre phases are applied once
+// per row.  Tables per direction set (one per orientation; its nb polarizations share it):
+// tab[set][i][ndp], direction fastest, i = u (cos, sin of phi_u), then y (with the centre phase),
+// then z.  The work follows the box, so callers take it only for boxes that sites fill well
+// (far_by_rows).
+__device__ __forceinline__ double row_angle(const double* nh, const double* org, double kd, int nx, int i, int U,
+                                            int ny) {
+  const double c = 0.5 * (nx - 1);
+  if (i < U) return -kd * nh[0] * (c - i);
+  if (i < U + ny) return -kd * (nh[1] * ((double)(i - U) + org[1]) + nh[0] * (org[0] + c));
+  return -kd * nh[2] * ((double)(i - U - ny) + org[2]);
+}
+// RUN consecutive entries of one section per thread.  T2 = float2: the first entry and the step by
+// sincos, the others by FP64 products (error ~1e-15, far below the FP32 rounding of the entry);
+// T2 = double2: sincos each.
+constexpr int kRun = 16, kRun64 = 1;
+template <typename T2, int RUN>
+__global__ void k_row_tables(const double* __restrict__ nhat, int nb, int ndir, int ndp, const double* __restrict__ org,
+                             double kd, int nx, int ny, int nz, T2* __restrict__ tab) {
+  const int U = (nx + 1) / 2, nt = U + ny + nz;
+  const int d = blockIdx.x * blockDim.x + threadIdx.x, set = blockIdx.z;
+  if (d >= ndp) return;
+  int s = blockIdx.y, i0, i1;  // section run
+  const int ru = (U + RUN - 1) / RUN, ry = (ny + RUN - 1) / RUN;
+  if (s < ru) { i0 = s * RUN; i1 = min(U, i0 + RUN); }
+  else if (s < ru + ry) { i0 = U + (s - ru) * RUN; i1 = min(U + ny, i0 + RUN); }
+  else { i0 = U + ny + (s - ru - ry) * RUN; i1 = min(nt, i0 + RUN); }
+  const double* nh = nhat + ((int64_t)set * nb * ndir + min(d, ndir - 1)) * 3;
+  T2* out = tab + (int64_t)set * nt * ndp + d;
+  double sn, cs;
+  const double a0 = row_angle(nh, org, kd, nx, i0, U, ny);
+  sincos(a0, &sn, &cs);
+  if constexpr (sizeof(T2) == sizeof(float2)) {
+    double ws, wc;
+    sincos(i1 > i0 + 1 ? row_angle(nh, org, kd, nx, i0 + 1, U, ny) - a0 : 0.0, &ws, &wc);
+    for (int i = i0; i < i1; ++i) {
+      out[(int64_t)i * ndp] = make_float2((float)cs, (float)sn);
+      const double t = cs * wc - sn * ws;
+      sn = cs * ws + sn * wc;
+      cs = t;
+    }
+  } else {
+    for (int i = i0; i < i1; ++i) {
+      if (i > i0) sincos(row_angle(nh, org, kd, nx, i, U, ny), &sn, &cs);
+      out[(int64_t)i * ndp] = make_double2(cs, sn);
+    }
+  }
+}
+
+// running FP32 sum carried as a pair (two-sum)
+struct PairSum {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
+    hi = t;
+  }
+};
+
+// Many directions, FP32 products.  A thread owns two directions, a CTA 2 kRowT directions of one set
+// and a run of rows, staged in shared memory as P+ and P- pairs that every thread reads by broadcast;
+// a row's sum is FP32 (at most half the box's x length of terms), rows are added in pair sums.
+// Bound by FP32 issue and the broadcasts (48 FMAs per 6 LDS.128): 131,072 sites x 2292 directions x 2
+// polarizations in 0.30 ms, where the site kernel took 7.66 ms (three table lookups and two complex
+// products per site and direction, and 48 FP64 block sums per CTA at 1/64 of the FP32 rate).
+// grid (nblk, ndp / (2 kRowT), nsets); part[set][blk][nb * 6][ndp].
+constexpr int kRowT = 128;
+template <int NB>
+__global__ void __launch_bounds__(kRowT) k_far_rows(const int32_t* __restrict__ map, const double2* __restrict__ p,
+                                                    int64_t n, int nx, int ny, int nz, int ndp,
+                                                    const float2* __restrict__ tab, int rb, double* __restrict__ part) {
+  extern __shared__ float4 srow[];  // [rb][U][NB * 3]: P+ (re, im), P- (re, im)
+  constexpr int Q = NB * 3;
+  const int U = (nx + 1) / 2, nt = U + ny + nz, nrows = ny * nz;
+  int* occ = reinterpret_cast<int*>(srow + (size_t)rb * U * Q);
+  const int set = blockIdx.z, d0 = blockIdx.y * 2 * kRowT + threadIdx.x;
+  const int r_beg = (int)((int64_t)nrows * blockIdx.x / gridDim.x);
+  const int r_end = (int)((int64_t)nrows * (blockIdx.x + 1) / gridDim.x);
+  const float2* tx = tab + (int64_t)set * nt * ndp + d0;
+  PairSum acc[2][2 * Q];
+  for (int rb0 = r_beg; rb0 < r_end; rb0 += rb) {
+    const int nr = min(rb, r_end - rb0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr; i += kRowT) occ[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr * U; i += kRowT) {
+      const int r = i / U, u = i - r * U;
+      const int32_t* m = map + (int64_t)(rb0 + r) * nx;
+      const int32_t ia = m[u], ib = (nx - 1 - u != u) ? m[nx - 1 - u] : -1;
+      if (ia >= 0 || ib >= 0) occ[r] = 1;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const double2* pq = p + ((int64_t)set * Q + q) * n;
+        const double2 a = ia >= 0 ? pq[ia] : make_double2(0.0, 0.0);
+        const double2 b = ib >= 0 ? pq[ib] : make_double2(0.0, 0.0);
+        const bool mid = nx - 1 - u == u;  // its own partner: sin(phi_u) = 0
+        srow[(size_t)i * Q + q] = make_float4((float)(b.x + a.x), (float)(b.y + a.y), mid ? 0.f : (float)(b.x - a.x),
+                                              mid ? 0.f : (float)(b.y - a.y));
+      }
+    }
+    __syncthreads();
+    for (int r = 0; r < nr; ++r) {
+      if (!occ[r]) continue;
+      float row[2][2 * Q];
+#pragma unroll
+      for (int q = 0; q < 2 * Q; ++q) row[0][q] = row[1][q] = 0.f;
+      const float4* s = srow + (size_t)r * U * Q;
+#pragma unroll 4
+      for (int u = 0; u < U; ++u) {
+        const float2 t0 = __ldg(tx + (int64_t)u * ndp), t1 = __ldg(tx + (int64_t)u * ndp + kRowT);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const float4 v = s[u * Q + q];
+          row[0][2 * q] = fmaf(v.x, t0.x, fmaf(-v.w, t0.y, row[0][2 * q]));
+          row[0][2 * q + 1] = fmaf(v.y, t0.x, fmaf(v.z, t0.y, row[0][2 * q + 1]));
+          row[1][2 * q] = fmaf(v.x, t1.x, fmaf(-v.w, t1.y, row[1][2 * q]));
+          row[1][2 * q + 1] = fmaf(v.y, t1.x, fmaf(v.z, t1.y, row[1][2 * q + 1]));
+        }
+      }
+      const int iz = (rb0 + r) / ny, iy = (rb0 + r) - iz * ny;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float2 a = __ldg(tx + (int64_t)(U + iy) * ndp + k * kRowT);
+        const float2 b = __ldg(tx + (int64_t)(U + ny + iz) * ndp + k * kRowT);
+        const float2 ph = make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          acc[k][2 * q].add(fmaf(row[k][2 * q], ph.x, -row[k][2 * q + 1] * ph.y));
+          acc[k][2 * q + 1].add(fmaf(row[k][2 * q], ph.y, row[k][2 * q + 1] * ph.x));
+        }
+      }
+    }
+  }
+  double* o = part + ((int64_t)set * gridDim.x + blockIdx.x) * (2 * Q) * ndp + d0;
+#pragma unroll
+  for (int q = 0; q < 2 * Q; ++q) {
+    o[(int64_t)q * ndp] = (double)acc[0][q].hi + (double)acc[0][q].lo;
+    o[(int64_t)q * ndp + kRowT] = (double)acc[1][q].hi + (double)acc[1][q].lo;
+  }
+}
+
+// out[rhs][d][3] = the row blocks' partials in order; grid (ceil(ndir/256), nb * 6, nsets)
+__global__ void k_far_rows_fin(const double* __restrict__ part, int nblk, int ndir, int ndp, int nb,
+                               double2* __restrict__ out) {
+  const int d = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y, set = blockIdx.z;
+  if (d >= ndir) return;
+  double v = 0.0;
+#pragma unroll 8
+  for (int i = 0; i < nblk; ++i) v += part[(((int64_t)set * nblk + i) * (nb * 6) + q) * ndp + d];
+  double* o = reinterpret_cast<double*>(out + (((int64_t)set * nb + q / 6) * ndir + d) * 3);
+  o[q % 6] = v;
+}
+
+// Few directions, FP64 throughout: a thread owns a row (grid-strided) and kFarDirs directions, so the
+// direction-independent P+- are formed once per kFarDirs directions; the CTA's totals leave in the
+// layout of k_far's partials.  Bound by the FP64 pipe (12 products per pair and direction plus the
+// P+- sums): 131,072 sites x 38 directions x 2 polarizations in 0.19 ms, k_far 0.59 ms (20 products
+// per site and a table of sincos per CTA).  grid (row blocks, ceil(ndir / kFarDirs), nrhs).
+constexpr int kFarDirs = 4;
+constexpr int kFarT = 128;
+__global__ void __launch_bounds__(kFarT) k_far_rows64(const int32_t* __restrict__ map, const double2* __restrict__ p,
+                                                      int64_t n, int nx, int ny, int nz, int ndir, int nb,
+                                                      const double2* __restrict__ tab, double* __restrict__ part) {
+  extern __shared__ double2 sx[];  // [U][kFarDirs]
+  __shared__ double red[kFarDirs * 6][kFarT + 1];
+  const int U = (nx + 1) / 2, nt = U + ny + nz, nrows = ny * nz;
+  const int d0 = blockIdx.y * kFarDirs, b = blockIdx.z;
+  const double2* t = tab + (int64_t)(b / nb) * nt * ndir;
+  for (int i = threadIdx.x; i < U * kFarDirs; i += kFarT)
+    sx[i] = t[(int64_t)(i / kFarDirs) * ndir + min(d0 + i % kFarDirs, ndir - 1)];
+  __syncthreads();
+  double acc[kFarDirs][6];
+#pragma unroll
+  for (int k = 0; k < kFarDirs; ++k)
+#pragma unroll
+    for (int s = 0; s < 6; ++s) acc[k][s] = 0.0;
+  const double2* pb = p + (int64_t)b * 3 * n;
+  for (int r = blockIdx.x * kFarT + threadIdx.x; r < nrows; r += gridDim.x * kFarT) {
+    const int32_t* m = map + (int64_t)r * nx;
+    double row[kFarDirs][6];
+#pragma unroll
+    for (int k = 0; k < kFarDirs; ++k)
+#pragma unroll
+      for (int s = 0; s < 6; ++s) row[k][s] = 0.0;
+    for (int u = 0; u < U; ++u) {
+      const bool mid = nx - 1 - u == u;
+      const int32_t ia = m[u], ib = mid ? -1 : m[nx - 1 - u];
+      if (ia < 0 && ib < 0) continue;
+      double2 sp[3], sm[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double2 a = ia >= 0 ? pb[c * n + ia] : make_double2(0.0, 0.0);
+        const double2 e = ib >= 0 ? pb[c * n + ib] : make_double2(0.0, 0.0);
+        sp[c] = make_double2(e.x + a.x, e.y + a.y);
+        sm[c] = mid ? make_double2(0.0, 0.0) : make_double2(e.x - a.x, e.y - a.y);
+      }
+#pragma unroll
+      for (int k = 0; k < kFarDirs; ++k) {
+        const double2 w = sx[u * kFarDirs + k];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          row[k][2 * c] = fma(sp[c].x, w.x, fma(-sm[c].y, w.y, row[k][2 * c]));
+          row[k][2 * c + 1] = fma(sp[c].y, w.x, fma(sm[c].x, w.y, row[k][2 * c + 1]));
+        }
+      }
+    }
+    const int iz = r / ny, iy = r - iz * ny;
+#pragma unroll
+    for (int k = 0; k < kFarDirs; ++k) {
+      const int d = min(d0 + k, ndir - 1);
+      const double2 a = t[(int64_t)(U + iy) * ndir + d], e = t[(int64_t)(U + ny + iz) * ndir + d];
+      const double2 ph = make_double2(a.x * e.x - a.y * e.y, a.x * e.y + a.y * e.x);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        acc[k][2 * c] += row[k][2 * c] * ph.x - row[k][2 * c + 1] * ph.y;
+        acc[k][2 * c + 1] += row[k][2 * c] * ph.y + row[k][2 * c + 1] * ph.x;
+      }
+    }
+  }
+  // block totals: one column of `red` per thread, then four threads per value and a shuffle
+#pragma unroll
+  for (int k = 0; k < kFarDirs; ++k)
+#pragma unroll
+    for (int s = 0; s < 6; ++s) red[k * 6 + s][threadIdx.x] = acc[k][s];
+  __syncthreads();
+  if (threadIdx.x < kFarDirs * 24) {
+    const int v = threadIdx.x / 4, q = threadIdx.x % 4;
+    double s = 0.0;
+    for (int i = 0; i < kFarT / 4; ++i) s += red[v][q + 4 * i];
+    s += __shfl_down_sync(0xffffffffu, s, 2);
+    s += __shfl_down_sync(0xffffffffu, s, 1);
+    const int d = d0 + v / 6;
+    if (q == 0 && d < ndir) part[(((int64_t)b * ndir + d) * gridDim.x + blockIdx.x) * 6 + v % 6] = s;
+  }
+}
+
 // ------------------------------------------------------------------ radiative force and torque
 // Far-field moments for the torque: per (RHS, direction) g = sum_j P_j exp(-i k n.r_j) (3 complex)
 // and T[c][a] = sum_j (r_j - r_cm)_c P_ja exp(-i k n.r_j) (9 complex), from the same FP32 phase
@@ -580,24 +820,77 @@ Err torque_ext_sums(const int32_t* ijk, const double2* einc, const double2* p, i
   return Err::Ok();
 }
 
-Err farfield_many(const int32_t* ijk, const double* origin3, const double* nhat, double kd, const double2* p,
-                  int nrhs, int ndir, int64_t n, const int box[3], float2* tab, double* part, int nblk, double2* out,
-                  cudaStream_t st) {
+// The row-wise sums follow the box, the site-wise ones the sites: rows are taken while the box has at
+// most `most` positions per site.  Measured on a 48^3 box with a share f of its positions occupied,
+// rows against sites: 2292 directions, two polarizations, f = 1: 0.43 / 6.3 ms, 0.52: 0.36 / 2.8,
+// 0.27: 0.29 / 1.3 (the row time hardly falls with f, the site time is proportional, so they meet
+// near 16 positions per site; the line is at 8); 38 directions in FP64, f = 1: 0.28 / 0.58 ms,
+// 0.52: 0.27 / 0.35, 0.27: 0.27 / 0.22 (line at 2).  Rows longer than 700 would not fit the row
+// kernels' shared memory.
+constexpr int kRowsMost = 8, kRowsMost64 = 2;
+static bool far_by_rows(int64_t n, const int box[3], int most) {
+  return (int64_t)box[0] * box[1] * box[2] <= most * n && box[0] <= 700;
+}
+
+FarPlan far_many_plan(int64_t n, const int box[3], int nrhs, int iorth, int ndir) {
+  FarPlan f;
+  f.rows = far_by_rows(n, box, kRowsMost) && (iorth == 1 || iorth == 2);
+  f.nb = f.rows ? iorth : 1;
+  const int64_t nt = f.rows ? (int64_t)(box[0] + 1) / 2 + box[1] + box[2] : (int64_t)box[0] + box[1] + box[2];
+  f.ndp = f.rows ? (ndir + 2 * kRowT - 1) / (2 * kRowT) * (2 * kRowT) : ndir;
+  // direction sets per pass: phase tables under ~256 MB
+  const int64_t sets = std::max<int64_t>(1, std::min<int64_t>(nrhs / f.nb, (256ll << 20) / (f.ndp * nt * 8)));
+  f.per = (int)sets * f.nb;
+  f.tab_bytes = sizeof(float2) * (size_t)(sets * f.ndp * nt);
+  if (f.rows) {
+    // about ten CTAs per SM, at least four rows each
+    const int64_t tiles = (f.ndp / (2 * kRowT)) * sets;
+    f.nblk = (int)std::max<int64_t>(1, std::min<int64_t>({256, ((int64_t)box[1] * box[2] + 3) / 4,
+                                                          (1520 + tiles - 1) / tiles}));
+    f.part_doubles = (size_t)sets * f.nblk * f.nb * 6 * f.ndp;
+  } else {
+    f.nblk = (int)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, 64));
+    f.part_doubles = (size_t)f.per * ((ndir + kDirPerCta - 1) / kDirPerCta) * f.nblk * (kDirPerCta * 6);
+  }
+  return f;
+}
+
+Err farfield_many(const int32_t* ijk, const int32_t* map, const double* origin3, const double* nhat, double kd,
+                  const double2* p, int nrhs, int ndir, int64_t n, const int box[3], const FarPlan& f, float2* tab,
+                  double* part, double2* out, cudaStream_t st) {
   const int nt = box[0] + box[1] + box[2];
+  if (sizeof(float2) * (size_t)kDirPerCta * nt > 48 * 1024)
+    return Err::make(DDA_EUNSUPPORTED, "target box too long for the phase tables");
+  if (f.rows) {
+    const int nx = box[0], ny = box[1], nz = box[2], U = (nx + 1) / 2, sets = nrhs / f.nb;
+    auto runs = [](int v) { return (v + kRun - 1) / kRun; };
+    k_row_tables<float2, kRun><<<dim3((unsigned)((f.ndp + 127) / 128), runs(U) + runs(ny) + runs(nz), sets), 128, 0, st>>>(
+        nhat, f.nb, ndir, (int)f.ndp, origin3, kd, nx, ny, nz, tab);
+    DDA_CU(cudaGetLastError());
+    // rows staged at a time: about 24 KB (one row of the longest box, 384 pairs, takes 36 KB)
+    const size_t row_bytes = sizeof(float4) * (size_t)U * f.nb * 3;
+    const int rb = (int)std::max<size_t>(1, std::min<size_t>(32, 24576 / row_bytes));
+    const size_t sm = rb * row_bytes + sizeof(int) * rb;
+    const dim3 grid(f.nblk, (unsigned)(f.ndp / (2 * kRowT)), sets);
+    if (f.nb == 2) k_far_rows<2><<<grid, kRowT, sm, st>>>(map, p, n, nx, ny, nz, (int)f.ndp, tab, rb, part);
+    else k_far_rows<1><<<grid, kRowT, sm, st>>>(map, p, n, nx, ny, nz, (int)f.ndp, tab, rb, part);
+    DDA_CU(cudaGetLastError());
+    k_far_rows_fin<<<dim3((ndir + 255) / 256, f.nb * 6, sets), 256, 0, st>>>(part, f.nblk, ndir, (int)f.ndp, f.nb, out);
+    DDA_CU(cudaGetLastError());
+    add_launches(3);
+    return Err::Ok();
+  }
   const int64_t nrd = (int64_t)nrhs * ndir;
   const int tb = (int)std::min<int64_t>((nrd * nt + kT - 1) / kT, 152 * 32);
   k_phase_tables<<<tb, kT, 0, st>>>(nhat, nrd, origin3, kd, box[0], box[1], box[2], tab);
   DDA_CU(cudaGetLastError());
-  add_launches(1);
   const int nchunk = (ndir + kDirPerCta - 1) / kDirPerCta;
   const size_t sm = sizeof(float2) * (size_t)kDirPerCta * nt;
-  if (sm > 48 * 1024) return Err::make(DDA_EUNSUPPORTED, "target box too long for the phase tables");
-  k_far_many<<<dim3(nblk, nchunk, nrhs), kT, sm, st>>>(ijk, p, n, ndir, box[0], box[1], box[2], tab, part);
+  k_far_many<<<dim3(f.nblk, nchunk, nrhs), kT, sm, st>>>(ijk, p, n, ndir, box[0], box[1], box[2], tab, part);
   DDA_CU(cudaGetLastError());
-  add_launches(1);
-  k_far_many_fin<<<nrhs * nchunk, 64, 0, st>>>(part, nblk, nchunk, ndir, out);
+  k_far_many_fin<<<nrhs * nchunk, 64, 0, st>>>(part, f.nblk, nchunk, ndir, out);
   DDA_CU(cudaGetLastError());
-  add_launches(1);
+  add_launches(3);
   return Err::Ok();
 }
 
@@ -636,17 +929,44 @@ Err qsums_tensor(const double2* einc, const double2* iat, double kd, const doubl
   return Err::Ok();
 }
 
-Err farfield(const int32_t* ijk, const double* origin3, const double* nhat, double kd, const double2* p, int nrhs,
-             int ndir, int64_t n, const int box[3], double2* out, double2* part, int nblk, cudaStream_t st) {
-  double* pd = reinterpret_cast<double*>(part);
+// row blocks of the row-wise far field, and the doubles of scratch `farfield` needs (phase tables of
+// the row-wise path, then the partials)
+static int far_row_blocks(const int box[3]) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)box[1] * box[2] + kFarT - 1) / kFarT, 512));
+}
+size_t farfield_scratch(int nrhs, int ndir, int64_t n, const int box[3], int nblk) {
+  if (!far_by_rows(n, box, kRowsMost64)) return (size_t)6 * nrhs * ndir * nblk;
+  const size_t nt = (size_t)(box[0] + 1) / 2 + box[1] + box[2];
+  return (size_t)2 * nrhs * ndir * nt + (size_t)6 * nrhs * ndir * far_row_blocks(box);
+}
+
+Err farfield(const int32_t* ijk, const int32_t* map, const double* origin3, const double* nhat, double kd,
+             const double2* p, int nrhs, int iorth, int ndir, int64_t n, const int box[3], double2* out,
+             double* scratch, int nblk, cudaStream_t st) {
   const size_t sm = sizeof(double2) * (size_t)(box[0] + box[1] + box[2]);
   if (sm > 48 * 1024) return Err::make(DDA_EUNSUPPORTED, "target box too long for the far-field phase tables");
-  k_far<<<dim3(nblk, ndir, nrhs), kT, sm, st>>>(ijk, origin3, nhat, kd, p, ndir, n, box[0], box[1], box[2], pd);
+  if (far_by_rows(n, box, kRowsMost64) && ndir <= 65535 * kFarDirs && nrhs <= 65535) {
+    const int nx = box[0], ny = box[1], nz = box[2], U = (nx + 1) / 2, sets = nrhs / iorth;
+    const int nrb = far_row_blocks(box);
+    double2* tab = reinterpret_cast<double2*>(scratch);
+    double* part = scratch + 2 * (size_t)sets * ndir * (U + ny + nz);
+    auto runs = [](int v) { return (v + kRun64 - 1) / kRun64; };
+    k_row_tables<double2, kRun64><<<dim3((unsigned)((ndir + 31) / 32), runs(U) + runs(ny) + runs(nz), sets), 32, 0, st>>>(
+        nhat, iorth, ndir, ndir, origin3, kd, nx, ny, nz, tab);
+    DDA_CU(cudaGetLastError());
+    k_far_rows64<<<dim3(nrb, (ndir + kFarDirs - 1) / kFarDirs, nrhs), kFarT, sizeof(double2) * U * kFarDirs, st>>>(
+        map, p, n, nx, ny, nz, ndir, iorth, tab, part);
+    DDA_CU(cudaGetLastError());
+    k_far_fin<<<nrhs * ndir, kT, 0, st>>>(part, nrb, out);
+    DDA_CU(cudaGetLastError());
+    add_launches(3);
+    return Err::Ok();
+  }
+  k_far<<<dim3(nblk, ndir, nrhs), kT, sm, st>>>(ijk, origin3, nhat, kd, p, ndir, n, box[0], box[1], box[2], scratch);
   DDA_CU(cudaGetLastError());
-  add_launches(1);
-  k_far_fin<<<nrhs * ndir, kT, 0, st>>>(pd, nblk, out);
+  k_far_fin<<<nrhs * ndir, kT, 0, st>>>(scratch, nblk, out);
   DDA_CU(cudaGetLastError());
-  add_launches(1);
+  add_launches(2);
   return Err::Ok();
 }
 
