@@ -80,6 +80,18 @@ struct Geom {
   FftPlan plx, ply, plz;
 };
 
+// Fourier-space tensor in memory: the six components (xx, xy, xz, yy, yz, zz) of a spectral point as
+// 16-byte pieces (three for complex64, two components each; six for the 16-byte types), stored
+// [kx][kz][piece][ky]: threads on consecutive ky load consecutive 16-byte words.  (Records of six
+// contiguous components make the lanes of each 16-byte load 48 or 96 bytes apart, three to six times
+// the L1 wavefronts: z columns of 256 x 256 x 320 with 32 RHS 7.87 -> 7.62 ms.)  ghat_at: index of the first piece in 16-byte units; the next is py further.
+template <typename C>
+constexpr int kGhatPieces = 6 * (int)sizeof(C) / 16;
+template <typename C>
+__host__ __device__ inline int64_t ghat_at(int kx, int kz, int ky, int pz, int py) {
+  return ((int64_t)kx * pz + kz) * (kGhatPieces<C> * py) + ky;
+}
+
 struct KState;
 
 // Device-resident data shared by matvec kernels of one precision.
@@ -87,7 +99,7 @@ template <typename C>
 struct MvData {
   const int32_t* map;   // nx*ny*nz box -> site index or -1
   const uint8_t* comp;  // N x 3 compositions (0-based, per site and axis), may be null when ncomp == 1
-  const C* ghat;        // [px][py][pz][6] Fourier-space tensor (xx,xy,xz,yy,yz,zz), scaled by 1/M
+  const C* ghat;        // Fourier-space tensor (ghat_at), scaled by 1/M
   const C* ia;          // [nrhs][ncomp][3] diagonal of alpha^{-1}
   const C* twx;         // twiddles exp(-2 pi i j / L), L entries each
   const C* twy;

@@ -31,6 +31,30 @@ struct FftPlan {
   int len[kMaxStages];    // sub-transform length entering each DIF stage
 };
 
+// Stage list of an even 2,3,5-smooth length: a leading radix 2 (pruned stage for zero-padded data),
+// then the remaining power of two as radix-8 stages with one radix-4 or radix-2 stage for the
+// remainder (a radix 8 right after the leading radix 2 keeps the register sub-blocks of the second
+// pass short), then radix 3 and 5 stages.  Up to L = 320 (the compile-time transforms), a radix 2
+// follows the first 8 when more than 12 elements per sub-block would remain: the two can then be
+// taken together as a radix-16 first pass, which leaves sub-blocks of 8 or 10 instead of 16 or 20.
+// Returns the number of stages.
+constexpr int plan_radices(int L, int* r) {
+  int k = 0, rest = L / 2, a = 0;
+  r[k++] = 2;
+  while (rest % 2 == 0) { rest /= 2; ++a; }
+  if (L <= 320 && a >= 4 && (L / 16) > 12) {
+    r[k++] = 8;
+    r[k++] = 2;
+    a -= 4;
+  }
+  while (a >= 3) { r[k++] = 8; a -= 3; }
+  if (a == 2) r[k++] = 4;
+  else if (a == 1) r[k++] = 2;
+  while (rest % 3 == 0) { rest /= 3; r[k++] = 3; }
+  while (rest % 5 == 0) { rest /= 5; r[k++] = 5; }
+  return k;
+}
+
 #ifdef __CUDACC__
 // ------------------------------------------------------------------ complex helpers
 template <typename T> struct C2;

@@ -3,11 +3,14 @@
 // A length L = 2 * RA * LB transform (the same stage list as make_plan: a
 // radix-2 stage, then the plan's radices) is split into two passes, each done
 // in registers by one thread:
-//   pass A  stage 0 (radix 2) fused with stage 1 (radix RA).  Thread n1 in
-//           [0, LB) reads the RA inputs at n1 + LB*j and writes 2*RA outputs
-//           at b*L/2 + n1 + LB*k (b = 0, 1).  Forward, the upper half of the
-//           input is zero (zero padding), so stage 0 is y0 = x, y1 = x w^n.
+//   pass A  stage 0 (radix 2) fused with the NA stages after it, RA = the product
+//           of their radices (NA = 1 or 2).  Thread n1 in [0, LB) reads the RA
+//           inputs at n1 + LB*j and writes 2*RA outputs at b*L/2 + n1 + LB*k
+//           (b = 0, 1; k in the plan's digit order).  Forward, the upper half of
+//           the input is zero (zero padding), so stage 0 is y0 = x, y1 = x w^n.
 //   pass B  the remaining stages on one contiguous sub-block of LB elements.
+// Where the split lies changes neither the result's order nor its place, so
+// each kernel takes the split that suits it.
 // Forward passes are decimation in frequency and leave the spectrum in the
 // same digit-reversed order as the generic engine (fft.cuh); inverse passes
 // undo them exactly (decimation in time, conjugate twiddles, unnormalized),
@@ -30,35 +33,27 @@ struct CPlan {
   int r[kMaxStages];
 };
 
-// Compile-time copy of make_plan's stage list (targets.cpp): 2, then radix-8
-// stages for the remaining power of two with one radix 4 or 2 for the
-// remainder, then 3s and 5s.
 constexpr CPlan cplan(int L) {
   CPlan p{};
-  int k = 0;
-  int rest = L / 2;
-  p.r[k++] = 2;
-  int a = 0;
-  while (rest % 2 == 0) { rest /= 2; ++a; }
-  int r2[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  int n2 = 0;
-  while (a >= 3) { r2[n2++] = 8; a -= 3; }
-  if (a == 2) r2[n2++] = 4;
-  else if (a == 1) r2[n2++] = 2;
-  for (int i = 0; i < n2; ++i) p.r[k++] = r2[i];
-  while (rest % 3 == 0) { rest /= 3; p.r[k++] = 3; }
-  while (rest % 5 == 0) { rest /= 5; p.r[k++] = 5; }
-  p.nst = k;
+  int r[32]{};
+  p.nst = plan_radices(L, r);
+  for (int i = 0; i < p.nst; ++i) p.r[i] = r[i];
   return p;
 }
 
-template <int L>
+template <int L, int NA = 1>
 struct Shape {
   static constexpr CPlan P = cplan(L);
-  static constexpr int RA = P.nst > 1 ? P.r[1] : 1;  // radix fused with the radix-2 stage
+  static constexpr int R1 = P.nst > 1 ? P.r[1] : 1;             // radix fused with the radix-2 stage
+  static constexpr int R2 = (NA > 1 && P.nst > 2) ? P.r[2] : 1;  // and the one after it
+  static constexpr int RA = R1 * R2;
   static constexpr int LB = L / (2 * RA);             // sub-block length handled by pass B
   static constexpr int H = L / 2;
+  static constexpr int SB = P.nst > NA ? NA + 1 : P.nst;  // pass B's first stage
   static_assert(L % 2 == 0, "even lengths only");
+  static_assert(NA == 1 || NA == 2, "pass A takes one or two stages after the radix 2");
+  // natural frequency (mod RA) of pass A's output slot s: the digits of the two stages
+  static constexpr int nat(int s) { return s / R2 + R1 * (s % R2); }
 };
 
 // a + b * conj(w) as four FMAs (the last DIT stage when only one output half is kept)
@@ -68,68 +63,6 @@ __device__ __forceinline__ C addmulc(C a, C b, C w) {
   r.x = fma(b.x, w.x, fma(b.y, w.y, a.x));
   r.y = fma(b.y, w.x, fma(-b.x, w.y, a.y));
   return r;
-}
-
-// ------------------------------------------------------------------ pass A
-// x[j] = input at n1 + LB*j (upper half of the input is zero); out[b*RA+k] goes to b*H + n1 + LB*k.
-template <int L, typename C>
-__device__ __forceinline__ void passA_fwd(C* x, int n1, const C* tw, C* out) {
-  constexpr int RA = Shape<L>::RA, LB = Shape<L>::LB;
-  if constexpr (RA == 1) {
-    out[0] = x[0];
-    out[1] = cmul(x[0], tw[n1]);
-  } else {
-    C y[RA];
-#pragma unroll
-    for (int j = 0; j < RA; ++j) y[j] = cmul(x[j], tw[n1 + LB * j]);
-    Dft<RA, -1, C>::run(x);
-    Dft<RA, -1, C>::run(y);
-    out[0] = x[0];
-    out[RA] = y[0];
-#pragma unroll
-    for (int k = 1; k < RA; ++k) {
-      const C w = tw[2 * n1 * k];
-      out[k] = cmul(x[k], w);
-      out[RA + k] = cmul(y[k], w);
-    }
-  }
-}
-
-// in[b*RA+k] from b*H + n1 + LB*k; lo[j] = output at n1 + LB*j, hi[j] at H + n1 + LB*j (if HI).
-template <int L, bool HI, typename C>
-__device__ __forceinline__ void passA_inv(C* in, int n1, const C* tw, C* lo, C* hi) {
-  constexpr int RA = Shape<L>::RA, LB = Shape<L>::LB;
-  if constexpr (RA == 1) {
-    if constexpr (HI) {
-      const C t = cmulc(in[1], tw[n1]);
-      lo[0] = cadd(in[0], t);
-      hi[0] = csub(in[0], t);
-    } else {
-      lo[0] = addmulc(in[0], in[1], tw[n1]);
-    }
-  } else {
-    C u0[RA], u1[RA];
-    u0[0] = in[0];
-    u1[0] = in[RA];
-#pragma unroll
-    for (int k = 1; k < RA; ++k) {
-      const C w = tw[2 * n1 * k];
-      u0[k] = cmulc(in[k], w);
-      u1[k] = cmulc(in[RA + k], w);
-    }
-    Dft<RA, 1, C>::run(u0);
-    Dft<RA, 1, C>::run(u1);
-#pragma unroll
-    for (int j = 0; j < RA; ++j) {
-      if constexpr (HI) {
-        const C t = cmulc(u1[j], tw[n1 + LB * j]);
-        lo[j] = cadd(u0[j], t);
-        hi[j] = csub(u0[j], t);
-      } else {
-        lo[j] = addmulc(u0[j], u1[j], tw[n1 + LB * j]);  // pruned: the upper half is never needed
-      }
-    }
-  }
 }
 
 // ------------------------------------------------------------------ compile-time twiddles
@@ -216,13 +149,120 @@ constexpr int stage_len() {  // sub-transform length entering stage S
   return ls;
 }
 
+// The RA-point DFT of pass A in registers.  Forward: natural order in, pass A's slot order out (for
+// two stages R1, R2: slot k1 R2 + k2 holds frequency k1 + R1 k2); inverse: slots in, natural out.
+template <typename SH, int S, typename C>
+__device__ __forceinline__ void dftA(C* v) {
+  constexpr int R1 = SH::R1, R2 = SH::R2;
+  if constexpr (R2 == 1) {
+    Dft<R1, S, C>::run(v);
+  } else if constexpr (S < 0) {
+    C o[R1 * R2];
+    sfor<R2>([&](auto jc) {
+      constexpr int j2 = decltype(jc)::value;
+      C t[R1];
+#pragma unroll
+      for (int j = 0; j < R1; ++j) t[j] = v[j2 + R2 * j];
+      Dft<R1, S, C>::run(t);
+      sfor<R1>([&](auto kc) {
+        constexpr int k1 = decltype(kc)::value;
+        o[k1 * R2 + j2] = twc<R1 * R2, j2 * k1, S>(t[k1]);
+      });
+    });
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) Dft<R2, S, C>::run(o + k1 * R2);
+#pragma unroll
+    for (int i = 0; i < R1 * R2; ++i) v[i] = o[i];
+  } else {
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) Dft<R2, S, C>::run(v + k1 * R2);
+    C o[R1 * R2];
+    sfor<R2>([&](auto jc) {
+      constexpr int j2 = decltype(jc)::value;
+      C t[R1];
+      sfor<R1>([&](auto kc) {
+        constexpr int k1 = decltype(kc)::value;
+        t[k1] = twc<R1 * R2, j2 * k1, S>(v[k1 * R2 + j2]);
+      });
+      Dft<R1, S, C>::run(t);
+#pragma unroll
+      for (int j = 0; j < R1; ++j) o[j2 + R2 * j] = t[j];
+    });
+#pragma unroll
+    for (int i = 0; i < R1 * R2; ++i) v[i] = o[i];
+  }
+}
+
+// ------------------------------------------------------------------ pass A
+// x[j] = input at n1 + LB*j (upper half of the input is zero); out[b*RA+k] goes to b*H + n1 + LB*k.
+template <int L, int NA = 1, typename C>
+__device__ __forceinline__ void passA_fwd(C* x, int n1, const C* tw, C* out) {
+  using S = Shape<L, NA>;
+  constexpr int RA = S::RA, LB = S::LB;
+  if constexpr (RA == 1) {
+    out[0] = x[0];
+    out[1] = cmul(x[0], tw[n1]);
+  } else {
+    C y[RA];
+#pragma unroll
+    for (int j = 0; j < RA; ++j) y[j] = cmul(x[j], tw[n1 + LB * j]);
+    dftA<S, -1>(x);
+    dftA<S, -1>(y);
+    out[0] = x[0];
+    out[RA] = y[0];
+#pragma unroll
+    for (int k = 1; k < RA; ++k) {
+      const C w = tw[2 * n1 * S::nat(k)];
+      out[k] = cmul(x[k], w);
+      out[RA + k] = cmul(y[k], w);
+    }
+  }
+}
+
+// in[b*RA+k] from b*H + n1 + LB*k; lo[j] = output at n1 + LB*j, hi[j] at H + n1 + LB*j (if HI).
+template <int L, bool HI, int NA = 1, typename C>
+__device__ __forceinline__ void passA_inv(C* in, int n1, const C* tw, C* lo, C* hi) {
+  using S = Shape<L, NA>;
+  constexpr int RA = S::RA, LB = S::LB;
+  if constexpr (RA == 1) {
+    if constexpr (HI) {
+      const C t = cmulc(in[1], tw[n1]);
+      lo[0] = cadd(in[0], t);
+      hi[0] = csub(in[0], t);
+    } else {
+      lo[0] = addmulc(in[0], in[1], tw[n1]);
+    }
+  } else {
+    C u0[RA], u1[RA];
+    u0[0] = in[0];
+    u1[0] = in[RA];
+#pragma unroll
+    for (int k = 1; k < RA; ++k) {
+      const C w = tw[2 * n1 * S::nat(k)];
+      u0[k] = cmulc(in[k], w);
+      u1[k] = cmulc(in[RA + k], w);
+    }
+    dftA<S, 1>(u0);
+    dftA<S, 1>(u1);
+#pragma unroll
+    for (int j = 0; j < RA; ++j) {
+      if constexpr (HI) {
+        const C t = cmulc(u1[j], tw[n1 + LB * j]);
+        lo[j] = cadd(u0[j], t);
+        hi[j] = csub(u0[j], t);
+      } else {
+        lo[j] = addmulc(u0[j], u1[j], tw[n1 + LB * j]);  // pruned: the upper half is never needed
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ pass B
 // DIF stage S of the plan applied to one sub-block v[LB] (all indices compile-time).
-template <int L, int S, typename C>
+template <int L, int S, int LB, typename C>
 __device__ __forceinline__ void passB_fwd_stage(C* v) {
   constexpr CPlan P = Shape<L>::P;
   if constexpr (S < P.nst) {
-    constexpr int LB = Shape<L>::LB;
     constexpr int R = P.r[S];
     constexpr int Ls = stage_len<L, S>();
     constexpr int m = Ls / R;
@@ -242,16 +282,15 @@ __device__ __forceinline__ void passB_fwd_stage(C* v) {
         });
       });
     });
-    passB_fwd_stage<L, S + 1>(v);
+    passB_fwd_stage<L, S + 1, LB>(v);
   }
 }
 
-template <int L, int S, typename C>
+template <int L, int S, int LB, typename C>
 __device__ __forceinline__ void passB_inv_stage(C* v) {
   constexpr CPlan P = Shape<L>::P;
   if constexpr (S < P.nst) {
-    passB_inv_stage<L, S + 1>(v);  // inverse runs the stages backwards
-    constexpr int LB = Shape<L>::LB;
+    passB_inv_stage<L, S + 1, LB>(v);  // inverse runs the stages backwards
     constexpr int R = P.r[S];
     constexpr int Ls = stage_len<L, S>();
     constexpr int m = Ls / R;
@@ -274,13 +313,13 @@ __device__ __forceinline__ void passB_inv_stage(C* v) {
   }
 }
 
-template <int L, typename C>
+template <int L, int NA = 1, typename C>
 __device__ __forceinline__ void passB_fwd(C* v, const C* /*tw: unused, twiddles are compile-time*/) {
-  passB_fwd_stage<L, 2>(v);
+  passB_fwd_stage<L, Shape<L, NA>::SB, Shape<L, NA>::LB>(v);
 }
-template <int L, typename C>
+template <int L, int NA = 1, typename C>
 __device__ __forceinline__ void passB_inv(C* v, const C* /*tw*/) {
-  passB_inv_stage<L, 2>(v);
+  passB_inv_stage<L, Shape<L, NA>::SB, Shape<L, NA>::LB>(v);
 }
 
 }  // namespace f2

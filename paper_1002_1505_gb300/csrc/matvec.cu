@@ -38,10 +38,14 @@ __device__ __forceinline__ void load_tw(C* dst, const C* src, int L) {
   for (int i = threadIdx.x; i < L; i += blockDim.x) dst[i] = src[i];
 }
 
-// u = Ghat v, Ghat symmetric with components (xx, xy, xz, yy, yz, zz)
+// u = Ghat v, Ghat symmetric with components (xx, xy, xz, yy, yz, zz) from their 16-byte pieces
 template <typename C>
-__device__ __forceinline__ void gmul(const C* gh, C& v0, C& v1, C& v2) {
-  const C g0 = gh[0], g1 = gh[1], g2 = gh[2], g3 = gh[3], g4 = gh[4], g5 = gh[5];
+__device__ __forceinline__ void gmul(const C* ghat, int64_t at, int py, C& v0, C& v1, C& v2) {
+  constexpr int per = 16 / (int)sizeof(C);
+  const C* gh = ghat + at * per;
+  const int64_t st = (int64_t)py * per;
+  const C g0 = gh[0], g1 = gh[per == 2 ? 1 : st], g2 = gh[per == 2 ? st : 2 * st];
+  const C g3 = gh[per == 2 ? st + 1 : 3 * st], g4 = gh[per == 2 ? 2 * st : 4 * st], g5 = gh[per == 2 ? 2 * st + 1 : 5 * st];
   C u0 = cadd(cadd(cmul(g0, v0), cmul(g1, v1)), cmul(g2, v2));
   C u1 = cadd(cadd(cmul(g1, v0), cmul(g3, v1)), cmul(g4, v2));
   C u2 = cadd(cadd(cmul(g2, v0), cmul(g4, v1)), cmul(g5, v2));
@@ -161,10 +165,9 @@ __device__ __forceinline__ void zcol_process(C* col, const Geom& g, const MvData
     const int gg = i % G, kz = i / G;
     const int ky = ky0 + gg;
     if (ky >= g.py) continue;
-    const C* gh = d.ghat + (((int64_t)kx * g.pz + kz) * g.py + ky) * 6;
     C* e = col + (kz * 3) * G + gg;
     C v0 = e[0], v1 = e[G], v2 = e[2 * G];
-    gmul(gh, v0, v1, v2);
+    gmul(d.ghat, ghat_at<C>(kx, kz, ky, g.pz, g.py), g.py, v0, v1, v2);
     e[0] = v0;
     e[G] = v1;
     e[2 * G] = v2;
@@ -390,8 +393,9 @@ __global__ void k_green_expand_y(Geom g, const int32_t* __restrict__ stx, const 
   }
 }
 
-// f[c][z][ky][kx] (all z; natural ky <= Py/2, kx <= Px/2) from t[c][zq][sty[ky]][kx]:
-// planes z > Pz/2 mirror Pz - z with the z parity
+// f[c][z][kx][ky] (all z; natural kx <= Px/2, ky <= Py/2) from t[c][zq][sty[ky]][kx]:
+// planes z > Pz/2 mirror Pz - z with the z parity.  ky runs fastest because the pack below reads
+// every element four times with consecutive ky (in storage order) per warp.
 __global__ void k_green_expand_z(Geom g, const int32_t* __restrict__ sty, const double2* __restrict__ t,
                                  double2* __restrict__ f) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
@@ -401,7 +405,7 @@ __global__ void k_green_expand_z(Geom g, const int32_t* __restrict__ sty, const 
     const int64_t i = o - c * F;
     const int z = (int)(i / P);
     const int64_t r = i - (int64_t)z * P;
-    const int ky = (int)(r / hx1), kx = (int)(r - (int64_t)ky * hx1);
+    const int kx = (int)(r / hy1), ky = (int)(r - (int64_t)kx * hy1);
     const bool mir = z > g.pz / 2;
     const int zs = mir ? g.pz - z : z;
     double2 v = t[(int64_t)c * T + ((int64_t)zs * g.py + sty[ky]) * hx1 + kx];
@@ -410,33 +414,49 @@ __global__ void k_green_expand_z(Geom g, const int32_t* __restrict__ sty, const 
   }
 }
 
-// ghat[kx][kz][ky][6] (storage positions) = f[c][kz][ky'][kx'] / M, with kx', ky' the natural
-// frequencies folded into [0, P/2] and the sign of the parities of the folds
+// the six components of one spectral point, scaled, into the complex128, complex64 and double-float
+// tensors (ghat_at); consecutive threads write consecutive 16-byte words of every piece
+__device__ __forceinline__ void ghat_put(const double2 (&w)[6], int kx, int kz, int ky, int pz, int py,
+                                         double2* __restrict__ g128, float2* __restrict__ g64,
+                                         dfp::dfc* __restrict__ gdf) {
+  const int64_t a16 = ghat_at<double2>(kx, kz, ky, pz, py), a8 = ghat_at<float2>(kx, kz, ky, pz, py);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) g128[a16 + (int64_t)c * py] = w[c];
+  float4* q = reinterpret_cast<float4*>(g64) + a8;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+    q[(int64_t)c * py] = make_float4((float)w[2 * c].x, (float)w[2 * c].y, (float)w[2 * c + 1].x, (float)w[2 * c + 1].y);
+  if (gdf) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) gdf[a16 + (int64_t)c * py] = dfp::from_c128(w[c]);
+  }
+}
+
+// Ghat (storage positions) = f[c][kz][kx'][ky'] / M, with kx', ky' the natural frequencies folded
+// into [0, P/2] and the sign of the parities of the folds.  One thread per spectral point, ky
+// fastest; grid (ceil(py / blockDim), pz, px).  Bound by the three tensors it writes (240 bytes a
+// point).
 __global__ void k_green_pack(Geom g, const int32_t* __restrict__ natx, const int32_t* __restrict__ naty,
                              const double2* __restrict__ f, double2* __restrict__ g128, float2* __restrict__ g64,
                              dfp::dfc* __restrict__ gdf) {
-  const int64_t M = (int64_t)g.px * g.py * g.pz;
+  const int ky = blockIdx.x * blockDim.x + threadIdx.x, kz = blockIdx.y, kx = blockIdx.z;
+  if (ky >= g.py) return;
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1;
   const int64_t P = (int64_t)hx1 * hy1, F = P * g.pz;
-  const double inv = 1.0 / (double)M;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < 6 * M; o += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(o % 6);
-    const int64_t pt = o / 6;
-    const int ky = (int)(pt % g.py);
-    const int64_t rest = pt / g.py;
-    const int kz = (int)(rest % g.pz), kx = (int)(rest / g.pz);
-    int nx = natx[kx], ny = naty[ky];
-    const bool fx = nx > g.px / 2, fy = ny > g.py / 2;
-    if (fx) nx = g.px - nx;
-    if (fy) ny = g.py - ny;
-    double2 v = f[(int64_t)c * F + (int64_t)kz * P + (int64_t)ny * hx1 + nx];
-    const bool neg = (fx && odd_in(c, 0)) != (fy && odd_in(c, 1));
-    const double sc = neg ? -inv : inv;
-    const double2 w = make_double2(v.x * sc, v.y * sc);
-    g128[o] = w;
-    g64[o] = make_float2((float)w.x, (float)w.y);
-    if (gdf) gdf[o] = dfp::from_c128(w);
+  const double inv = 1.0 / ((double)g.px * g.py * g.pz);
+  int nx = natx[kx], ny = naty[ky];
+  const bool fx = nx > g.px / 2, fy = ny > g.py / 2;
+  if (fx) nx = g.px - nx;
+  if (fy) ny = g.py - ny;
+  const double2* src = f + (int64_t)kz * P + (int64_t)nx * hy1 + ny;
+  double2 w[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const double2 v = src[(int64_t)c * F];
+    const double sc = (fx && odd_in(c, 0)) != (fy && odd_in(c, 1)) ? -inv : inv;
+    w[c] = make_double2(v.x * sc, v.y * sc);
   }
+  ghat_put(w, kx, kz, ky, g.pz, g.py, g128, g64, gdf);
 }
 
 // natural frequency of storage position p of an in-place DIF transform with this plan:
@@ -653,7 +673,6 @@ void green_perm_tables(const Geom& g, std::vector<int32_t>* out) {
 Err build_green(const Geom& g, double kd, const double2* twx, const double2* twy, const double2* twz,
                 const int32_t* perm, double2* gw, double2* ghat128, float2* ghat64, dfp::dfc* ghatdf,
                 cudaStream_t st) {
-  const int64_t M = (int64_t)g.px * g.py * g.pz;
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
   const int64_t Q = (int64_t)g.px * hy1 * hz1, T = (int64_t)hx1 * g.py * hz1, F = (int64_t)hx1 * hy1 * g.pz;
   auto nblk = [](int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); };
@@ -685,7 +704,8 @@ Err build_green(const Geom& g, double kd, const double2* twx, const double2* twy
   if (e.ok())
     e = fft_strided<double2>(gw, g.pz, (int64_t)hx1 * hy1, (int64_t)hx1 * hy1, 6, F, g.plz, twz, false, st);
   if (e.ok()) {
-    k_green_pack<<<nblk(6 * M), 256, 0, st>>>(g, d_natx, d_naty, gw, ghat128, ghat64, ghatdf);
+    k_green_pack<<<dim3((g.py + 127) / 128, g.pz, g.px), std::min(128, (g.py + 31) / 32 * 32), 0, st>>>(
+        g, d_natx, d_naty, gw, ghat128, ghat64, ghatdf);
     if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green pack failed");
   }
   g_launches += 4;
@@ -767,23 +787,20 @@ __global__ void __launch_bounds__(kPbcT) k_green_fill_pbc(Geom g, double kd, dou
   }
 }
 
-// ghat[kx][kz][ky][6] (storage positions) = gw[c][kz][ky][kx] / M after the full transform
+// Ghat (storage positions) = gw[c][kz][ky][kx] / M after the full transform; grid as k_green_pack
 __global__ void k_green_pack_full(Geom g, const double2* __restrict__ f, double2* __restrict__ g128,
                                   float2* __restrict__ g64, dfp::dfc* __restrict__ gdf) {
+  const int ky = blockIdx.x * blockDim.x + threadIdx.x, kz = blockIdx.y, kx = blockIdx.z;
+  if (ky >= g.py) return;
   const int64_t M = (int64_t)g.px * g.py * g.pz;
   const double inv = 1.0 / (double)M;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < 6 * M; o += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(o % 6);
-    const int64_t pt = o / 6;
-    const int ky = (int)(pt % g.py);
-    const int64_t rest = pt / g.py;
-    const int kz = (int)(rest % g.pz), kx = (int)(rest / g.pz);
+  double2 w[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
     const double2 v = f[(int64_t)c * M + ((int64_t)kz * g.py + ky) * g.px + kx];
-    const double2 w = make_double2(v.x * inv, v.y * inv);
-    g128[o] = w;
-    g64[o] = make_float2((float)w.x, (float)w.y);
-    if (gdf) gdf[o] = dfp::from_c128(w);
+    w[c] = make_double2(v.x * inv, v.y * inv);
   }
+  ghat_put(w, kx, kz, ky, g.pz, g.py, g128, g64, gdf);
 }
 }  // namespace
 
@@ -804,8 +821,8 @@ Err build_green_pbc(const Geom& g, double kd, const double k_tf[3], double py, d
   DDA_TRY(fft_rows<double2>(gw, 6 * (int64_t)g.py * g.pz, g.px, g.plx, twx, g.px, g.px, false, st));
   DDA_TRY(fft_strided<double2>(gw, g.py, g.px, g.px, 6 * (int64_t)g.pz, (int64_t)g.px * g.py, g.ply, twy, false, st));
   DDA_TRY(fft_strided<double2>(gw, g.pz, (int64_t)g.px * g.py, (int64_t)g.px * g.py, 6, M, g.plz, twz, false, st));
-  const int nb = (int)std::min<int64_t>((6 * M + 255) / 256, 152 * 16);
-  k_green_pack_full<<<nb, 256, 0, st>>>(g, gw, ghat128, ghat64, ghatdf);
+  k_green_pack_full<<<dim3((g.py + 127) / 128, g.pz, g.px), std::min(128, (g.py + 31) / 32 * 32), 0, st>>>(
+      g, gw, ghat128, ghat64, ghatdf);
   if (cudaGetLastError() != cudaSuccess) return Err::make(DDA_ECUDA, "periodic Green pack failed");
   g_launches += 2;
   return Err::Ok();

@@ -107,7 +107,6 @@ __global__ void __launch_bounds__(ClusterCfg<S>::NT, ClusterCfg<S>::MINB) k_yz_c
   }
   __syncthreads();
   // z pass B, Ghat, inverse z pass B in registers for the three components
-  const C* gk = d.ghat + (int64_t)kx * PZ * PY * 6 + (int64_t)h * PYS * 6;
   for (int i = threadIdx.x; i < PYS * 2 * RAz; i += NT) {
     const int ky = i % PYS, blk = i / PYS;
     C v0[LBz], v1[LBz], v2[LBz];
@@ -122,7 +121,8 @@ __global__ void __launch_bounds__(ClusterCfg<S>::NT, ClusterCfg<S>::MINB) k_yz_c
     f2::passB_fwd<PZ>(v1, twz);
     f2::passB_fwd<PZ>(v2, twz);
 #pragma unroll
-    for (int e = 0; e < LBz; ++e) gmul3(gk + ((int64_t)(blk * LBz + e) * PY + ky) * 6, v0[e], v1[e], v2[e]);
+    for (int e = 0; e < LBz; ++e)
+      gmul3(d.ghat, ghat_at<C>(kx, blk * LBz + e, h * PYS + ky, PZ, PY), PY, v0[e], v1[e], v2[e]);
     f2::passB_inv<PZ>(v0, twz);
     f2::passB_inv<PZ>(v1, twz);
     f2::passB_inv<PZ>(v2, twz);

@@ -4,7 +4,8 @@
 // 3x3 Ghat multiply and the inverse pass B in registers, and global loads and
 // stores are arranged so that consecutive threads touch consecutive addresses.
 //
-// Ghat layout: [kx][kz][ky][6] (xx, xy, xz, yy, yz, zz), scaled by 1/M.
+// Ghat layout: ghat_at (dda_internal.h): (xx, xy, xz, yy, yz, zz) of a spectral point in 16-byte
+// pieces [kx][kz][piece][ky], scaled by 1/M.
 // Workspace:   W[b][c][kx][z][ys], ys = ny (3-pass) or py (5-pass).
 //
 // The templates take the compute type C: float2 (complex64), double2
@@ -29,17 +30,19 @@ using f2::Shape;
 template <typename C>
 __device__ __forceinline__ C conjc(C a) { a.y = -a.y; return a; }
 
+// one Ghat record (GhatAt, dda_internal.h): the six components sit in 16-byte pieces one row of ky
+// apart, so that consecutive ky load consecutive 16-byte words
 template <typename C>
-__device__ __forceinline__ void load6(const C* __restrict__ gh, C (&g)[6]) {
-  if constexpr (sizeof(C) == 8) {  // 48 bytes, 16-byte aligned: three 128-bit loads
-    const float4* q = reinterpret_cast<const float4*>(gh);
-    const float4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
+__device__ __forceinline__ void load6(const C* __restrict__ gh, int64_t at, int py, C (&g)[6]) {
+  const float4* q = reinterpret_cast<const float4*>(gh) + at;
+  if constexpr (sizeof(C) == 8) {
+    const float4 a = __ldg(q), b = __ldg(q + py), c = __ldg(q + 2 * py);
     g[0] = make_float2(a.x, a.y); g[1] = make_float2(a.z, a.w);
     g[2] = make_float2(b.x, b.y); g[3] = make_float2(b.z, b.w);
     g[4] = make_float2(c.x, c.y); g[5] = make_float2(c.z, c.w);
   } else {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) g[i] = gh[i];
+    for (int i = 0; i < 6; ++i) g[i] = *reinterpret_cast<const C*>(q + i * py);
   }
 }
 
@@ -65,15 +68,10 @@ __device__ __forceinline__ void gmul3_r(const C (&gg)[6], C& v0, C& v1, C& v2) {
 }
 
 template <typename C>
-__device__ __forceinline__ void gmul3(const C* __restrict__ gh, C& v0, C& v1, C& v2) {
+__device__ __forceinline__ void gmul3(const C* __restrict__ gh, int64_t at, int py, C& v0, C& v1, C& v2) {
   C gg[6];
-  load6(gh, gg);
-  const C u0 = cdot3(gg[0], v0, gg[1], v1, gg[2], v2);
-  const C u1 = cdot3(gg[1], v0, gg[3], v1, gg[4], v2);
-  const C u2 = cdot3(gg[2], v0, gg[4], v1, gg[5], v2);
-  v0 = u0;
-  v1 = u1;
-  v2 = u2;
+  load6(gh, at, py, gg);
+  gmul3_r(gg, v0, v1, v2);
 }
 
 // true when RHS b of this launch belongs to a finished solve (whole CTA exits before any barrier)
@@ -497,7 +495,6 @@ __global__ void __launch_bounds__(NT) k_yz_plane(Geom g, MvData<C> d) {
   }
   __syncthreads();
   // z pass B, Ghat, inverse z pass B -- in registers for the three components
-  const C* gk = d.ghat + (int64_t)kx * PZ * PY * 6;
   for (int i = threadIdx.x; i < PY * 2 * RAz; i += blockDim.x) {
     const int ky = i % PY, blk = i / PY;
     C v0[LBz], v1[LBz], v2[LBz];
@@ -512,7 +509,8 @@ __global__ void __launch_bounds__(NT) k_yz_plane(Geom g, MvData<C> d) {
     f2::passB_fwd<PZ>(v1, twz);
     f2::passB_fwd<PZ>(v2, twz);
 #pragma unroll
-    for (int e = 0; e < LBz; ++e) gmul3(gk + ((int64_t)(blk * LBz + e) * PY + ky) * 6, v0[e], v1[e], v2[e]);
+    for (int e = 0; e < LBz; ++e)
+      gmul3(d.ghat, ghat_at<C>(kx, blk * LBz + e, ky, PZ, PY), PY, v0[e], v1[e], v2[e]);
     f2::passB_inv<PZ>(v0, twz);
     f2::passB_inv<PZ>(v1, twz);
     f2::passB_inv<PZ>(v2, twz);
@@ -691,45 +689,47 @@ __global__ void __launch_bounds__(256) k_y_rows(Geom g, C* __restrict__ work, co
 // each pass-B sub-block of LB positions: in pass B a warp touches G consecutive columns of several
 // sub-blocks at once, and for complex64 with G = 8 and an even LB the unpadded sub-blocks all start
 // on the same shared-memory bank, which doubles the wavefronts of every such warp access.
-// RFUSE: pass B, the Ghat multiply and the inverse pass B of all three components in registers
-// even for long sub-blocks (one item per thread: NT = G * 2 * RA threads, up to 3 CTAs per SM),
-// which halves the shared-memory traffic of the column pass at the cost of occupancy.
-template <typename C, int PZ, int G>
+// Pass B, the Ghat multiply and the inverse pass B of all three components stay in registers
+// (kFuse) where the sub-blocks are short enough; else pass B and the multiply go through shared
+// memory.  NA = 2 takes two stages after the radix 2 into pass A (radix 16), which shortens the
+// sub-blocks of the long transforms to 8 and 10 elements so that they fuse (256 x 256 x 320, 32 RHS:
+// 8.40 -> 7.87 ms; with the coalesced Ghat pieces 7.62 ms).
+template <typename C, int PZ, int G, int NA>
 constexpr int zcols_pad() {
   // complex64: a warp's column group spans 2G words; when that is under the 32 banks, place
   // consecutive sub-blocks one group width apart (mod 32 words)
   if constexpr (sizeof(C) != 8 || 2 * G >= 32) {
     return 0;
   } else {
-    constexpr int gw = 2 * G, stride = (Shape<PZ>::LB * 3 * G * 2) % 32;
+    constexpr int gw = 2 * G, stride = (Shape<PZ, NA>::LB * 3 * G * 2) % 32;
     return ((gw - stride + 32) % 32) / 2;
   }
 }
-template <typename C, int PZ, int G>
+template <typename C, int PZ, int G, int NA>
 constexpr size_t zcols_smem_elems() {
-  return (size_t)PZ + (size_t)PZ * 3 * G + (size_t)2 * Shape<PZ>::RA * zcols_pad<C, PZ, G>();
+  return (size_t)PZ + (size_t)PZ * 3 * G + (size_t)2 * Shape<PZ, NA>::RA * zcols_pad<C, PZ, G, NA>();
+}
+// stages of pass A after the radix 2: two for the complex64 lengths whose sub-blocks would
+// otherwise be too long to fuse
+template <typename C, int PZ>
+constexpr int zcols_na() {
+  return (sizeof(C) == 8 && Shape<PZ, 1>::LB > 12 && Shape<PZ, 2>::LB >= 2) ? 2 : 1;
 }
 
-// CTAs per SM the register budget is sized for: the fused variants 3; the complex64 kernel whose
-// pass B goes through shared memory as many as its shared tile allows (up to 3), so that registers
-// do not cap its occupancy below what shared memory permits
-template <typename C, int PZ, int G, bool RFUSE>
+// CTAs per SM the register budget is sized for: 2 in complex64 (128 registers; without the cap the
+// Pz = 128 .. 192 kernels take 167 to 211 and run one CTA per SM: 128^3, 32 RHS 0.91 -> 0.65 ms,
+// 192^3, 16 RHS 1.81 -> 1.36 ms); the narrow variant 3
+template <typename C, int PZ, int NT, int NA>
 constexpr int zcols_min_ctas() {
-  if constexpr (RFUSE) {
-    return 3;
-  } else if constexpr (sizeof(C) == 8 && Shape<PZ>::LB * sizeof(C) > 96) {
-    constexpr size_t b = sizeof(C) * zcols_smem_elems<C, PZ, G>() + 1024;
-    return b * 3 <= 228 * 1024 ? 3 : (b * 2 <= 228 * 1024 ? 2 : 1);
-  } else {
-    return 1;
-  }
+  return sizeof(C) == 8 ? (NT < 256 ? 3 : 2) : 1;
 }
 
-template <typename C, int PZ, int G, int NT = 256, bool RFUSE = false>
-__global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_cols(Geom g, MvData<C> d) {
-  constexpr int RA = Shape<PZ>::RA, LB = Shape<PZ>::LB, H = Shape<PZ>::H;
-  constexpr int P = zcols_pad<C, PZ, G>();  // spare elements after each sub-block
-  constexpr bool kFuse = RFUSE || (LB * sizeof(C) <= 96);
+template <typename C, int PZ, int G, int NT = 256, int NA = zcols_na<C, PZ>()>
+__global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, NT, NA>())) k_z_cols(Geom g, MvData<C> d) {
+  using SZ = Shape<PZ, NA>;
+  constexpr int RA = SZ::RA, LB = SZ::LB, H = SZ::H;
+  constexpr int P = zcols_pad<C, PZ, G, NA>();  // spare elements after each sub-block
+  constexpr bool kFuse = LB * sizeof(C) <= 96;
   pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
         const int gg = i % G, r = i / G;
         const int c = r % 3, n1 = r / 3;
         C o[2 * RA];
-        f2::passA_fwd<PZ>(xa[it], n1, tw, o);
+        f2::passA_fwd<PZ, NA>(xa[it], n1, tw, o);
 #pragma unroll
         for (int bb = 0; bb < 2; ++bb)
 #pragma unroll
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
         const int zz = n1 + LB * j;
         x[j] = (zz < nz && ky < py) ? wb[c * cstride + (int64_t)zz * g.ys + ky] : czero<C>();
       }
-      f2::passA_fwd<PZ>(x, n1, tw, o);
+      f2::passA_fwd<PZ, NA>(x, n1, tw, o);
 #pragma unroll
       for (int bb = 0; bb < 2; ++bb)
 #pragma unroll
@@ -795,7 +795,6 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
     }
   }
   __syncthreads();
-  const C* gk = d.ghat + (int64_t)kx * PZ * py * 6;
   if constexpr (kFuse) {
     for (int i = threadIdx.x; i < G * 2 * RA; i += blockDim.x) {
       const int gg = i % G, blk = i / G;
@@ -808,16 +807,17 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
         v1[e] = q[G];
         v2[e] = q[2 * G];
       }
-      f2::passB_fwd<PZ>(v0, tw);
-      f2::passB_fwd<PZ>(v1, tw);
-      f2::passB_fwd<PZ>(v2, tw);
+      f2::passB_fwd<PZ, NA>(v0, tw);
+      f2::passB_fwd<PZ, NA>(v1, tw);
+      f2::passB_fwd<PZ, NA>(v2, tw);
       if (ky < py) {
 #pragma unroll
-        for (int e = 0; e < LB; ++e) gmul3(gk + ((int64_t)(blk * LB + e) * py + ky) * 6, v0[e], v1[e], v2[e]);
+        for (int e = 0; e < LB; ++e)
+          gmul3(d.ghat, ghat_at<C>(kx, blk * LB + e, ky, PZ, py), py, v0[e], v1[e], v2[e]);
       }
-      f2::passB_inv<PZ>(v0, tw);
-      f2::passB_inv<PZ>(v1, tw);
-      f2::passB_inv<PZ>(v2, tw);
+      f2::passB_inv<PZ, NA>(v0, tw);
+      f2::passB_inv<PZ, NA>(v1, tw);
+      f2::passB_inv<PZ, NA>(v2, tw);
 #pragma unroll
       for (int e = 0; e < LB; ++e) {
         C* q = s + ((blk * LB + e) * 3) * G + gg + blk * P;
@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
       C v[LB];
 #pragma unroll
       for (int e = 0; e < LB; ++e) v[e] = s[((blk * LB + e) * 3 + c) * G + gg + blk * P];
-      f2::passB_fwd<PZ>(v, tw);
+      f2::passB_fwd<PZ, NA>(v, tw);
 #pragma unroll
       for (int e = 0; e < LB; ++e) s[((blk * LB + e) * 3 + c) * G + gg + blk * P] = v[e];
     }
@@ -850,7 +850,7 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
         const int i = i0 + u * blockDim.x;
         const int gg = i % G, kz = i / G;
         ok[u] = i < PZ * G && ky0 + gg < py;
-        if (ok[u]) load6(gk + ((int64_t)kz * py + ky0 + gg) * 6, gv[u]);
+        if (ok[u]) load6(d.ghat, ghat_at<C>(kx, kz, ky0 + gg, PZ, py), py, gv[u]);
       }
 #pragma unroll
       for (int u = 0; u < kGBatch; ++u) {
@@ -873,7 +873,7 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
       C v[LB];
 #pragma unroll
       for (int e = 0; e < LB; ++e) v[e] = s[((blk * LB + e) * 3 + c) * G + gg + blk * P];
-      f2::passB_inv<PZ>(v, tw);
+      f2::passB_inv<PZ, NA>(v, tw);
 #pragma unroll
       for (int e = 0; e < LB; ++e) s[((blk * LB + e) * 3 + c) * G + gg + blk * P] = v[e];
     }
@@ -890,7 +890,7 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, G, RFUSE>())) k_z_c
     for (int bb = 0; bb < 2; ++bb)
 #pragma unroll
       for (int k = 0; k < RA; ++k) v[bb * RA + k] = s[((bb * H + n1 + LB * k) * 3 + c) * G + gg + (bb * RA + k) * P];
-    f2::passA_inv<PZ, false>(v, n1, tw, lo, (C*)nullptr);
+    f2::passA_inv<PZ, false, NA>(v, n1, tw, lo, (C*)nullptr);
     if (ky < py) {
 #pragma unroll
       for (int j = 0; j < RA; ++j) {
@@ -985,7 +985,7 @@ size_t yrows_fast_smem(const Geom& g) {
 template <typename C>
 size_t zcols_fast_smem(const Geom& g) {
   switch (g.pz) {
-#define DDA_CASE(L_) case L_: return sizeof(C) * zcols_smem_elems<C, L_, zcols_g_rt(sizeof(C), L_)>();
+#define DDA_CASE(L_) case L_: return sizeof(C) * zcols_smem_elems<C, L_, zcols_g_rt(sizeof(C), L_), zcols_na<C, L_>()>();
     DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
     default: return sizeof(C) * ((size_t)g.pz + (size_t)g.pz * 3 * zcols_g_rt(sizeof(C), g.pz));
@@ -1102,26 +1102,22 @@ Err launch_y_rows(const Geom& g, C* work, const C* tw, int64_t nrows, bool inv, 
   return Err::Ok();
 }
 
-// register-fused z columns (RFUSE): complex64 lengths whose pass-B sub-block is too long for the
-// default fused loop; 8 columns per CTA, one (column, sub-block) item per thread
+// narrow z columns (tuner candidate, complex64, Pz = 160): 8 columns per CTA and one (column,
+// sub-block) item per thread, 128 threads, three CTAs per SM
 constexpr int kZrG = 8;
 template <typename C>
 constexpr bool zcols_rfuse_exists(int pz) {
-  return sizeof(C) == 8 && (pz == 160 || pz == 320);
+  return sizeof(C) == 8 && pz == 160;
 }
 
 template <typename C>
 Err launch_z_cols(const Geom& g, const MvData<C>& d, int nrhs, cudaStream_t st, bool rfuse = false) {
   if constexpr (sizeof(C) == 8) {
     if (rfuse && zcols_rfuse_exists<C>(g.pz)) {
-      const size_t sm = sizeof(C) * (g.pz == 160 ? zcols_smem_elems<C, 160, kZrG>() : zcols_smem_elems<C, 320, kZrG>());
+      constexpr int NT = kZrG * 2 * Shape<160>::RA;
+      const size_t sm = sizeof(C) * zcols_smem_elems<C, 160, kZrG, 1>();
       const dim3 grid(nrhs, (g.py + kZrG - 1) / kZrG, g.px);
-      if (g.pz == 160)
-        DDA_CU(launch_k(k_z_cols<C, 160, kZrG, kZrG * 2 * Shape<160>::RA, true>, grid,
-                        dim3(kZrG * 2 * Shape<160>::RA), sm, st, g, d));
-      else
-        DDA_CU(launch_k(k_z_cols<C, 320, kZrG, kZrG * 2 * Shape<320>::RA, true>, grid,
-                        dim3(kZrG * 2 * Shape<320>::RA), sm, st, g, d));
+      DDA_CU(launch_k(k_z_cols<C, 160, kZrG, NT, 1>, grid, dim3(NT), sm, st, g, d));
       DDA_CU(cudaGetLastError());
       return Err::Ok();
     }
@@ -1175,8 +1171,7 @@ void optin_all(int smax) {
   optin_smem(k_yz_plane<C, A, B, 768, false>, smax);
     DDA_FAST_PLANES(DDA_CASE)
 #undef DDA_CASE
-    optin_smem(k_z_cols<C, 160, kZrG, kZrG * 2 * Shape<160>::RA, true>, smax);
-    optin_smem(k_z_cols<C, 320, kZrG, kZrG * 2 * Shape<320>::RA, true>, smax);
+    optin_smem(k_z_cols<C, 160, kZrG, kZrG * 2 * Shape<160>::RA, 1>, smax);
   }
 }
 

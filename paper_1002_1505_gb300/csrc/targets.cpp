@@ -241,28 +241,16 @@ bool is_smooth235(int v) {
   return v == 1;
 }
 
-// Stage list: a leading radix 2 (pruned stage for zero-padded data), then the
-// remaining power of two as radix-8 stages with one radix-4 or radix-2 stage
-// for the remainder (a radix 8 right after the leading radix 2 keeps the
-// register sub-blocks of the second pass short), then radix 3 and 5 stages.
+// Stage list of plan_radices (fft.cuh), shared with the compile-time transforms.
 Err make_plan(int L, FftPlan* out) {
   if (L < 2 || (L % 2) != 0 || !is_smooth235(L))
     return Err::make(DDA_EINVAL, "FFT length must be even and a product of 2, 3 and 5");
   FftPlan p{};
   p.L = L;
-  int k = 0;
-  int rest = L / 2;
-  p.radix[k++] = 2;
-  int a = 0;
-  while (rest % 2 == 0) { rest /= 2; ++a; }
-  std::vector<int> r2;
-  while (a >= 3) { r2.push_back(8); a -= 3; }
-  if (a == 2) r2.push_back(4);
-  else if (a == 1) r2.push_back(2);
-  for (int r : r2) p.radix[k++] = r;
-  while (rest % 3 == 0) { rest /= 3; p.radix[k++] = 3; }
-  while (rest % 5 == 0) { rest /= 5; p.radix[k++] = 5; }
+  int r[32];  // L < 2^31: at most 31 prime factors
+  const int k = plan_radices(L, r);
   if (k > kMaxStages) return Err::make(DDA_EINVAL, "FFT length needs too many stages");
+  for (int s = 0; s < k; ++s) p.radix[s] = r[s];
   p.nst = k;
   int len = L;
   for (int s = 0; s < k; ++s) {
