@@ -63,9 +63,10 @@ template <> struct C2<double> { using t = double2; };
 
 __host__ __device__ __forceinline__ float2 mk(float a, float b) { return make_float2(a, b); }
 __host__ __device__ __forceinline__ double2 mk(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+// complex64 sums on the packed FP32 instructions (one issue slot for both parts; the same roundings)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
@@ -83,6 +84,20 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
 template <typename C> __device__ __forceinline__ C cscale(C a, decltype(a.x) s) { C r; r.x = a.x * s; r.y = a.y * s; return r; }
 // multiply by i*s (s = +1 or -1)
 template <typename C> __device__ __forceinline__ C cmuli(C a, int s) { C r; r.x = -s * a.y; r.y = s * a.x; return r; }
+// a + i s b (s = +1 or -1), without forming i b
+template <typename C> __device__ __forceinline__ C caddi(C a, C b, int s) {
+  C r;
+  r.x = s > 0 ? a.x - b.y : a.x + b.y;
+  r.y = s > 0 ? a.y + b.x : a.y - b.x;
+  return r;
+}
+// r a + b, r real
+template <typename C> __device__ __forceinline__ C cfma(decltype(C::x) r, C a, C b) {
+  return mk(fma(r, a.x, b.x), fma(r, a.y, b.y));
+}
+template <> __device__ __forceinline__ float2 cfma<float2>(float r, float2 a, float2 b) {
+  return __ffma2_rn(make_float2(r, r), a, b);
+}
 template <typename C> __device__ __forceinline__ C czero() { C r; r.x = 0; r.y = 0; return r; }
 
 // ------------------------------------------------------------------ small DFTs
@@ -103,9 +118,7 @@ template <int S, typename C> struct Dft<3, S, C> {
     const R h = (R)(S * 0.86602540378443864676);  // S sin(2 pi / 3)
     const C s = cadd(v[1], v[2]);
     const C d = csub(v[1], v[2]);
-    C m;  // x0 - s/2
-    m.x = fma((R)-0.5, s.x, v[0].x);
-    m.y = fma((R)-0.5, s.y, v[0].y);
+    const C m = cfma((R)-0.5, s, v[0]);  // x0 - s/2
     v[0] = cadd(v[0], s);
     // outputs m +- i h d, one FMA per real part
     v[1] = mk(fma(-h, d.y, m.x), fma(h, d.x, m.y));
@@ -115,12 +128,12 @@ template <int S, typename C> struct Dft<3, S, C> {
 
 template <int S, typename C> struct Dft<4, S, C> {
   static __device__ __forceinline__ void run(C* v) {
-    C a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
-    C c = cadd(v[1], v[3]), d = cmuli(csub(v[1], v[3]), S);
+    const C a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+    const C c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
     v[0] = cadd(a, c);
     v[2] = csub(a, c);
-    v[1] = cadd(b, d);
-    v[3] = csub(b, d);
+    v[1] = caddi(b, d, S);
+    v[3] = caddi(b, d, -S);
   }
 };
 
@@ -131,18 +144,18 @@ template <int S, typename C> struct Dft<5, S, C> {
     const R c2 = (R)-0.80901699437494742410;  // cos(4 pi/5)
     const R s1 = (R)0.95105651629515357212;   // sin(2 pi/5)
     const R s2 = (R)0.58778525229247312917;   // sin(4 pi/5)
-    C p1 = cadd(v[1], v[4]), m1 = csub(v[1], v[4]);
-    C p2 = cadd(v[2], v[3]), m2 = csub(v[2], v[3]);
-    C x0 = v[0];
-    C a1 = cadd(x0, cadd(cscale(p1, c1), cscale(p2, c2)));
-    C a2 = cadd(x0, cadd(cscale(p1, c2), cscale(p2, c1)));
-    C b1 = cmuli(cadd(cscale(m1, s1), cscale(m2, s2)), S);
-    C b2 = cmuli(csub(cscale(m1, s2), cscale(m2, s1)), S);
+    const C p1 = cadd(v[1], v[4]), m1 = csub(v[1], v[4]);
+    const C p2 = cadd(v[2], v[3]), m2 = csub(v[2], v[3]);
+    const C x0 = v[0];
+    const C a1 = cfma(c1, p1, cfma(c2, p2, x0));
+    const C a2 = cfma(c2, p1, cfma(c1, p2, x0));
+    const C b1 = cfma(s1, m1, cscale(m2, s2));
+    const C b2 = cfma(s2, m1, cscale(m2, -s1));
     v[0] = cadd(x0, cadd(p1, p2));
-    v[1] = cadd(a1, b1);
-    v[4] = csub(a1, b1);
-    v[2] = cadd(a2, b2);
-    v[3] = csub(a2, b2);
+    v[1] = caddi(a1, b1, S);
+    v[4] = caddi(a1, b1, -S);
+    v[2] = caddi(a2, b2, S);
+    v[3] = caddi(a2, b2, -S);
   }
 };
 
@@ -158,15 +171,14 @@ template <int S, typename C> struct Dft<8, S, C> {
     // The 1/sqrt2 factor is folded into the butterflies' FMAs.
     const C a1 = mk(o[1].x - S * o[1].y, o[1].y + S * o[1].x);  // (1 + iS) o1
     const C a3 = mk(-o[3].x - S * o[3].y, S * o[3].x - o[3].y);  // (-1 + iS) o3
-    const C o2 = cmuli(o[2], S);
     v[0] = cadd(e[0], o[0]);
     v[4] = csub(e[0], o[0]);
-    v[1] = mk(fma(r2, a1.x, e[1].x), fma(r2, a1.y, e[1].y));
-    v[5] = mk(fma(-r2, a1.x, e[1].x), fma(-r2, a1.y, e[1].y));
-    v[2] = cadd(e[2], o2);
-    v[6] = csub(e[2], o2);
-    v[3] = mk(fma(r2, a3.x, e[3].x), fma(r2, a3.y, e[3].y));
-    v[7] = mk(fma(-r2, a3.x, e[3].x), fma(-r2, a3.y, e[3].y));
+    v[1] = cfma(r2, a1, e[1]);
+    v[5] = cfma(-r2, a1, e[1]);
+    v[2] = caddi(e[2], o[2], S);
+    v[6] = caddi(e[2], o[2], -S);
+    v[3] = cfma(r2, a3, e[3]);
+    v[7] = cfma(-r2, a3, e[3]);
   }
 };
 
