@@ -329,12 +329,14 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
   __syncthreads();
   const C* ia = d.ia + (int64_t)(rhs0 + b) * g.ncomp * 3;
   [[maybe_unused]] kred::AccF re, im, tt;
-  // kXU elements per thread per round, site indices first (independent loads in flight); as in
-  // the forward gather, 8 for x lengths of 256 and more, 4 below
+  // kXU elements per thread per round, site indices first, then the input values (independent loads
+  // in flight: 256 x 256 x 320, 32 RHS 1.81 -> 1.69 ms); as in the forward gather, 8 for x lengths of
+  // 256 and more, 4 below
   constexpr int kXU = PX >= 256 ? 8 : 4;
   for (RowWalk w(g.nx); w.r < NC * TY;) {
    int32_t idxs[kXU];
    int rs[kXU], xs[kXU];
+   typename Io<C>::t pvs[kXU];
 #pragma unroll
    for (int u = 0; u < kXU; ++u) {
      rs[u] = w.r;
@@ -344,6 +346,9 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
      w.next(g.nx);
    }
 #pragma unroll
+   for (int u = 0; u < kXU; ++u)
+     pvs[u] = idxs[u] >= 0 ? p[((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u]] : typename Io<C>::t{};
+#pragma unroll
    for (int u = 0; u < kXU; ++u) {
     const int32_t idx = idxs[u];
     if (idx < 0) continue;
@@ -352,7 +357,7 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
     const int c = c0 + cl;
     const int64_t o = ((int64_t)b * 3 + c) * g.n + idx;
     const int cc = d.comp ? d.comp[3 * idx + c] : 0;  // composition of axis c
-    C pv = io_get<C>(p[o]);
+    C pv = io_get<C>(pvs[u]);
     if (conj) pv = conjc(pv);
     C res;
     if (d.iat) {  // rotated dielectric frame: row c of the full symmetric alpha^{-1} of this site
@@ -636,8 +641,9 @@ __global__ void __launch_bounds__(256) k_y_rows(Geom g, C* __restrict__ work, co
         for (int k = 0; k < RA; ++k) s[r * RP + bb * H + n1 + LB * k] = o[bb * RA + k];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nr * 2 * RA; i += blockDim.x) {
-      const int r = i % nr, blk = i / nr;
+    for (int i = threadIdx.x; i < RPB * 2 * RA; i += blockDim.x) {
+      const int r = i % RPB, blk = i / RPB;
+      if (r >= nr) continue;
       C* row = s + r * RP + blk * LB;
       C v[LB];
 #pragma unroll
@@ -652,18 +658,22 @@ __global__ void __launch_bounds__(256) k_y_rows(Geom g, C* __restrict__ work, co
       work[(r0 + r) * PY + y] = s[r * RP + y];
     }
   } else {
-    // the tile's rows are one contiguous run of nr * PY elements; for a full complex64 tile each
-    // thread issues all its loads before its first shared-memory store
-    constexpr int kPer = RPB * PY / 256;
-    if (sizeof(C) == 8 && nr == RPB && RPB * PY % 256 == 0 && kPer <= 16 && blockDim.x == 256) {
+    // the tile's rows are one contiguous run of nr * PY elements; on a full complex64 tile each thread
+    // issues all its loads before its first shared-memory store, also where the threads do not divide
+    // the tile (25 rows of 160, 21 of 192: 16 RHS 0.49 -> 0.24 and 0.72 -> 0.42 ms)
+    constexpr int kPer = (RPB * PY + 255) / 256;
+    if (sizeof(C) == 8 && kPer <= 20 && nr == RPB) {
       const C* src = work + r0 * PY;
-      C t[kPer > 0 ? kPer : 1];
-#pragma unroll
-      for (int u = 0; u < kPer; ++u) t[u] = src[threadIdx.x + 256 * u];
+      C t[kPer];
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         const int i = threadIdx.x + 256 * u;
-        s[(i / PY) * RP + i % PY] = t[u];
+        if (RPB * PY % 256 == 0 || i < RPB * PY) t[u] = src[i];
+      }
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) {
+        const int i = threadIdx.x + 256 * u;
+        if (RPB * PY % 256 == 0 || i < RPB * PY) s[(i / PY) * RP + i % PY] = t[u];
       }
     } else {
       for (int i = threadIdx.x; i < nr * PY; i += blockDim.x) {
@@ -672,8 +682,9 @@ __global__ void __launch_bounds__(256) k_y_rows(Geom g, C* __restrict__ work, co
       }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nr * 2 * RA; i += blockDim.x) {
-      const int r = i % nr, blk = i / nr;
+    for (int i = threadIdx.x; i < RPB * 2 * RA; i += blockDim.x) {
+      const int r = i % RPB, blk = i / RPB;
+      if (r >= nr) continue;
       C* row = s + r * RP + blk * LB;
       C v[LB];
 #pragma unroll
