@@ -527,6 +527,18 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
       }
     }
   }
+  if constexpr (sizeof(C) == sizeof(float2)) {
+    int smax = 0;
+    cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    if (dda::plane_half_ok_c64(g0, smax))
+      for (int nt : {256, 384}) {
+        dda::MvTune t = base;
+        t.plane = true;
+        t.clus = 0;
+        t.half = nt;
+        cand.push_back(t);
+      }
+  }
   cand.push_back(t5);
   dda::MvTune best = cand[0];
   {
@@ -586,7 +598,7 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
     // and bulk-copy staging of the plane pass's HBM blocks
     int smax_b = 0;
     cudaDeviceGetAttribute(&smax_b, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    if (err.ok() && sizeof(C) == sizeof(float2) && best.plane && best.clus == 0 &&
+    if (err.ok() && sizeof(C) == sizeof(float2) && best.plane && best.clus == 0 && best.half == 0 &&
         dda::plane_bulk_ok_c64(g0, smax_b)) {
       dda::MvTune t = best;
       t.bulk = true;
@@ -1147,7 +1159,8 @@ dda_status dda_build_green_fft(dda_ctx* c, const int32_t pad[3]) {
     // DDA_SCHEDULE pins the schedule instead of autotuning it: "generic" (shared-memory
     // engine of fft.cuh), "fast5" (compile-time kernels, 5 passes), "plane512" / "plane768"
     // (compile-time kernels, fused plane pass where it exists), "cluster2" / "cluster4"
-    // (complex64 plane pass split over a cluster of 2 or 4 CTAs where it fits)
+    // (complex64 plane pass split over a cluster of 2 or 4 CTAs where it fits), "half256" / "half384"
+    // (complex64 plane pass half by half with that many threads, where it exists)
     // the same grid as the previous build keeps its tuned schedules (no new tuning, no new graph)
     const bool same_grid = c->have_sched && c->g64.n == g.n && c->g64.nx == g.nx && c->g64.ny == g.ny &&
                            c->g64.nz == g.nz && c->g64.px == g.px && c->g64.py == g.py && c->g64.pz == g.pz &&
@@ -1170,6 +1183,12 @@ dda_status dda_build_green_fft(dda_ctx* c, const int32_t pad[3]) {
       } else if (sched == "cluster2" || sched == "cluster4") {
         const int S = sched == "cluster2" ? 2 : 4;
         if (t64.plane_ok && dda::plane_cluster_capacity_c64(g64, S, smax) > 0) t64.clus = S;
+        c->forced_schedule = true;
+      } else if (sched == "half256" || sched == "half384") {
+        if (dda::plane_half_ok_c64(g64, smax)) {
+          t64.plane = true;
+          t64.half = sched == "half384" ? 384 : 256;
+        }
         c->forced_schedule = true;
       }
     }
@@ -2615,7 +2634,7 @@ dda_status dda_schedule_info(dda_ctx* c, int dtype, int32_t info[12]) {
   const dda::MvTune& t = dtype == DDA_C64 ? c->t64 : c->t128;
   info[0] = t.plane ? 3 : 5;
   info[1] = t.fast ? 1 : 0;
-  info[2] = t.plane ? (t.clus == 2 ? 384 : t.clus == 4 ? 256 : t.thr_p) : 0;
+  info[2] = t.plane ? (t.half ? t.half : t.clus == 2 ? 384 : t.clus == 4 ? 256 : t.thr_p) : 0;
   info[3] = c->tuned_nrhs[dtype == DDA_C64 ? 0 : 1];
   info[4] = t.plane && t.clus > 1 ? t.clus : 1;
   info[6] = t.plane && t.bulk ? 1 : 0;

@@ -132,6 +132,7 @@ struct MvTune {
   int xty = 0;            // y rows per CTA of the compile-time x passes (0: the length's default)
   int xnc = 0;            // components per CTA of the x passes (0 or 3: all three; 1: one)
   bool bulk = false;      // plane pass stages its HBM blocks with bulk copies
+  int half = 0;           // plane pass half by half with this many threads (0: whole planes)
   int zr = 0;             // 5-pass z columns with pass B, Ghat and inverse pass B fused in registers
 };
 
@@ -164,6 +165,7 @@ int plane_cluster_capacity_c64(const Geom& g, int S, int smax);  // co-resident 
 // complex64 plane pass with its HBM blocks staged by bulk copies (matvec_plane_bulk.cu)
 Err launch_plane_bulk_c64(const Geom& g, const MvData<float2>& d, int nrhs, cudaStream_t st);
 bool plane_bulk_ok_c64(const Geom& g, int smax);
+bool plane_half_ok_c64(const Geom& g, int smax);  // the half-by-half plane kernel exists for this grid
 void plane_bulk_optin_c64(int smax);
 void cluster_optin_c64(int smax);
 void fast_optin_c128(int smax);

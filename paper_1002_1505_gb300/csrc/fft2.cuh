@@ -257,6 +257,31 @@ __device__ __forceinline__ void passA_inv(C* in, int n1, const C* tw, C* lo, C* 
   }
 }
 
+// Pass A of one spectral half h (the radix-2 digit): the RA outputs / inputs of block h only, so a
+// zero-padded transform can be worked off half by half.  Forward: x[j] -> out[k] (position n1 + LB k
+// of the half); inverse: in[k] -> v[j], the half's share of the output at n1 + LB*j before the last
+// radix-2 step (half 1 still to be multiplied by conj(tw[n1 + LB*j])).
+template <int L, int NA = 1, typename C>
+__device__ __forceinline__ void passA_half_fwd(C* x, int n1, int h, const C* tw) {
+  using S = Shape<L, NA>;
+  constexpr int RA = S::RA, LB = S::LB;
+  if (h) {
+#pragma unroll
+    for (int j = 0; j < RA; ++j) x[j] = cmul(x[j], tw[n1 + LB * j]);
+  }
+  if constexpr (RA > 1) dftA<S, -1>(x);
+#pragma unroll
+  for (int k = 1; k < RA; ++k) x[k] = cmul(x[k], tw[2 * n1 * S::nat(k)]);
+}
+template <int L, int NA = 1, typename C>
+__device__ __forceinline__ void passA_half_inv(C* v, int n1, const C* tw) {
+  using S = Shape<L, NA>;
+  constexpr int RA = S::RA;
+#pragma unroll
+  for (int k = 1; k < RA; ++k) v[k] = cmulc(v[k], tw[2 * n1 * S::nat(k)]);
+  if constexpr (RA > 1) dftA<S, 1>(v);
+}
+
 // ------------------------------------------------------------------ pass B
 // DIF stage S of the plan applied to one sub-block v[LB] (all indices compile-time).
 template <int L, int S, int LB, typename C>

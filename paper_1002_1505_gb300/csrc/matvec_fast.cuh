@@ -608,6 +608,183 @@ __global__ void __launch_bounds__(NT) k_yz_plane(Geom g, MvData<C> d) {
   }
 }
 
+// ------------------------------------------------------------------ the plane in two halves of ky
+// The zero-padded y transform's radix-2 step splits ky into two halves that share nothing but their
+// input and the sum of their outputs, so a CTA can take the plane half by half in half the shared
+// memory: two CTAs fit on an SM where the whole plane leaves room for one, and one CTA's barriers and
+// loads run under the other's arithmetic.  The half of ky h, storage positions [h PY/2, (h+1) PY/2):
+// y pass A and B, z pass A, pass B with Ghat and inverse pass B, inverse z pass A, inverse y pass B.
+// Between the halves one phase per (row, n1) takes half 0's inverse pass A out of its slots, exchanges
+// the result for the input in the workspace and puts half 1's pass A into the same slots; the last
+// phase adds half 1's share to half 0's in the workspace.  Bound by the shared-memory pipe (L1
+// wavefronts 69 % busy on 96 x 96, of which 16 % bank conflicts), so what the second CTA can give is
+// bounded too.  Middle passes, us, best whole-plane or 5-pass schedule / this one: 96 x 96 with 128 RHS
+// 1626 / 1605, 80 x 80 with 16 RHS 150 / 133, 128 x 128 (64 kx, 2 RHS) 53 / 39, 128 x 64 (128 kx, 8
+// RHS) 156 / 126; 96 x 64 with 2 RHS 30.4 / 32.4, where the whole plane stays.  The tuner decides.
+// grid (nrhs, px), block NT.  smem: twy[PY] | twz[PZ] | pl[PZ*3][RP] (row (z,c) = z*3 + c)
+template <int PY>
+constexpr int half_pitch() { return (PY / 2) | 1; }
+constexpr size_t half_bytes(int py, int pz) {
+  return sizeof(float2) * ((size_t)py + pz + (size_t)pz * 3 * ((py / 2) | 1));
+}
+constexpr int half_min_ctas(int py, int pz) { return 2 * (half_bytes(py, pz) + 1024) <= 228 * 1024 ? 2 : 1; }
+
+template <int PY, int PZ, int NT>
+__global__ void __launch_bounds__(NT, (half_min_ctas(PY, PZ))) k_yz_half(Geom g, MvData<float2> d) {
+  using C = float2;
+  using SY = Shape<PY>;
+  using SZ = Shape<PZ>;
+  constexpr int RAy = SY::RA, LBy = SY::LB, PH = PY / 2, RP = half_pitch<PY>();
+  constexpr int RAz = SZ::RA, LBz = SZ::LB, Hz = SZ::H;
+  pdl_begin();
+  extern __shared__ unsigned char smem_raw[];
+  C* twy = reinterpret_cast<C*>(smem_raw);
+  C* twz = twy + PY;
+  C* pl = twz + PZ;
+  const int b = blockIdx.x, kx = blockIdx.y;
+  if (rhs_done(d, b)) return;
+  const int nz = g.nz, ny = g.ny;
+  C* wb = d.work + ((int64_t)b * 3 * g.px + kx) * ((int64_t)nz * g.ys);
+  const int64_t cstride = (int64_t)g.px * nz * g.ys;
+  copy_tw(twy, d.twy, PY);
+  copy_tw(twz, d.twz, PZ);
+  __syncthreads();
+  const int nrow = 3 * nz;
+  // y pass A of half 0: rows (z, c) from the workspace
+  for (int i = threadIdx.x; i < nrow * LBy; i += NT) {
+    const int n1 = i % LBy, r = i / LBy;
+    const int c = r / nz, z = r - c * nz;
+    const C* src = wb + c * cstride + (int64_t)z * g.ys;
+    C x[RAy];
+#pragma unroll
+    for (int j = 0; j < RAy; ++j) {
+      const int yy = n1 + LBy * j;
+      x[j] = yy < ny ? src[yy] : czero<C>();
+    }
+    f2::passA_half_fwd<PY>(x, n1, 0, twy);
+    C* row = pl + (z * 3 + c) * RP + n1;
+#pragma unroll
+    for (int k = 0; k < RAy; ++k) row[LBy * k] = x[k];
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    // y pass B
+    for (int i = threadIdx.x; i < nrow * RAy; i += NT) {
+      const int blk = i / nrow, rr = i - blk * nrow;
+      C* row = pl + rr * RP + blk * LBy;
+      C v[LBy];
+#pragma unroll
+      for (int e = 0; e < LBy; ++e) v[e] = row[e];
+      f2::passB_fwd<PY>(v, twy);
+#pragma unroll
+      for (int e = 0; e < LBy; ++e) row[e] = v[e];
+    }
+    __syncthreads();
+    // z pass A (pencils (c, ky), rows z < nz nonzero)
+    for (int i = threadIdx.x; i < 3 * PH * LBz; i += NT) {
+      const int ky = i % PH, r = i / PH;
+      const int c = r % 3, n1 = r / 3;
+      C x[RAz], o[2 * RAz];
+#pragma unroll
+      for (int j = 0; j < RAz; ++j) {
+        const int zz = n1 + LBz * j;
+        x[j] = (zz < nz) ? pl[(zz * 3 + c) * RP + ky] : czero<C>();
+      }
+      f2::passA_fwd<PZ>(x, n1, twz, o);
+#pragma unroll
+      for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+        for (int k = 0; k < RAz; ++k) pl[((bb * Hz + n1 + LBz * k) * 3 + c) * RP + ky] = o[bb * RAz + k];
+    }
+    __syncthreads();
+    // z pass B, Ghat, inverse z pass B -- in registers for the three components
+    for (int i = threadIdx.x; i < PH * 2 * RAz; i += NT) {
+      const int ky = i % PH, blk = i / PH;
+      C* q = pl + (blk * LBz * 3) * RP + ky;
+      C v0[LBz], v1[LBz], v2[LBz];
+#pragma unroll
+      for (int e = 0; e < LBz; ++e) {
+        v0[e] = q[(3 * e) * RP];
+        v1[e] = q[(3 * e + 1) * RP];
+        v2[e] = q[(3 * e + 2) * RP];
+      }
+      f2::passB_fwd<PZ>(v0, twz);
+      f2::passB_fwd<PZ>(v1, twz);
+      f2::passB_fwd<PZ>(v2, twz);
+#pragma unroll
+      for (int e = 0; e < LBz; ++e)
+        gmul3(d.ghat, ghat_at<C>(kx, blk * LBz + e, h * PH + ky, PZ, PY), PY, v0[e], v1[e], v2[e]);
+      f2::passB_inv<PZ>(v0, twz);
+      f2::passB_inv<PZ>(v1, twz);
+      f2::passB_inv<PZ>(v2, twz);
+#pragma unroll
+      for (int e = 0; e < LBz; ++e) {
+        q[(3 * e) * RP] = v0[e];
+        q[(3 * e + 1) * RP] = v1[e];
+        q[(3 * e + 2) * RP] = v2[e];
+      }
+    }
+    __syncthreads();
+    // z inverse, pass A: rows z < nz only
+    for (int i = threadIdx.x; i < 3 * PH * LBz; i += NT) {
+      const int ky = i % PH, r = i / PH;
+      const int c = r % 3, n1 = r / 3;
+      C v[2 * RAz], lo[RAz];
+#pragma unroll
+      for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+        for (int k = 0; k < RAz; ++k) v[bb * RAz + k] = pl[((bb * Hz + n1 + LBz * k) * 3 + c) * RP + ky];
+      f2::passA_inv<PZ, false>(v, n1, twz, lo, (C*)nullptr);
+#pragma unroll
+      for (int j = 0; j < RAz; ++j) {
+        const int zz = n1 + LBz * j;
+        if (zz < nz) pl[(zz * 3 + c) * RP + ky] = lo[j];
+      }
+    }
+    __syncthreads();
+    // y inverse, pass B
+    for (int i = threadIdx.x; i < nrow * RAy; i += NT) {
+      const int blk = i / nrow, rr = i - blk * nrow;
+      C* row = pl + rr * RP + blk * LBy;
+      C v[LBy];
+#pragma unroll
+      for (int e = 0; e < LBy; ++e) v[e] = row[e];
+      f2::passB_inv<PY>(v, twy);
+#pragma unroll
+      for (int e = 0; e < LBy; ++e) row[e] = v[e];
+    }
+    __syncthreads();
+    // y inverse, pass A; after half 0 the workspace's input moves into half 1's pass A
+    for (int i = threadIdx.x; i < nrow * LBy; i += NT) {
+      const int n1 = i % LBy, r = i / LBy;
+      const int c = r / nz, z = r - c * nz;
+      C* io = wb + c * cstride + (int64_t)z * g.ys;
+      C* row = pl + (z * 3 + c) * RP + n1;
+      C v[RAy], x[RAy];
+#pragma unroll
+      for (int j = 0; j < RAy; ++j) {  // half 0: the input; half 1: half 0's result
+        const int yy = n1 + LBy * j;
+        x[j] = yy < ny ? io[yy] : czero<C>();
+      }
+#pragma unroll
+      for (int k = 0; k < RAy; ++k) v[k] = row[LBy * k];
+      f2::passA_half_inv<PY>(v, n1, twy);
+#pragma unroll
+      for (int j = 0; j < RAy; ++j) {
+        const int yy = n1 + LBy * j;
+        if (yy < ny) io[yy] = h == 0 ? v[j] : f2::addmulc(x[j], v[j], twy[yy]);
+      }
+      if (h == 0) {
+        f2::passA_half_fwd<PY>(x, n1, 1, twy);
+#pragma unroll
+        for (int k = 0; k < RAy; ++k) row[LBy * k] = x[k];
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // ------------------------------------------------------------------ 5-pass: y rows
 // rows (b, c, kx, z) of W with ys = PY; RPB rows per CTA.  smem: tw[PY] | s[RPB][PY+1]
 template <typename C, int PY, int RPB, bool INV>
@@ -938,6 +1115,17 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, NT, NA>())) k_z_col
   X(16, 16) X(24, 24) X(32, 32) X(40, 40) X(48, 48) X(64, 64) X(80, 80) X(96, 96) X(96, 64) X(64, 96) \
   X(96, 48) X(48, 96) X(64, 32) X(32, 64) X(96, 40) X(80, 40) X(48, 32) X(32, 48)
 
+// plane pairs with the half-by-half kernel: planes too large for two whole ones on an SM, and (128, *)
+// planes of which only a half fits at all; threads per CTA 256 or 384 (t.half)
+#define DDA_HALF_PLANES(X) X(64, 96) X(80, 80) X(96, 64) X(96, 96) X(128, 128) X(128, 64) X(64, 128) X(128, 96) X(96, 128)
+
+inline bool half_plane_pair(int py, int pz) {
+#define DDA_CASE(A, B) if (py == A && pz == B) return true;
+  DDA_HALF_PLANES(DDA_CASE)
+#undef DDA_CASE
+  return false;
+}
+
 inline bool fast_length(int L) {
   switch (L) {
 #define DDA_CASE(L_) case L_:
@@ -1112,6 +1300,21 @@ Err launch_plane(const Geom& g, const MvData<C>& d, int nrhs, int nt, cudaStream
   return Err::make(DDA_EUNSUPPORTED, "no fast plane kernel for this pair");
 }
 
+inline Err launch_plane_half(const Geom& g, const MvData<float2>& d, int nrhs, int nt, cudaStream_t st) {
+  const dim3 grid(nrhs, g.px);
+  const size_t sm = half_bytes(g.py, g.pz);
+#define DDA_CASE(A, B)                                                                              \
+  if (g.py == A && g.pz == B) {                                                                     \
+    if (nt == 384) DDA_CU(launch_k(k_yz_half<A, B, 384>, grid, dim3(384), sm, st, g, d));           \
+    else DDA_CU(launch_k(k_yz_half<A, B, 256>, grid, dim3(256), sm, st, g, d));                     \
+    DDA_CU(cudaGetLastError());                                                                     \
+    return Err::Ok();                                                                               \
+  }
+  DDA_HALF_PLANES(DDA_CASE)
+#undef DDA_CASE
+  return Err::make(DDA_EUNSUPPORTED, "no half-plane kernel for this pair");
+}
+
 template <typename C>
 Err launch_y_rows(const Geom& g, C* work, const C* tw, int64_t nrows, bool inv, cudaStream_t st) {
   const size_t sm = yrows_fast_smem<C>(g);
@@ -1202,6 +1405,11 @@ void optin_all(int smax) {
   optin_smem(k_yz_plane<C, A, B, 768, false>, smax);
     DDA_FAST_PLANES(DDA_CASE)
 #undef DDA_CASE
+#define DDA_CASE(A, B)                          \
+  optin_smem(k_yz_half<A, B, 256>, smax);       \
+  optin_smem(k_yz_half<A, B, 384>, smax);
+    DDA_HALF_PLANES(DDA_CASE)
+#undef DDA_CASE
     optin_smem(k_z_cols<C, 160, kZrG, kZrG * 2 * Shape<160>::RA, 1>, smax);
   }
 }
@@ -1212,7 +1420,9 @@ template <typename C>
 Err launch_middle(const Geom& g, const MvData<C>& d, const MvTune& t, int nrhs, cudaStream_t st, int& pass) {
   if (t.plane) {
     if constexpr (sizeof(C) == 8) {
-      if (t.clus > 1) {
+      if (t.half) {
+        DDA_TRY(launch_plane_half(g, d, nrhs, t.half, st));
+      } else if (t.clus > 1) {
         DDA_TRY(launch_plane_cluster_c64(g, d, t.clus, nrhs, st));
       } else if (t.bulk) {
         DDA_TRY(launch_plane_bulk_c64(g, d, nrhs, st));
