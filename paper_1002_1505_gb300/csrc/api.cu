@@ -125,6 +125,7 @@ struct dda_ctx {
   double2* d_F = nullptr;             // far-field sums
   double* d_fpart = nullptr;          // far-field partial sums
   float2* d_ftab = nullptr;           // far-field phase tables (many directions)
+  char* d_far = nullptr;              // the buffer that holds the four
   cudaGraphExec_t gexec[2] = {nullptr, nullptr};  // cached solver graphs (complex64, complex128)
   // A captured iteration graph holds device pointers and launch parameters by value.  `gen`
   // changes whenever a device buffer is (re)allocated or the launch schedule or geometry
@@ -337,6 +338,20 @@ dda::RedBuf redbuf(dda_ctx* c, int nrhs, int64_t n3) {
   return rb;
 }
 
+// The far-field buffers: nrd (RHS, direction) pairs of directions and sums, scratch, phase tables, in one
+// allocation of at least 8 MB, so that a context's first observables usually need one cudaMalloc.
+Err far_buffers(dda_ctx* c, size_t nrd, size_t scratch_doubles, size_t tab_bytes) {
+  auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t nh = al(sizeof(double) * 3 * nrd), F = al(sizeof(double2) * 3 * nrd);
+  const size_t part = al(sizeof(double) * scratch_doubles);
+  DDA_TRY(grow(c, &c->d_far, std::max<size_t>(nh + F + part + al(tab_bytes), (size_t)8 << 20)));
+  c->d_nh = reinterpret_cast<double*>(c->d_far);
+  c->d_F = reinterpret_cast<double2*>(c->d_far + nh);
+  c->d_fpart = reinterpret_cast<double*>(c->d_far + nh + F);
+  c->d_ftab = reinterpret_cast<float2*>(c->d_far + nh + F + part);
+  return Err::Ok();
+}
+
 // Workspace for `want` RHS (capped by a memory budget); returns capacity in RHS.
 template <typename C>
 Err ensure_work(dda_ctx* c, int want, int* cap_out);
@@ -492,7 +507,7 @@ template <typename C>
 Err ensure_tuned(dda_ctx* c, int nrhs) {
   const int idx = (sizeof(C) == sizeof(float2)) ? 0 : 1;
   const dda::MvTune base = idx == 0 ? c->t64 : c->t128;
-  if (c->forced_schedule || !base.fast || c->tuned_nrhs[idx] == nrhs) return Err::Ok();
+  if (c->forced_schedule || !base.fast || base.fixed || c->tuned_nrhs[idx] == nrhs) return Err::Ok();
   const dda::Geom& g0 = idx == 0 ? c->g64 : c->g128;
   const std::array<int, 8> key = {g0.nx, g0.ny, g0.nz, g0.px, g0.py, g0.pz, nrhs, (int)sizeof(C)};
   {
@@ -1232,7 +1247,7 @@ dda_status dda_build_green_fft(dda_ctx* c, const int32_t pad[3]) {
     if (e.ok()) e = grow(c, &c->d_gscratch, sizeof(double2) * 6 * M);
     // the double-float copy exists only where the double-float product can run
     c->ghatdf_valid = false;
-    const bool want_df = c->t128.fast && !c->t128.plane;
+    const bool want_df = c->t128.fast && !c->t128.plane && dda::df_lengths(c->g128);
     if (e.ok() && want_df) e = grow(c, &c->d_ghatdf, sizeof(dda::dfp::dfc) * 6 * M);
     if (!e.ok()) return fail(c, e);
     // frequency-order tables of the Green build (kept while px, py stay the same)
@@ -1882,10 +1897,8 @@ dda_status dda_cross_sections(dda_ctx* c, const void* p_dev, double* q_out, cons
         }
       }
       const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
-      e = grow(c, &c->d_nh, sizeof(double) * nh.size());
-      if (e.ok()) e = grow(c, &c->d_F, sizeof(double2) * (size_t)nrhs * ndir * 3);
       const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
-      if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * dda::farfield_scratch(nrhs, ndir, c->n, box, nblk));
+      e = far_buffers(c, (size_t)nrhs * ndir, dda::farfield_scratch(nrhs, ndir, c->n, box, nblk), 0);
       double2* d_F = c->d_F;
       if (e.ok()) {
         e = cuda_ok(cudaMemcpy(c->d_nh, nh.data(), sizeof(double) * nh.size(), cudaMemcpyHostToDevice),
@@ -1993,10 +2006,8 @@ dda_status dda_periodic_scattering(dda_ctx* c, const void* p_dev, int n_spec, co
     std::vector<double> nh((size_t)nrhs * ndir * 3);
     for (int b = 0; b < nrhs; ++b) std::copy(nd.begin(), nd.end(), nh.begin() + (size_t)b * ndir * 3);
     const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
-    e = grow(c, &c->d_nh, sizeof(double) * nh.size());
-    if (e.ok()) e = grow(c, &c->d_F, sizeof(double2) * (size_t)nrhs * ndir * 3);
     const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
-    if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * dda::farfield_scratch(nrhs, ndir, c->n, box, nblk));
+    e = far_buffers(c, (size_t)nrhs * ndir, dda::farfield_scratch(nrhs, ndir, c->n, box, nblk), 0);
     if (e.ok())
       e = cuda_ok(cudaMemcpy(c->d_nh, nh.data(), sizeof(double) * nh.size(), cudaMemcpyHostToDevice),
                   "direction upload");
@@ -2098,8 +2109,26 @@ unsigned long long dda_kernel_launches(void) { return dda::launches(); }
 namespace {
 template <typename C>
 Err matvec_fixed_scratch(dda_ctx* c, const C* p, C* ap, int nrhs) {
-  const dda::Geom g = Sel<C>::geom(c);
-  const size_t need = sizeof(C) * 3ull * g.px * g.nz * g.ys * (size_t)nrhs;
+  dda::Geom g = Sel<C>::geom(c);
+  dda::MvTune t = Sel<C>::tune(c);
+  size_t need = sizeof(C) * 3ull * g.px * g.nz * g.ys * (size_t)nrhs;
+  if (need > dda::kNoAllocScratchBytes && t.fixed && !t.plane) {
+    // these lengths have a compile-time 5-pass schedule only, whose rows are Py long; where that does
+    // not fit, the general 3-pass engine (rows of Ny) may
+    dda::MvTune tg = t;
+    tg.fast = false;
+    tg.plane = true;
+    dda::Geom gg = g;
+    gg.ys = g.ny;
+    int smax = 0;
+    cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    const size_t small = sizeof(C) * 3ull * g.px * g.nz * g.ny * (size_t)nrhs;
+    if (small <= dda::kNoAllocScratchBytes && dda::plane_smem_bytes<C>(gg, tg) <= (size_t)smax) {
+      g = gg;
+      t = tg;
+      need = small;
+    }
+  }
   if (need > dda::kNoAllocScratchBytes)
     return Err::make(DDA_EINVAL, "dda_matvec_noalloc: this grid needs " + std::to_string(need) +
                                      " bytes of FFT scratch for " + std::to_string(nrhs) +
@@ -2109,7 +2138,6 @@ Err matvec_fixed_scratch(dda_ctx* c, const C* p, C* ap, int nrhs) {
   DDA_TRY(dda::noalloc_scratch(c->device, &scratch));
   dda::MvData<C> d = Sel<C>::data(c);
   d.work = (C*)scratch;
-  dda::MvTune t = Sel<C>::tune(c);
   // a bulk-staged plane pass reports a bounded wait that gave up through the context's fault
   // flag; without that flag (no earlier allocating call made it) run the plane pass unstaged
   if (!d.fault) t.bulk = false;
@@ -2245,10 +2273,7 @@ dda_status dda_angular_averages(dda_ctx* c, const void* p_dev, double eta, doubl
       nl[3 * d + 1] = std::sin(t) * std::cos(f);
       nl[3 * d + 2] = std::sin(t) * std::sin(f);
     }
-    e = grow(c, &c->d_ftab, plan.tab_bytes);
-    if (e.ok()) e = grow(c, &c->d_fpart, sizeof(double) * plan.part_doubles);
-    if (e.ok()) e = grow(c, &c->d_nh, sizeof(double) * (size_t)per * ndir * 3);
-    if (e.ok()) e = grow(c, &c->d_F, sizeof(double2) * (size_t)per * ndir * 3);
+    e = far_buffers(c, (size_t)per * ndir, plan.part_doubles, plan.tab_bytes);
     std::vector<double> nh((size_t)per * ndir * 3);
     std::vector<double2> F((size_t)per * ndir * 3);
     for (int b0 = 0; b0 < nrhs && e.ok(); b0 += per) {
@@ -2643,10 +2668,10 @@ dda_status dda_schedule_info(dda_ctx* c, int dtype, int32_t info[12]) {
     const dda::Geom& g = dtype == DDA_C64 ? c->g64 : c->g128;
     const size_t cs = dtype == DDA_C64 ? sizeof(float2) : sizeof(double2);
     info[5] = !t.fast ? 0
-              : t.xnc == 1 ? dda::x_tile_height_one_component(cs)
+              : dda::x_components(g.px, t) == 1 ? dda::x_tile_height_one_component(cs)
                            : (t.xty > 0 && dda::x_tile_height_ok(cs, g.px, t.xty) ? t.xty
                                                                                   : dda::x_tile_height_default(cs, g.px));
-    info[7] = !t.fast ? 0 : (t.xnc == 1 ? 1 : 3);
+    info[7] = !t.fast ? 0 : dda::x_components(g.px, t);
   }
   return DDA_OK;
 }

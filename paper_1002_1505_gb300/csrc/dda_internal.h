@@ -127,6 +127,7 @@ struct MvTune {
   int thr_p = 512;    // threads, plane / z passes
   bool plane = true;  // 3-pass schedule (plane fits in shared memory)
   bool fast = false;  // compile-time-length kernels exist for px, py, pz (matvec_fast.cuh)
+  bool fixed = false;     // one schedule only: a length outside the first list, nothing to tune
   bool plane_ok = false;  // the fast 3-pass plane kernel exists and fits for this grid
   int clus = 0;           // plane pass split over a cluster of this many CTAs (0: one CTA per plane)
   int xty = 0;            // y rows per CTA of the compile-time x passes (0: the length's default)
@@ -175,6 +176,15 @@ void fast_optin_c128(int smax);
 Err launch_matvec_df(const Geom& g, const MvData<dfp::dfc>& d, const MvTune& t, const double2* p, double2* ap,
                      int nrhs, int rhs0, bool conj, cudaStream_t st);
 void fast_optin_df(int smax);
+// The passes for the lengths outside the first list of matvec_fast.cuh (DDA_MORE_LENGTHS), in
+// translation units of their own; C = float2, double2.
+template <typename C> Err more_x_fwd(const Geom& g, const MvData<C>& d, const MvTune& t, const C* p, int nrhs, bool conj, cudaStream_t st);
+template <typename C> Err more_x_inv(const Geom& g, const MvData<C>& d, const MvTune& t, const C* p, C* ap, int nrhs, int rhs0, bool conj, cudaStream_t st);
+template <typename C> Err more_y_rows(const Geom& g, C* work, const C* tw, int64_t nrows, bool inv, cudaStream_t st);
+template <typename C> Err more_z_cols(const Geom& g, const MvData<C>& d, int nrhs, cudaStream_t st);
+void more_optin_c64(int smax);
+void more_optin_c128(int smax);
+void more_optin_fused(int smax);
 // Does a fast schedule exist for this grid (all lengths instantiated, tiles fit)?  Sets t.fast and t.plane.
 void choose_fast_schedule(const Geom& g, bool c64, int smax, MvTune* t);
 // x-pass tile heights (y rows per CTA) of the compile-time kernels: the default for a length, and
@@ -182,6 +192,8 @@ void choose_fast_schedule(const Geom& g, bool c64, int smax, MvTune* t);
 int x_tile_height_default(size_t csize, int px);
 bool x_tile_height_ok(size_t csize, int px, int ty);
 int x_tile_height_one_component(size_t csize);
+int x_components(int px, const MvTune& t);  // components per CTA of the x passes
+bool df_lengths(const Geom& g);             // the double-float kernels exist for these lengths
 // profiling hook: record the i-th pass event if per-pass events are on
 void mark_pass(int i, cudaStream_t st);
 size_t x_smem_bytes(const Geom& g, const MvTune& t, size_t csize);
@@ -320,6 +332,9 @@ template <typename C> Err ccg_beta_update(const KrylovVecs<C>& kv, KState* ks, R
 Err launch_bicg_half_c64(const Geom& g, const MvData<float2>& d, const MvTune& t, const KrylovVecs<float2>& kv,
                          KState* ks, const RedBuf& rbx, int nrhs, int half, cudaStream_t st);
 int x_ctas_per_rhs_c64(const Geom& g, const MvTune& t);
+// its x passes for the other lengths; mode: 1 p update, 2 s update (forward), 3 <rhat, v>, 4 <t, s> (inverse)
+Err more_x_fused(int mode, const Geom& g, const MvData<float2>& d, const MvTune& t, const KrylovVecs<float2>& kv,
+                 KState* ks, const RedBuf& rbx, int nrhs, cudaStream_t st);
 // the register-fused 5-pass z-column kernel exists for this complex64 grid
 bool zcols_rfuse_available_c64(const Geom& g);
 // the passes between the x passes of the complex64 product (plane pass or y/z/y), matvec_fast_c64.cu

@@ -37,10 +37,17 @@ struct FftPlan {
 // pass short), then radix 3 and 5 stages.  Up to L = 320 (the compile-time transforms), a radix 2
 // follows the first 8 when more than 12 elements per sub-block would remain: the two can then be
 // taken together as a radix-16 first pass, which leaves sub-blocks of 8 or 10 instead of 16 or 20.
-// Returns the number of stages.
+// 180, 200, 240 and 288 are ordered so that two stages multiply to 9, 10 or 12 and leave sub-blocks of
+// 10 or 12.  Returns the number of stages.
 constexpr int plan_radices(int L, int* r) {
   int k = 0, rest = L / 2, a = 0;
   r[k++] = 2;
+  if (L == 180 || L == 200 || L == 240 || L == 288) {
+    const int alt[4][4] = {{3, 3, 2, 5}, {2, 5, 2, 5}, {4, 3, 2, 5}, {4, 3, 4, 3}};
+    const int q = L == 180 ? 0 : (L == 200 ? 1 : (L == 240 ? 2 : 3));
+    for (int i = 0; i < 4; ++i) r[k++] = alt[q][i];
+    return k;
+  }
   while (rest % 2 == 0) { rest /= 2; ++a; }
   if (L <= 320 && a >= 4 && (L / 16) > 12) {
     r[k++] = 8;

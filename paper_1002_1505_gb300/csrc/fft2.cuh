@@ -41,7 +41,14 @@ constexpr CPlan cplan(int L) {
   return p;
 }
 
-template <int L, int NA = 1>
+// stages pass A takes after the radix 2: a second one where the first alone would leave sub-blocks of
+// more than 8 elements and the two together stay below radix 16 (36 = 2 (2 3) 3, 90 = 2 (3 3) 5, ...)
+constexpr int na_of(int L) {
+  const CPlan p = cplan(L);
+  return p.nst > 2 && L / (2 * p.r[1]) > 8 && p.r[1] * p.r[2] < 16 ? 2 : 1;
+}
+
+template <int L, int NA = na_of(L)>
 struct Shape {
   static constexpr CPlan P = cplan(L);
   static constexpr int R1 = P.nst > 1 ? P.r[1] : 1;             // radix fused with the radix-2 stage
@@ -195,7 +202,7 @@ __device__ __forceinline__ void dftA(C* v) {
 
 // ------------------------------------------------------------------ pass A
 // x[j] = input at n1 + LB*j (upper half of the input is zero); out[b*RA+k] goes to b*H + n1 + LB*k.
-template <int L, int NA = 1, typename C>
+template <int L, int NA = na_of(L), typename C>
 __device__ __forceinline__ void passA_fwd(C* x, int n1, const C* tw, C* out) {
   using S = Shape<L, NA>;
   constexpr int RA = S::RA, LB = S::LB;
@@ -220,7 +227,7 @@ __device__ __forceinline__ void passA_fwd(C* x, int n1, const C* tw, C* out) {
 }
 
 // in[b*RA+k] from b*H + n1 + LB*k; lo[j] = output at n1 + LB*j, hi[j] at H + n1 + LB*j (if HI).
-template <int L, bool HI, int NA = 1, typename C>
+template <int L, bool HI, int NA = na_of(L), typename C>
 __device__ __forceinline__ void passA_inv(C* in, int n1, const C* tw, C* lo, C* hi) {
   using S = Shape<L, NA>;
   constexpr int RA = S::RA, LB = S::LB;
@@ -261,7 +268,7 @@ __device__ __forceinline__ void passA_inv(C* in, int n1, const C* tw, C* lo, C* 
 // zero-padded transform can be worked off half by half.  Forward: x[j] -> out[k] (position n1 + LB k
 // of the half); inverse: in[k] -> v[j], the half's share of the output at n1 + LB*j before the last
 // radix-2 step (half 1 still to be multiplied by conj(tw[n1 + LB*j])).
-template <int L, int NA = 1, typename C>
+template <int L, int NA = na_of(L), typename C>
 __device__ __forceinline__ void passA_half_fwd(C* x, int n1, int h, const C* tw) {
   using S = Shape<L, NA>;
   constexpr int RA = S::RA, LB = S::LB;
@@ -273,7 +280,7 @@ __device__ __forceinline__ void passA_half_fwd(C* x, int n1, int h, const C* tw)
 #pragma unroll
   for (int k = 1; k < RA; ++k) x[k] = cmul(x[k], tw[2 * n1 * S::nat(k)]);
 }
-template <int L, int NA = 1, typename C>
+template <int L, int NA = na_of(L), typename C>
 __device__ __forceinline__ void passA_half_inv(C* v, int n1, const C* tw) {
   using S = Shape<L, NA>;
   constexpr int RA = S::RA;
@@ -338,11 +345,11 @@ __device__ __forceinline__ void passB_inv_stage(C* v) {
   }
 }
 
-template <int L, int NA = 1, typename C>
+template <int L, int NA = na_of(L), typename C>
 __device__ __forceinline__ void passB_fwd(C* v, const C* /*tw: unused, twiddles are compile-time*/) {
   passB_fwd_stage<L, Shape<L, NA>::SB, Shape<L, NA>::LB>(v);
 }
-template <int L, int NA = 1, typename C>
+template <int L, int NA = na_of(L), typename C>
 __device__ __forceinline__ void passB_inv(C* v, const C* /*tw*/) {
   passB_inv_stage<L, Shape<L, NA>::SB, Shape<L, NA>::LB>(v);
 }

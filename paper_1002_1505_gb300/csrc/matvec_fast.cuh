@@ -22,8 +22,32 @@
 #include "fft2.cuh"
 #include "kred.cuh"
 
+// The kernels are instantiated per length in two sets: DDA_CORE_LENGTHS with every launch variant, and
+// DDA_MORE_LENGTHS (the other even 2,3,5-smooth lengths of 18 to 200, and 216, 240 and 288) with one
+// x-pass variant and no fused plane, compiled in translation units that define DDA_MORE_SET before they
+// include this header.  Everything length-dependent then lives in namespace fast_more instead of fast.
+// Grids with a length of the second set run the 5-pass schedule with one component per x-pass CTA,
+// nothing to tune; on the general engine a 90 x 54 x 80 grid with 2 RHS took 109 us in complex64 and
+// 901 us in complex128, here 44 and 508.
+#define DDA_CORE_LENGTHS(X) X(16) X(24) X(32) X(40) X(48) X(64) X(80) X(96) X(128) X(160) X(192) X(256) X(320)
+#define DDA_MORE_LENGTHS(X) \
+  X(18) X(20) X(30) X(36) X(50) X(54) X(60) X(72) X(90) X(100) X(108) X(120) X(144) X(150) X(162) X(180) X(200) X(216) X(240) X(288)
+#ifdef DDA_MORE_SET
+#define DDA_FAST_LENGTHS DDA_MORE_LENGTHS
+#define DDA_FAST_NS fast_more
+#else
+#define DDA_FAST_LENGTHS DDA_CORE_LENGTHS
+#define DDA_FAST_NS fast
+#endif
+
 namespace dda {
-namespace fast {
+namespace DDA_FAST_NS {
+
+#ifdef DDA_MORE_SET
+constexpr bool kMoreSet = true;
+#else
+constexpr bool kMoreSet = false;
+#endif
 
 using f2::Shape;
 
@@ -921,7 +945,7 @@ constexpr size_t zcols_smem_elems() {
 // otherwise be too long to fuse
 template <typename C, int PZ>
 constexpr int zcols_na() {
-  return (sizeof(C) == 8 && Shape<PZ, 1>::LB > 12 && Shape<PZ, 2>::LB >= 2) ? 2 : 1;
+  return (sizeof(C) == 8 && Shape<PZ, 1>::LB > 12 && Shape<PZ, 2>::LB >= 2) ? 2 : f2::na_of(PZ);
 }
 
 // CTAs per SM the register budget is sized for: 2 in complex64 (128 registers; without the cap the
@@ -1110,7 +1134,6 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, NT, NA>())) k_z_col
 }
 
 // ------------------------------------------------------------------ dispatch
-#define DDA_FAST_LENGTHS(X) X(16) X(24) X(32) X(40) X(48) X(64) X(80) X(96) X(128) X(160) X(192) X(256) X(320)
 #define DDA_FAST_PLANES(X)                                                                               \
   X(16, 16) X(24, 24) X(32, 32) X(40, 40) X(48, 48) X(64, 64) X(80, 80) X(96, 96) X(96, 64) X(64, 96) \
   X(96, 48) X(48, 96) X(64, 32) X(32, 64) X(96, 40) X(80, 40) X(48, 32) X(32, 48)
@@ -1126,15 +1149,25 @@ inline bool half_plane_pair(int py, int pz) {
   return false;
 }
 
-inline bool fast_length(int L) {
+inline bool core_length(int L) {
   switch (L) {
 #define DDA_CASE(L_) case L_:
-    DDA_FAST_LENGTHS(DDA_CASE)
+    DDA_CORE_LENGTHS(DDA_CASE)
 #undef DDA_CASE
     return true;
     default: return false;
   }
 }
+inline bool more_length(int L) {
+  switch (L) {
+#define DDA_CASE(L_) case L_:
+    DDA_MORE_LENGTHS(DDA_CASE)
+#undef DDA_CASE
+    return true;
+    default: return false;
+  }
+}
+inline bool fast_length(int L) { return core_length(L) || more_length(L); }
 
 inline bool fast_plane_pair(int py, int pz) {
 #define DDA_CASE(A, B) if (py == A && pz == B) return true;
@@ -1150,14 +1183,15 @@ template <typename C, int PX> constexpr int x_ty() {
 inline int x_ty_rt(size_t csize, int px) { return csize == 8 ? (px <= 128 ? 16 : 8) : (px <= 128 ? 8 : 4); }
 // the tile heights instantiated besides the default (small batches want more, shorter tiles)
 inline bool x_ty_valid(size_t csize, int px, int ty) {
+  if (more_length(px)) return false;
   return ty == x_ty_rt(csize, px) || ty == 4 || (ty == 8 && x_ty_rt(csize, px) > 8);
 }
 // the one-component variant (each CTA transforms one of the three components) has this tile height
 template <typename C> constexpr int x_nc1_ty() { return sizeof(C) == 8 ? 16 : 8; }
 inline int x_nc1_ty_rt(size_t csize) { return csize == 8 ? 16 : 8; }
-inline int x_nc_pick(const MvTune& t) { return t.xnc == 1 ? 1 : 3; }
+inline int x_nc_pick(const MvTune& t, int px) { return t.xnc == 1 || more_length(px) ? 1 : 3; }
 inline int x_ty_pick(const MvTune& t, size_t csize, int px) {
-  if (x_nc_pick(t) == 1) return x_nc1_ty_rt(csize);
+  if (x_nc_pick(t, px) == 1) return x_nc1_ty_rt(csize);
   return (t.xty > 0 && x_ty_valid(csize, px, t.xty)) ? t.xty : x_ty_rt(csize, px);
 }
 
@@ -1170,6 +1204,7 @@ inline int odd_pitch(int n) { return (n % 2) ? n : n + 1; }
 
 template <typename C>
 size_t x_fast_smem(const Geom& g, int TY = 0, int NC = 3) {
+  if (more_length(g.px)) NC = 1, TY = x_nc1_ty<C>();
   if (TY <= 0) TY = x_ty_rt(sizeof(C), g.px);
   return sizeof(C) * ((size_t)g.px + (size_t)NC * TY * odd_pitch(g.nx) + (size_t)NC * g.px * TY);
 }
@@ -1192,7 +1227,8 @@ constexpr int y_rows_per_cta() {
 inline int y_rows_per_cta_rt(int py) {
   switch (py) {
 #define DDA_CASE(L_) case L_: return y_rows_per_cta<L_>();
-    DDA_FAST_LENGTHS(DDA_CASE)
+    DDA_CORE_LENGTHS(DDA_CASE)
+    DDA_MORE_LENGTHS(DDA_CASE)
 #undef DDA_CASE
     default: return 8;
   }
@@ -1205,11 +1241,16 @@ template <typename C>
 size_t zcols_fast_smem(const Geom& g) {
   switch (g.pz) {
 #define DDA_CASE(L_) case L_: return sizeof(C) * zcols_smem_elems<C, L_, zcols_g_rt(sizeof(C), L_), zcols_na<C, L_>()>();
-    DDA_FAST_LENGTHS(DDA_CASE)
+    DDA_CORE_LENGTHS(DDA_CASE)
+    DDA_MORE_LENGTHS(DDA_CASE)
 #undef DDA_CASE
     default: return sizeof(C) * ((size_t)g.pz + (size_t)g.pz * 3 * zcols_g_rt(sizeof(C), g.pz));
   }
 }
+
+// the passes of this type exist in the second set of lengths too
+template <typename C>
+constexpr bool kHasMore = !kMoreSet && !std::is_same<C, dfp::dfc>::value;
 
 // k_x_fwd / k_x_inv for the variant chosen at run time: three components per CTA with tile
 // height TY (the default, 4 or 8), or one component per CTA with the one-component height
@@ -1221,12 +1262,14 @@ Err with_x(int nc, int ty, F&& f) {
     if (ty == x_nc1_ty<C>()) return f(std::integral_constant<int, x_nc1_ty<C>()>{}, std::integral_constant<int, 1>{});
     return Err::make(DDA_EUNSUPPORTED, "x tile height not instantiated");
   }
-  if (ty == D) return f(std::integral_constant<int, D>{}, I3{});
-  if constexpr (D != 4) {
-    if (ty == 4) return f(std::integral_constant<int, 4>{}, I3{});
-  }
-  if constexpr (D > 8) {
-    if (ty == 8) return f(std::integral_constant<int, 8>{}, I3{});
+  if constexpr (!kMoreSet) {
+    if (ty == D) return f(std::integral_constant<int, D>{}, I3{});
+    if constexpr (D != 4) {
+      if (ty == 4) return f(std::integral_constant<int, 4>{}, I3{});
+    }
+    if constexpr (D > 8) {
+      if (ty == 8) return f(std::integral_constant<int, 8>{}, I3{});
+    }
   }
   return Err::make(DDA_EUNSUPPORTED, "x tile height not instantiated");
 }
@@ -1234,7 +1277,7 @@ Err with_x(int nc, int ty, F&& f) {
 template <typename C>
 Err launch_x_fwd(const Geom& g, const MvData<C>& d, const MvTune& t, const typename Io<C>::t* p, int nrhs, bool conj,
                  cudaStream_t st) {
-  const int NC = x_nc_pick(t);
+  const int NC = x_nc_pick(t, g.px);
   const int TY = x_ty_pick(t, sizeof(C), g.px);
   const size_t sm = x_fast_smem<C>(g, TY, NC);
   const dim3 grid((g.ny + TY - 1) / TY, g.nz, nrhs * (3 / NC));
@@ -1250,7 +1293,9 @@ Err launch_x_fwd(const Geom& g, const MvData<C>& d, const MvTune& t, const typen
     break;
     DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
-    default: return Err::make(DDA_EUNSUPPORTED, "no fast x kernel for this length");
+    default:
+      if constexpr (kHasMore<C>) return more_x_fwd<C>(g, d, t, p, nrhs, conj, st);
+      return Err::make(DDA_EUNSUPPORTED, "no fast x kernel for this length");
   }
   DDA_CU(cudaGetLastError());
   return Err::Ok();
@@ -1259,7 +1304,7 @@ Err launch_x_fwd(const Geom& g, const MvData<C>& d, const MvTune& t, const typen
 template <typename C>
 Err launch_x_inv(const Geom& g, const MvData<C>& d, const MvTune& t, const typename Io<C>::t* p,
                  typename Io<C>::t* ap, int nrhs, int rhs0, bool conj, cudaStream_t st) {
-  const int NC = x_nc_pick(t);
+  const int NC = x_nc_pick(t, g.px);
   const int TY = x_ty_pick(t, sizeof(C), g.px);
   const size_t sm = x_fast_smem<C>(g, TY, NC);
   const dim3 grid((g.ny + TY - 1) / TY, g.nz, nrhs * (3 / NC));
@@ -1275,7 +1320,9 @@ Err launch_x_inv(const Geom& g, const MvData<C>& d, const MvTune& t, const typen
     break;
     DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
-    default: return Err::make(DDA_EUNSUPPORTED, "no fast x kernel for this length");
+    default:
+      if constexpr (kHasMore<C>) return more_x_inv<C>(g, d, t, p, ap, nrhs, rhs0, conj, st);
+      return Err::make(DDA_EUNSUPPORTED, "no fast x kernel for this length");
   }
   DDA_CU(cudaGetLastError());
   return Err::Ok();
@@ -1284,7 +1331,7 @@ Err launch_x_inv(const Geom& g, const MvData<C>& d, const MvTune& t, const typen
 // complex64 only: a complex128 plane does not fit in shared memory at these sizes
 template <typename C>
 Err launch_plane(const Geom& g, const MvData<C>& d, int nrhs, int nt, cudaStream_t st) {
-  if constexpr (sizeof(C) == 8) {
+  if constexpr (sizeof(C) == 8 && !kMoreSet) {
     const size_t sm = plane_fast_smem<C>(g);
     const dim3 grid(nrhs, g.px);
 #define DDA_CASE(A, B)                                               \
@@ -1330,7 +1377,9 @@ Err launch_y_rows(const Geom& g, C* work, const C* tw, int64_t nrows, bool inv, 
     break;
     DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
-    default: return Err::make(DDA_EUNSUPPORTED, "no fast y kernel for this length");
+    default:
+      if constexpr (kHasMore<C>) return more_y_rows<C>(g, work, tw, nrows, inv, st);
+      return Err::make(DDA_EUNSUPPORTED, "no fast y kernel for this length");
   }
   DDA_CU(cudaGetLastError());
   return Err::Ok();
@@ -1341,12 +1390,12 @@ Err launch_y_rows(const Geom& g, C* work, const C* tw, int64_t nrows, bool inv, 
 constexpr int kZrG = 8;
 template <typename C>
 constexpr bool zcols_rfuse_exists(int pz) {
-  return sizeof(C) == 8 && pz == 160;
+  return !kMoreSet && sizeof(C) == 8 && pz == 160;
 }
 
 template <typename C>
 Err launch_z_cols(const Geom& g, const MvData<C>& d, int nrhs, cudaStream_t st, bool rfuse = false) {
-  if constexpr (sizeof(C) == 8) {
+  if constexpr (sizeof(C) == 8 && !kMoreSet) {
     if (rfuse && zcols_rfuse_exists<C>(g.pz)) {
       constexpr int NT = kZrG * 2 * Shape<160>::RA;
       const size_t sm = sizeof(C) * zcols_smem_elems<C, 160, kZrG, 1>();
@@ -1366,7 +1415,9 @@ Err launch_z_cols(const Geom& g, const MvData<C>& d, int nrhs, cudaStream_t st, 
     break;
     DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
-    default: return Err::make(DDA_EUNSUPPORTED, "no fast z kernel for this length");
+    default:
+      if constexpr (kHasMore<C>) return more_z_cols<C>(g, d, nrhs, st);
+      return Err::make(DDA_EUNSUPPORTED, "no fast z kernel for this length");
   }
   DDA_CU(cudaGetLastError());
   return Err::Ok();
@@ -1375,15 +1426,17 @@ Err launch_z_cols(const Geom& g, const MvData<C>& d, int nrhs, cudaStream_t st, 
 template <typename C, int L_>
 void optin_x(int smax) {
   constexpr int D = x_ty<C, L_>();
-  optin_smem(k_x_fwd<C, L_, D>, smax);
-  optin_smem(k_x_inv<C, L_, D>, smax);
-  if constexpr (D != 4) {
-    optin_smem(k_x_fwd<C, L_, 4>, smax);
-    optin_smem(k_x_inv<C, L_, 4>, smax);
-  }
-  if constexpr (D > 8) {
-    optin_smem(k_x_fwd<C, L_, 8>, smax);
-    optin_smem(k_x_inv<C, L_, 8>, smax);
+  if constexpr (!kMoreSet) {
+    optin_smem(k_x_fwd<C, L_, D>, smax);
+    optin_smem(k_x_inv<C, L_, D>, smax);
+    if constexpr (D != 4) {
+      optin_smem(k_x_fwd<C, L_, 4>, smax);
+      optin_smem(k_x_inv<C, L_, 4>, smax);
+    }
+    if constexpr (D > 8) {
+      optin_smem(k_x_fwd<C, L_, 8>, smax);
+      optin_smem(k_x_inv<C, L_, 8>, smax);
+    }
   }
   optin_smem(k_x_fwd<C, L_, x_nc1_ty<C>(), 1>, smax);
   optin_smem(k_x_inv<C, L_, x_nc1_ty<C>(), 1>, smax);
@@ -1399,7 +1452,7 @@ void optin_all(int smax) {
   optin_smem(k_z_cols<C, L_, zcols_g_rt(sizeof(C), L_)>, smax);
   DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
-  if constexpr (sizeof(C) == 8) {
+  if constexpr (sizeof(C) == 8 && !kMoreSet) {
 #define DDA_CASE(A, B)                                                                                    \
   optin_smem(k_yz_plane<C, A, B, 512, false>, smax);     \
   optin_smem(k_yz_plane<C, A, B, 768, false>, smax);
@@ -1464,7 +1517,7 @@ Err launch_matvec_fast(const Geom& g, const MvData<C>& d, const MvTune& t, const
 // ------------------------------------------------------------------ BiCGstab half-iterations, folded (complex64)
 // x-pass CTAs per RHS of the schedule t (the reduction slots of the folded dot products)
 inline int x_ctas_per_rhs(const Geom& g, const MvTune& t) {
-  const int NC = x_nc_pick(t);
+  const int NC = x_nc_pick(t, g.px);
   const int TY = x_ty_pick(t, sizeof(float2), g.px);
   return ((g.ny + TY - 1) / TY) * g.nz * (3 / NC);
 }
@@ -1472,7 +1525,7 @@ inline int x_ctas_per_rhs(const Geom& g, const MvTune& t) {
 template <int MODE, bool FWD>
 Err launch_x_fused(const Geom& g, const MvData<float2>& d, const MvTune& t, const KrylovVecs<float2>& kv, KState* ks,
                    const RedBuf& rbx, int nrhs, cudaStream_t st) {
-  const int NC = x_nc_pick(t);
+  const int NC = x_nc_pick(t, g.px);
   const int TY = x_ty_pick(t, sizeof(float2), g.px);
   const size_t sm = x_fast_smem<float2>(g, TY, NC);
   const dim3 grid((g.ny + TY - 1) / TY, g.nz, nrhs * (3 / NC));
@@ -1491,7 +1544,9 @@ Err launch_x_fused(const Geom& g, const MvData<float2>& d, const MvTune& t, cons
     break;
     DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
-    default: return Err::make(DDA_EUNSUPPORTED, "no fast x kernel for this length");
+    default:
+      if constexpr (!kMoreSet) return more_x_fused(MODE, g, d, t, kv, ks, rbx, nrhs, st);
+      return Err::make(DDA_EUNSUPPORTED, "no fast x kernel for this length");
   }
   DDA_CU(cudaGetLastError());
   return Err::Ok();
@@ -1508,11 +1563,13 @@ void optin_x_fused(int smax) {
     optin_smem(k_x_inv_fused<L_, TY_, NC_, kFuseTS>, smax);
   };
   using I3 = std::integral_constant<int, 3>;
-  all_modes(std::integral_constant<int, D>{}, I3{});
-  if constexpr (D != 4) all_modes(std::integral_constant<int, 4>{}, I3{});
-  if constexpr (D > 8) all_modes(std::integral_constant<int, 8>{}, I3{});
+  if constexpr (!kMoreSet) {
+    all_modes(std::integral_constant<int, D>{}, I3{});
+    if constexpr (D != 4) all_modes(std::integral_constant<int, 4>{}, I3{});
+    if constexpr (D > 8) all_modes(std::integral_constant<int, 8>{}, I3{});
+  }
   all_modes(std::integral_constant<int, x_nc1_ty<float2>()>{}, std::integral_constant<int, 1>{});
 }
 
-}  // namespace fast
+}  // namespace DDA_FAST_NS
 }  // namespace dda

@@ -7,5 +7,8 @@ Err launch_matvec_fast<double2>(const Geom& g, const MvData<double2>& d, const M
                                 double2* ap, int nrhs, int rhs0, bool conj, cudaStream_t st) {
   return fast::launch_matvec_fast<double2>(g, d, t, p, ap, nrhs, rhs0, conj, st);
 }
-void fast_optin_c128(int smax) { fast::optin_all<double2>(smax); }
+void fast_optin_c128(int smax) {
+  fast::optin_all<double2>(smax);
+  more_optin_c128(smax);
+}
 }  // namespace dda

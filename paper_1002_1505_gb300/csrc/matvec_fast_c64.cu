@@ -7,7 +7,10 @@ Err launch_matvec_fast<float2>(const Geom& g, const MvData<float2>& d, const MvT
                                int nrhs, int rhs0, bool conj, cudaStream_t st) {
   return fast::launch_matvec_fast<float2>(g, d, t, p, ap, nrhs, rhs0, conj, st);
 }
-void fast_optin_c64(int smax) { fast::optin_all<float2>(smax); }
+void fast_optin_c64(int smax) {
+  fast::optin_all<float2>(smax);
+  more_optin_c64(smax);
+}
 Err launch_middle_c64(const Geom& g, const MvData<float2>& d, const MvTune& t, int nrhs, cudaStream_t st) {
   int pass = 0;
   return fast::launch_middle<float2>(g, d, t, nrhs, st, pass);
@@ -42,9 +45,11 @@ Err selftest_bulk_wait(int* gave_up) {
 int x_tile_height_default(size_t csize, int px) { return fast::x_ty_rt(csize, px); }
 bool x_tile_height_ok(size_t csize, int px, int ty) { return fast::x_ty_valid(csize, px, ty); }
 int x_tile_height_one_component(size_t csize) { return fast::x_nc1_ty_rt(csize); }
+int x_components(int px, const MvTune& t) { return fast::x_nc_pick(t, px); }
+bool df_lengths(const Geom& g) { return fast::core_length(g.px) && fast::core_length(g.py) && fast::core_length(g.pz); }
 
 bool plane_half_ok_c64(const Geom& g, int smax) {
-  return fast::fast_length(g.px) && fast::half_plane_pair(g.py, g.pz) && fast::half_bytes(g.py, g.pz) <= (size_t)smax;
+  return fast::core_length(g.px) && fast::half_plane_pair(g.py, g.pz) && fast::half_bytes(g.py, g.pz) <= (size_t)smax;
 }
 
 void choose_fast_schedule(const Geom& g, bool c64, int smax, MvTune* t) {
@@ -59,7 +64,8 @@ void choose_fast_schedule(const Geom& g, bool c64, int smax, MvTune* t) {
     return;
   }
   (void)cs;
-  t->plane = c64 && fast::fast_plane_pair(g.py, g.pz) && fast::plane_fast_smem<float2>(g) <= (size_t)smax;
+  t->fixed = fast::more_length(g.px) || fast::more_length(g.py) || fast::more_length(g.pz);
+  t->plane = !t->fixed && c64 && fast::fast_plane_pair(g.py, g.pz) && fast::plane_fast_smem<float2>(g) <= (size_t)smax;
   t->plane_ok = t->plane;
 }
 }  // namespace dda

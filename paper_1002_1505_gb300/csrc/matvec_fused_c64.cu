@@ -25,5 +25,6 @@ void fused_optin_c64(int smax) {
 #define DDA_CASE(L_) fast::optin_x_fused<L_>(smax);
   DDA_FAST_LENGTHS(DDA_CASE)
 #undef DDA_CASE
+  more_optin_fused(smax);
 }
 }  // namespace dda

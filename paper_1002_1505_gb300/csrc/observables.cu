@@ -322,7 +322,7 @@ struct PairSum {
 // and a run of rows, staged in shared memory as P+ and P- pairs that every thread reads by broadcast;
 // a row's sum is FP32 (at most half the box's x length of terms), rows are added in pair sums.
 // Bound by FP32 issue and the broadcasts (48 FMAs per 6 LDS.128): 131,072 sites x 2292 directions x 2
-// polarizations in 0.30 ms, where the site kernel took 7.66 ms (three table lookups and two complex
+// polarizations in 0.28 ms, where the site kernel took 7.66 ms (three table lookups and two complex
 // products per site and direction, and 48 FP64 block sums per CTA at 1/64 of the FP32 rate).
 // grid (nblk, ndp / (2 kRowT), nsets); part[set][blk][nb * 6][ndp].
 constexpr int kRowT = 128;
@@ -843,10 +843,9 @@ FarPlan far_many_plan(int64_t n, const int box[3], int nrhs, int iorth, int ndir
   f.per = (int)sets * f.nb;
   f.tab_bytes = sizeof(float2) * (size_t)(sets * f.ndp * nt);
   if (f.rows) {
-    // about ten CTAs per SM, at least four rows each
+    // one wave of four CTAs per SM (what 108 registers allow), at least eight rows each
     const int64_t tiles = (f.ndp / (2 * kRowT)) * sets;
-    f.nblk = (int)std::max<int64_t>(1, std::min<int64_t>({256, ((int64_t)box[1] * box[2] + 3) / 4,
-                                                          (1520 + tiles - 1) / tiles}));
+    f.nblk = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)box[1] * box[2] + 7) / 8, 608 / tiles));
     f.part_doubles = (size_t)sets * f.nblk * f.nb * 6 * f.ndp;
   } else {
     f.nblk = (int)std::max<int64_t>(1, std::min<int64_t>((n + 2047) / 2048, 64));
