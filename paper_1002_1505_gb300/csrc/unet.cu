@@ -28,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -164,13 +165,16 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(const float* __restrict__
 
 // ------------------------------------------------------------------ tcgen05 convolution
 // The 3x3x3 implicit GEMM on the fifth-generation tensor cores.  A CTA owns a tile of Tz z planes
-// x Ty y rows x all X voxels of one sample.  Per 16-channel chunk, a TMA load brings the tile with
+// x Ty y rows x Tx voxels of one sample.  Per 16-channel chunk, a TMA load brings the tile with
 // its one-voxel halo (zero outside the volume: the load starts at coordinate -1) from a bfloat16
-// channels-last copy of the input into shared memory, as two 8-channel halves in which staged
-// voxel s = (zz * (Ty+2) + yy) * (X+2) + xx sits at byte 16 s.  In that layout the rows of an
+// copy of the input in planes of 8 channels ([sample][channel / 8][Z][Y][X][8]) into shared memory,
+// as two 8-channel halves in which staged voxel s = (zz * (Ty+2) + yy) * (Tx+2) + xx sits at byte
+// 16 s.  A row of a plane is contiguous, so the box's inner extent is 16 (Tx+2) bytes, up to 512
+// (with channels innermost in one tensor it was 16 bytes a voxel, and the copies set the pace:
+// 12 -> 12 channels on 2 x 64 x 48 x 32 in 71 us, now 36).  In that layout the rows of an
 // MMA's A operand are 16 bytes apart, so the K-major no-swizzle descriptor with an 8-row stride of
 // 128 bytes addresses 128 consecutive staged voxels from any start, and the operand of tap
-// (dz, dy, dx) is the output rows' operand moved by dz (Ty+2)(X+2) + dy (X+2) + dx rows: one
+// (dz, dy, dx) is the output rows' operand moved by dz (Ty+2)(Tx+2) + dy (Tx+2) + dx rows: one
 // descriptor per tap, no data movement.  The GEMM's M axis runs over consecutive staged positions
 // from the first interior voxel, in tiles of 128; positions in the halo columns are computed and
 // discarded.  The chunk's weights for all taps come in with one bulk copy.  One thread issues the
@@ -230,13 +234,13 @@ __device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
-// 5-D tiled TMA load (coordinates innermost first) into shared memory, completion counted on bar
-__device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                            int c4, uint64_t* bar) {
+// 4-D tiled TMA load (coordinates innermost first) into shared memory, completion counted on bar
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                            uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
-      "[%7];" ::"r"(saddr(dst)),
-      "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(saddr(bar))
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];" ::"r"(saddr(dst)),
+      "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(saddr(bar))
       : "memory");
 }
 }  // namespace tc
@@ -246,8 +250,9 @@ constexpr uint32_t kTcMaxPolls = 1u << 22;
 
 // tile geometry of the tcgen05 convolution (host-chosen)
 struct TcTile {
-  int Ty, Tz;          // y rows and z planes per CTA (all X voxels of a row)
-  int sx, sy, sz;      // staged extents X+2, Ty+2, Tz+2
+  int Tx, Ty, Tz;      // voxels of a row, y rows and z planes per CTA
+  int ntx;             // x tiles of a row
+  int sx, sy, sz;      // staged extents Tx+2 (at most 32), Ty+2, Tz+2
   int q_first;         // staged row of the first interior voxel (= the largest tap offset)
   int n_mt;            // 128-row M tiles
   int rows_alloc;      // staged rows per channel half (covers every row an MMA reads), multiple of 8
@@ -273,7 +278,8 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 5);
   unsigned char* buf0 = smem_tc + 1024;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int ty0 = blockIdx.x * tl.Ty, tz0 = blockIdx.y * tl.Tz, b = blockIdx.z;
+  const int tx0 = (blockIdx.x % tl.ntx) * tl.Tx, ty0 = (blockIdx.x / tl.ntx) * tl.Ty, tz0 = blockIdx.y * tl.Tz;
+  const int b = blockIdx.z;
   const uint32_t half_bytes = (uint32_t)tl.rows_alloc * 16u;
   const uint32_t act_bytes = tc_act_bytes(tl);
   const uint32_t w_bytes = (uint32_t)kTaps * NP * 32u;
@@ -299,8 +305,9 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
         eph[s] ^= 1u;
       }
       bulk::mbar_arrive_expect_tx(&full[s], 2u * box_bytes + w_bytes);
-      tc::tma_load_5d(act, &tmap, kc * 16, -1, ty0 - 1, tz0 - 1, b, &full[s]);
-      tc::tma_load_5d(act + half_bytes, &tmap, kc * 16 + 8, -1, ty0 - 1, tz0 - 1, b, &full[s]);
+      const int pl = (b * kc_n + kc) * 2;  // the chunk's two planes of 8 channels
+      tc::tma_load_4d(act, &tmap, 8 * (tx0 - 1), ty0 - 1, tz0 - 1, pl, &full[s]);
+      tc::tma_load_4d(act + half_bytes, &tmap, 8 * (tx0 - 1), ty0 - 1, tz0 - 1, pl + 1, &full[s]);
       bulk::load_g2s(wb, wpk + (int64_t)kc * kTaps * NP * 2, w_bytes, &full[s]);
       ok = bulk::mbar_wait(&full[s], fph[s], kTcMaxPolls, fault) && ok;
       fph[s] ^= 1u;
@@ -320,13 +327,14 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
   ok = bulk::mbar_wait(done, 0u, kTcMaxPolls, fault) && ok;
   tc::fence_after();
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+  const bool vec = ys % 4 == 0 && cout % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0;
   for (int mt = 0; mt < tl.n_mt; ++mt) {
     const int q = tl.q_first + mt * 128 + tid;
     const int zz = q / plane, r = q - zz * plane;
     const int yy = r / tl.sx, xx = r - yy * tl.sx;
-    const int z = tz0 + zz - 1, yv = ty0 + yy - 1, x = xx - 1;
-    const bool valid = ok && zz >= 1 && zz <= tl.Tz && yy >= 1 && yy <= tl.Ty && xx >= 1 && xx <= d.X && z < d.Z &&
-                       yv < d.Y;
+    const int z = tz0 + zz - 1, yv = ty0 + yy - 1, x = tx0 + xx - 1;
+    const bool valid = ok && zz >= 1 && zz <= tl.Tz && yy >= 1 && yy <= tl.Ty && xx >= 1 && xx <= tl.Tx && z < d.Z &&
+                       yv < d.Y && x < d.X;
     float* yo = y + ((((int64_t)b * d.Z + (valid ? z : 0)) * d.Y + (valid ? yv : 0)) * d.X + (valid ? x : 0)) * ys;
 #pragma unroll
     for (int c0 = 0; c0 < NP; c0 += 16) {
@@ -337,10 +345,19 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
         for (int j = 0; j < 16; ++j) {
           const int co = c0 + j;
           if (co < cout) {
-            float val = acc[j] + (bias ? bias[co] : 0.f);
-            if (relu) val = fmaxf(val, 0.f);
-            yo[co] = val;
+            acc[j] += bias ? bias[co] : 0.f;
+            if (relu) acc[j] = fmaxf(acc[j], 0.f);
           }
+        }
+        if (vec) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 4)
+            if (c0 + j < cout)
+              *reinterpret_cast<float4*>(yo + c0 + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (c0 + j < cout) yo[c0 + j] = acc[j];
         }
       }
     }
@@ -350,15 +367,17 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
   if (warp == 0) tc::dealloc(tmem, tl.ncol);
 }
 
-// bfloat16 channels-last copy of channels [0, cin) of x (xs per voxel), cpad channels (zeros above
-// cin): the tcgen05 convolution's TMA source.  One thread per 8 channels of a voxel.
-__global__ void k_to_bf16(const float* __restrict__ x, int xs, int cin, int cpad, int64_t V, uint4* __restrict__ out) {
+// bfloat16 copy of channels [0, cin) of x (xs per voxel) in planes of 8 channels, zeros above cin:
+// out[(sample * cpad/8 + c/8) * nvox + voxel] (8 channels each), the tcgen05 convolution's TMA source.
+// One thread per 8 channels of a voxel.
+__global__ void k_to_bf16(const float* __restrict__ x, int xs, int cin, int cpad, int64_t nvox, int B,
+                          uint4* __restrict__ out) {
   const int g8 = cpad / 8;
-  const int64_t total = V * g8;
+  const int64_t total = nvox * g8 * B;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t v = i / g8;
-    const int c = (int)(i - v * g8) * 8;
-    const float* src = x + v * xs;
+    const int64_t p = i / nvox;  // plane
+    const int c = (int)(p % g8) * 8;
+    const float* src = x + (p / g8 * nvox + (i - p * nvox)) * xs;
     float f[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) f[j] = (c + j < cin) ? __ldg(src + c + j) : 0.f;
@@ -719,7 +738,8 @@ struct dda_unet {
   double* h_loss = nullptr;
   bool use_tc = true;                  // convolutions on tcgen05 (DDA_UNET_TC=0: mma.sync throughout)
   unsigned int* d_fault = nullptr;     // set when a bounded tensor-core wait gave up
-  uint4* xb = nullptr;                 // bfloat16 channels-last copy of a tcgen05 convolution's input
+  std::vector<std::pair<std::array<int, 5>, dda::nn::TcTile>> tiles;  // tc_tile's answers by shape
+  uint4* xb = nullptr;                 // bfloat16 copy of a tcgen05 convolution's input
   size_t xb_bytes = 0;
 };
 
@@ -764,39 +784,41 @@ Err repack(dda_unet* n) {
 // with the least modelled time per SM, counting for each 16-channel chunk the bytes a CTA loads
 // (activation tile with halo, both halves, plus the chunk's weights for 27 taps) and its MMAs
 // (27 per 128-row M tile), overlapped when two buffers or two CTAs per SM fit.  false when no tile
-// fits (rows longer than 254 voxels): the caller uses the mma.sync kernel.
+// fits: the caller uses the mma.sync kernel.
 bool tc_tile(const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
   constexpr double kSmem = 227.0 * 1024.0, kBytesPerNs = 60.0, kMmaNs = 16.0;
-  const int X = d.X;
-  if (X + 2 > 256) return false;
   double best = 1e300;
   bool found = false;
-  for (int Tz = 1; Tz <= std::min(d.Z, 16); ++Tz)
+  const int ntx0 = (d.X + 29) / 30;  // rows of at most 30 voxels: the box's inner extent is at most 256 elements
+  for (int ntx = ntx0; ntx <= ntx0 + 1 && ntx <= d.X; ++ntx)
+   for (int Tz = 1; Tz <= std::min(d.Z, 16); ++Tz)
     for (int Ty = 1; Ty <= std::min(d.Y, 64); ++Ty) {
       dda::nn::TcTile t{};
+      t.ntx = ntx;
+      t.Tx = (d.X + ntx - 1) / ntx;
       t.Ty = Ty;
       t.Tz = Tz;
-      t.sx = X + 2;
+      t.sx = t.Tx + 2;
       t.sy = Ty + 2;
       t.sz = Tz + 2;
       const int plane = t.sx * t.sy;
       t.q_first = plane + t.sx + 1;
-      const int q_last = (Tz * t.sy + Ty) * t.sx + X;
+      const int q_last = (Tz * t.sy + Ty) * t.sx + t.Tx;
       t.n_mt = (q_last - t.q_first + 1 + 127) / 128;
-      if (t.n_mt * np > 512) continue;
+      if (t.n_mt * np > 512) break;  // grows with Ty
       t.ncol = 32;
       while ((int)t.ncol < t.n_mt * np) t.ncol *= 2;
       t.rows_alloc = (2 * t.q_first + t.n_mt * 128 + 7) / 8 * 8;
       const double act = 2.0 * t.rows_alloc * 16.0, w = 27.0 * np * 32.0;
       t.stage_bytes = (uint32_t)((act + w + 1023) / 1024) * 1024u;
-      if (1024.0 + t.stage_bytes > kSmem) continue;
+      if (1024.0 + t.stage_bytes > kSmem) break;
       t.stages = (1024.0 + 2.0 * t.stage_bytes <= kSmem) ? 2 : 1;
       const int cps = std::max(1, std::min((int)(kSmem / (1024.0 + t.stages * (double)t.stage_bytes)),
                                            (int)(512 / t.ncol)));
       const double load = (2.0 * 16.0 * t.sx * t.sy * t.sz + w) / kBytesPerNs;
       const double mma = t.n_mt * 27.0 * kMmaNs * std::max(1.0, np / 64.0);
       const double per_chunk = (t.stages == 2 || cps >= 2) ? std::max(load, mma) : load + mma;
-      const double ctas = (double)B * ((d.Y + Ty - 1) / Ty) * ((d.Z + Tz - 1) / Tz);
+      const double ctas = (double)B * t.ntx * ((d.Y + Ty - 1) / Ty) * ((d.Z + Tz - 1) / Tz);
       const double waves = std::ceil(ctas / (152.0 * cps));
       const double cost = waves * cps * per_chunk;
       if (cost < best) {
@@ -806,6 +828,23 @@ bool tc_tile(const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
       }
     }
   return found;
+}
+
+// tc_tile with its answers kept in the network (at most 64 shapes): the search takes tens of
+// microseconds of host time, more than a small convolution
+bool tc_tile_of(dda_unet* n, const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
+  const std::array<int, 5> key = {d.Z, d.Y, d.X, B, np};
+  for (auto& e : n->tiles)
+    if (e.first == key) {
+      *out = e.second;
+      return out->Tx > 0;
+    }
+  dda::nn::TcTile t{};
+  if (!tc_tile(d, B, np, &t)) t = dda::nn::TcTile{};
+  if (n->tiles.size() >= 64) n->tiles.erase(n->tiles.begin());
+  n->tiles.emplace_back(key, t);
+  *out = t;
+  return t.Tx > 0;
 }
 
 // the driver's tensor-map encoder, looked up once
@@ -821,17 +860,16 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
   return fn;
 }
 
-// 5-D map of the bfloat16 activations [B][Z][Y][X][cpad]: box 8 channels x (X+2) x (Ty+2) x (Tz+2) x 1
+// 4-D map of the bfloat16 activations [B * cpad/8][Z][Y][X * 8]: box 8 (Tx+2) x (Ty+2) x (Tz+2) x 1
 Err encode_act_map(CUtensorMap* m, const void* base, int cpad, const dda::nn::Dims& d, int B,
                    const dda::nn::TcTile& t) {
   auto enc = tmap_encoder();
   if (!enc) return Err::make(DDA_ECUDA, "cuTensorMapEncodeTiled is not available");
-  const cuuint64_t dims[5] = {(cuuint64_t)cpad, (cuuint64_t)d.X, (cuuint64_t)d.Y, (cuuint64_t)d.Z, (cuuint64_t)B};
-  const cuuint64_t strides[4] = {(cuuint64_t)cpad * 2, (cuuint64_t)cpad * 2 * d.X, (cuuint64_t)cpad * 2 * d.X * d.Y,
-                                 (cuuint64_t)cpad * 2 * d.X * d.Y * d.Z};
-  const cuuint32_t box[5] = {8u, (cuuint32_t)t.sx, (cuuint32_t)t.sy, (cuuint32_t)t.sz, 1u};
-  const cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
-  const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, estr,
+  const cuuint64_t dims[4] = {(cuuint64_t)d.X * 8, (cuuint64_t)d.Y, (cuuint64_t)d.Z, (cuuint64_t)B * (cpad / 8)};
+  const cuuint64_t strides[3] = {(cuuint64_t)16 * d.X, (cuuint64_t)16 * d.X * d.Y, (cuuint64_t)16 * d.X * d.Y * d.Z};
+  const cuuint32_t box[4] = {8u * (cuuint32_t)t.sx, (cuuint32_t)t.sy, (cuuint32_t)t.sz, 1u};
+  const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
+  const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return Err::make(DDA_ECUDA, "tensor-map encoding failed");
@@ -863,7 +901,7 @@ Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y
   if (n->use_tc && L.taps == dda::nn::kTaps) {
     const int np = np16(cout);
     dda::nn::TcTile tl;
-    if (tc_tile(d, B, np, &tl)) {
+    if (tc_tile_of(n, d, B, np, &tl)) {
       const int cpad = kc_n * 16;
       const size_t need = sizeof(uint16_t) * (size_t)V * cpad;
       if (need > n->xb_bytes) {
@@ -874,12 +912,13 @@ Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y
         n->xb_bytes = need;
       }
       const int64_t items = V * (cpad / 8);
-      dda::nn::k_to_bf16<<<dda::nn::blocks_for(items), 256, 0, n->stream>>>(x, xs, cin, cpad, V, n->xb);
+      dda::nn::k_to_bf16<<<dda::nn::blocks_for(items), 256, 0, n->stream>>>(x, xs, cin, cpad, d.nvox(), B, n->xb);
       DDA_CU(cudaGetLastError());
       CUtensorMap tmap;
       DDA_TRY(encode_act_map(&tmap, n->xb, cpad, d, B, tl));
       const uint4* wt = reinterpret_cast<const uint4*>(transposed ? L.wttc : L.wtc);
-      const dim3 grid((unsigned)((d.Y + tl.Ty - 1) / tl.Ty), (unsigned)((d.Z + tl.Tz - 1) / tl.Tz), (unsigned)B);
+      const dim3 grid((unsigned)(tl.ntx * ((d.Y + tl.Ty - 1) / tl.Ty)), (unsigned)((d.Z + tl.Tz - 1) / tl.Tz),
+                      (unsigned)B);
       const size_t smem = 1024 + (size_t)tl.stages * tl.stage_bytes;
       switch (np) {
 #define CASE(NP)                                                                                                  \
