@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -46,12 +47,13 @@ namespace nn {
 constexpr int kTaps = 27;
 constexpr int kConvThreads = 128;  // 4 warps, 16 voxels each
 constexpr int kVoxPerCta = 64;
-constexpr int kWgradChunk = 4096;  // voxels reduced by one weight-gradient CTA
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
+
+__device__ __forceinline__ uint32_t tc_saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint2 b) {
   asm volatile(
@@ -370,17 +372,19 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
 // bfloat16 copy of channels [0, cin) of x (xs per voxel) in planes of 8 channels, zeros above cin:
 // out[(sample * cpad/8 + c/8) * nvox + voxel] (8 channels each), the tcgen05 convolution's TMA source.
 // One thread per 8 channels of a voxel.
-__global__ void k_to_bf16(const float* __restrict__ x, int xs, int cin, int cpad, int64_t nvox, int B,
-                          uint4* __restrict__ out) {
+// mask (xs per voxel, optional): zero where it is not positive (the ReLU's gradient).
+__global__ void k_to_bf16(const float* __restrict__ x, const float* __restrict__ mask, int xs, int cin, int cpad,
+                          int64_t nvox, int B, uint4* __restrict__ out) {
   const int g8 = cpad / 8;
   const int64_t total = nvox * g8 * B;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t p = i / nvox;  // plane
     const int c = (int)(p % g8) * 8;
-    const float* src = x + (p / g8 * nvox + (i - p * nvox)) * xs;
+    const int64_t at = (p / g8 * nvox + (i - p * nvox)) * xs;
     float f[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) f[j] = (c + j < cin) ? __ldg(src + c + j) : 0.f;
+    for (int j = 0; j < 8; ++j)
+      f[j] = (c + j < cin) && (!mask || __ldg(mask + at + c + j) > 0.f) ? __ldg(x + at + c + j) : 0.f;
     out[i] = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
   }
 }
@@ -407,92 +411,224 @@ __global__ void k_pack_tc(const float* __restrict__ w, int taps, int cin, int co
   }
 }
 
-// Weight gradient partials: part[chunk][tap][kc*16 + row][nt*8 + col] = sum over the chunk's voxels
-// of x[nb(v, tap), ci] g[v, co].  grid (nchunk, taps, kc_n), block 128.
+// Weight and bias gradients.  A CTA reduces one tile of voxels of one sample for one 16-channel chunk of
+// the input and all taps: it stages the chunk's tile with its one-voxel halo and the tile's output
+// gradient (masked by the ReLU) once, in bfloat16, voxels as rows, and every tap's operand is the same
+// staged tile read at a shifted row.  Nine warps own the (dz, dy) pairs and keep three taps each; per 16
+// voxels a warp loads the gradient's fragments once (ldmatrix, transposed: voxels are the K axis of
+// both operands) and one input fragment per tap.  Rows are padded so that eight rows 16 bytes wide fall
+// on different banks.  part[tile][tap][kc*16 + row][NT*8]; the chunk-0 CTAs also sum the unrounded
+// gradient per channel (pair sums, then FP64): gbp[tile][NT*8].  Latency and staging bound; one CTA per
+// (4096 voxels, tap) with gathers straight from memory took 1.5 of the 2.6 ms of a training pass of 16
+// 16^3 samples and the channel sums 0.35, these kernels and their sums
+// about 0.25.
+constexpr int kWgT = 288;
+struct WgTile {
+  int Tx, Ty, Tz, ntx, nty, ntz;
+  int K, Kpad, rows;  // voxels, rounded to 16; staged input rows
+};
+constexpr int kWgXS = 48;  // bytes per staged input row: 16 channels and a pad of 16
+__host__ __device__ constexpr int wg_gs(int NT) { return (NT % 2 ? NT : NT + 1) * 16; }
+__host__ inline size_t wg_smem(const WgTile& t, int NT) {
+  const size_t main = (size_t)t.rows * kWgXS + (size_t)t.Kpad * wg_gs(NT) + (size_t)t.Kpad * 4;
+  const size_t red = sizeof(double) * (size_t)kWgT * 8 + sizeof(float) * 9 * 16 * NT * 8;
+  return (main > red ? main : red) + 16;
+}
+__device__ __forceinline__ void ldsm_x4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_x2t(uint32_t& r0, uint32_t& r1, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+// 8 consecutive channels c.. of a voxel row, zeros from climit on
+__device__ __forceinline__ void load8(const float* __restrict__ p, int c, int climit, bool vec, float (&f)[8]) {
+  if (vec && c + 8 <= climit) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p + c)), b = __ldg(reinterpret_cast<const float4*>(p + c) + 1);
+    f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+    f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) f[j] = c + j < climit ? __ldg(p + c + j) : 0.f;
+  }
+}
+__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
+  return make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+}
+
 template <int NT>
-__global__ void __launch_bounds__(kConvThreads) k_wgrad(const float* __restrict__ x, int xs, int cin,
-                                                      const float* __restrict__ gy, int gs, int cout, int taps,
-                                                      Dims d, int64_t V, float* __restrict__ part, int kc_n) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane >> 2, t = lane & 3;
-  const int chunk = blockIdx.x, tap = blockIdx.y, kc = blockIdx.z;
-  const int64_t vbeg = (int64_t)chunk * kWgradChunk;
-  const int64_t vend = min(V, vbeg + kWgradChunk);
-  float acc[NT][4];
+__global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int xs, int cin,
+                                               const float* __restrict__ gy, const float* __restrict__ mask, int gs,
+                                               int cout, int taps, Dims d, WgTile tl, float* __restrict__ part,
+                                               double* __restrict__ gbp, int kc_n) {
+  extern __shared__ __align__(16) unsigned char sm_wg[];
+  constexpr int GS = wg_gs(NT);
+  unsigned char* xt = sm_wg;
+  unsigned char* gt = xt + (size_t)tl.rows * kWgXS;
+  int* off = reinterpret_cast<int*>(gt + (size_t)tl.Kpad * GS);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int hal = taps == kTaps ? 1 : 0;
+  int t = blockIdx.x;
+  const int kc = blockIdx.y;
+  const int tile = t;
+  const int x0 = (t % tl.ntx) * tl.Tx;
+  t /= tl.ntx;
+  const int y0 = (t % tl.nty) * tl.Ty;
+  t /= tl.nty;
+  const int z0 = (t % tl.ntz) * tl.Tz, b = t / tl.ntz;
+  const int sx = tl.Tx + 2 * hal, sy = tl.Ty + 2 * hal;
+  const int64_t vb = (int64_t)b * d.nvox();
+  // input chunk with halo
+  const bool xv = xs % 4 == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+  for (int i = tid; i < tl.rows * 2; i += kWgT) {
+    const int r = i >> 1, h = i & 1;
+    const int xx = r % sx, q = r / sx;
+    const int yy = q % sy, zz = q / sy;
+    const int gx = x0 + xx - hal, gyy = y0 + yy - hal, gz = z0 + zz - hal;
+    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (gx >= 0 && gx < d.X && gyy >= 0 && gyy < d.Y && gz >= 0 && gz < d.Z)
+      load8(x + (vb + ((int64_t)gz * d.Y + gyy) * d.X + gx) * xs, kc * 16 + h * 8, cin, xv, f);
+    *reinterpret_cast<uint4*>(xt + (size_t)r * kWgXS + h * 16) = pack8(f);
+  }
+  // output gradient: thread = (voxel group, 8-channel column)
+  const bool gv = gs % 4 == 0 && (reinterpret_cast<uintptr_t>(gy) & 15) == 0 &&
+                  (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+  constexpr int NG = kWgT / NT;
+  const int nt0 = tid % NT, vg = tid / NT;
+  float bh[8], bl[8];
 #pragma unroll
-  for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-  const int ci_a = kc * 16 + g, ci_b = kc * 16 + g + 8;
-  for (int64_t vb = vbeg + warp * 16; vb < vend; vb += 4 * 16) {
-    // voxel columns of this k-step: vb + 2t, +1, +8, +9
-    const int64_t vc[4] = {vb + 2 * t, vb + 2 * t + 1, vb + 2 * t + 8, vb + 2 * t + 9};
-    float xa[4], xb[4];
-    int64_t vv[4];
+  for (int j = 0; j < 8; ++j) bh[j] = bl[j] = 0.f;
+  if (vg < NG)
+    for (int k = vg; k < tl.Kpad; k += NG) {
+      const int xx = k % tl.Tx, q = k / tl.Tx;
+      const int yy = q % tl.Ty, zz = q / tl.Ty;
+      float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (k < tl.K && x0 + xx < d.X && y0 + yy < d.Y && z0 + zz < d.Z) {
+        const int64_t v = vb + ((int64_t)(z0 + zz) * d.Y + y0 + yy) * d.X + x0 + xx;
+        load8(gy + v * gs, nt0 * 8, cout, gv, f);
+        if (mask) {
+          float o[8];
+          load8(mask + v * gs, nt0 * 8, cout, gv, o);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      vv[q] = vc[q] < vend ? vc[q] : -1;
-      const int64_t nb = vv[q] >= 0 ? neighbour(vv[q], d, tap, taps, false) : -1;
-      xa[q] = (nb >= 0 && ci_a < cin) ? __ldg(x + nb * xs + ci_a) : 0.f;
-      xb[q] = (nb >= 0 && ci_b < cin) ? __ldg(x + nb * xs + ci_b) : 0.f;
+          for (int j = 0; j < 8; ++j) f[j] = o[j] > 0.f ? f[j] : 0.f;
+        }
+      }
+      *reinterpret_cast<uint4*>(gt + (size_t)k * GS + nt0 * 16) = pack8(f);
+      // padding voxels (zero gradient) take the first voxel's rows, so that shifted rows stay in the tile
+      if (nt0 == 0) off[k] = k < tl.K ? ((zz + hal) * sy + yy + hal) * sx + xx + hal : (hal * sy + hal) * sx + hal;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float s = __fadd_rn(bh[j], f[j]), w = __fsub_rn(s, bh[j]);
+        bl[j] = __fadd_rn(bl[j], __fadd_rn(__fsub_rn(bh[j], __fsub_rn(s, w)), __fsub_rn(f[j], w)));
+        bh[j] = s;
+      }
     }
-    uint32_t a[4];
-    a[0] = pack_bf16(xa[0], xa[1]);
-    a[1] = pack_bf16(xb[0], xb[1]);
-    a[2] = pack_bf16(xa[2], xa[3]);
-    a[3] = pack_bf16(xb[2], xb[3]);
+  __syncthreads();
+  const uint32_t xa = tc_saddr(xt) + ((lane >> 3) & 1) * 16, ga = tc_saddr(gt);
+  const int arow = (lane >> 4) * 8 + (lane & 7);        // A: voxel of this lane's matrix row
+  const int brow = ((lane >> 3) & 1) * 8 + (lane & 7);  // B
+  constexpr int ND = 3;  // taps per warp
+  float acc[ND][NT][4];
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      const int co = n * 8 + g;
-      float gv[4];
+  for (int q = 0; q < ND; ++q)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) gv[q] = (vv[q] >= 0 && co < cout) ? __ldg(gy + vv[q] * gs + co) : 0.f;
-      const uint2 b = make_uint2(pack_bf16(gv[0], gv[1]), pack_bf16(gv[2], gv[3]));
-      mma_bf16(acc[n], a, b);
+    for (int n = 0; n < NT; ++n) acc[q][n][0] = acc[q][n][1] = acc[q][n][2] = acc[q][n][3] = 0.f;
+  const int shift = hal ? ((warp / 3 - 1) * sy + (warp % 3 - 1)) * sx - 1 : 0;
+  const int kstep = hal ? 16 : 16 * 9;
+  for (int k0 = hal ? 0 : warp * 16; k0 < tl.Kpad; k0 += kstep) {
+    uint32_t bf[NT][2];
+#pragma unroll
+    for (int n = 0; n + 1 < NT; n += 2) {
+      uint32_t r[4];
+      ldsm_x4t(r, ga + (uint32_t)((k0 + brow) * GS + n * 16 + (lane >> 4) * 16));
+      bf[n][0] = r[0]; bf[n][1] = r[1];
+      bf[n + 1][0] = r[2]; bf[n + 1][1] = r[3];
+    }
+    if constexpr (NT % 2 == 1) ldsm_x2t(bf[NT - 1][0], bf[NT - 1][1], ga + (uint32_t)((k0 + brow) * GS + (NT - 1) * 16));
+    const uint32_t o = xa + (uint32_t)((off[k0 + arow] + shift) * kWgXS);
+#pragma unroll
+    for (int q = 0; q < ND; ++q) {
+      if (!hal && q) continue;
+      uint32_t af[4];
+      ldsm_x4t(af, o + (uint32_t)(q * kWgXS));
+#pragma unroll
+      for (int n = 0; n < NT; ++n) mma_bf16(acc[q][n], af, make_uint2(bf[n][0], bf[n][1]));
     }
   }
-  // reduce the 4 warps in shared memory, fixed order
-  __shared__ float red[4][16][NT * 8];
+  const int g = lane >> 2, tq = lane & 3;
+  if (hal) {
 #pragma unroll
-  for (int n = 0; n < NT; ++n) {
-    red[warp][g][n * 8 + 2 * t] = acc[n][0];
-    red[warp][g][n * 8 + 2 * t + 1] = acc[n][1];
-    red[warp][g + 8][n * 8 + 2 * t] = acc[n][2];
-    red[warp][g + 8][n * 8 + 2 * t + 1] = acc[n][3];
+    for (int q = 0; q < ND; ++q) {
+      float* out = part + (((int64_t)tile * kTaps + warp * 3 + q) * kc_n * 16 + kc * 16) * (NT * 8);
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        *reinterpret_cast<float2*>(out + (int64_t)g * (NT * 8) + n * 8 + 2 * tq) = make_float2(acc[q][n][0], acc[q][n][1]);
+        *reinterpret_cast<float2*>(out + (int64_t)(g + 8) * (NT * 8) + n * 8 + 2 * tq) =
+            make_float2(acc[q][n][2], acc[q][n][3]);
+      }
+    }
+  }
+  __syncthreads();  // the staged tiles are read; their memory holds the reductions now
+  double* red = reinterpret_cast<double*>(sm_wg);  // [NG][NT * 8]
+  float* wred = reinterpret_cast<float*>(red + kWgT * 8);
+  if (!hal) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        wred[(warp * 16 + g + 8 * (e >> 1)) * (NT * 8) + n * 8 + 2 * tq + (e & 1)] = acc[0][n][e];
+  }
+  if (kc == 0 && vg < NG) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) red[vg * (NT * 8) + nt0 * 8 + j] = (double)bh[j] + (double)bl[j];
   }
   __syncthreads();
-  float* out = part + (((int64_t)chunk * taps + tap) * kc_n * 16 + kc * 16) * (NT * 8);
-  for (int i = threadIdx.x; i < 16 * NT * 8; i += blockDim.x) {
-    const int row = i / (NT * 8), col = i % (NT * 8);
-    out[(int64_t)row * (NT * 8) + col] = red[0][row][col] + red[1][row][col] + red[2][row][col] + red[3][row][col];
+  if (!hal) {
+    float* out = part + ((int64_t)tile * kc_n * 16 + kc * 16) * (NT * 8);
+    for (int i = tid; i < 16 * NT * 8; i += kWgT) {
+      float v = 0.f;
+      for (int w = 0; w < 9; ++w) v += wred[w * 16 * NT * 8 + i];
+      out[i] = v;
+    }
+  }
+  if (kc == 0) {
+    for (int i = tid; i < NT * 64; i += kWgT) {  // eight lanes per channel
+      const int c = i >> 3;
+      double v = 0.0;
+      for (int k = i & 7; k < NG; k += 8) v += red[k * (NT * 8) + c];
+      for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if ((i & 7) == 0) gbp[(int64_t)tile * (NT * 8) + c] = v;
+    }
   }
 }
 
-// gw[tap][ci][co] = sum_chunk part[chunk][tap][ci][co] (ci < cin, co < cout)
-__global__ void k_wgrad_sum(const float* __restrict__ part, int nchunk, int taps, int cinp, int coutp, int cin,
-                            int cout, float* __restrict__ gw) {
-  const int total = taps * cin * cout;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int co = i % cout;
-    const int r = i / cout;
-    const int ci = r % cin, tap = r / cin;
-    float s = 0.f;
-    for (int c = 0; c < nchunk; ++c) s += part[(((int64_t)c * taps + tap) * cinp + ci) * coutp + co];
-    gw[i] = s;
-  }
-}
-
-// gb[co] = sum_v g[v, co]  (one block per channel, fixed-order tree)
-__global__ void k_colsum(const float* __restrict__ g, int gs, int cout, int64_t V, float* __restrict__ gb) {
-  const int co = blockIdx.x;
+// gw[tap][ci][co] = sum over tiles of part (ci < cin, co < cout), then the bias sums: 32 values per CTA,
+// eight threads each over every eighth tile, added in order
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, const double* __restrict__ gbp,
+                                                   int ntile, int taps, int cinp, int coutp, int cin, int cout,
+                                                   float* __restrict__ gw, float* __restrict__ gb) {
+  __shared__ double red[8][33];
+  const int nw = taps * cin * cout;
+  const int i = blockIdx.x * 32 + (threadIdx.x & 31), seg = threadIdx.x >> 5;
   double s = 0.0;
-  for (int64_t v = threadIdx.x; v < V; v += blockDim.x) s += g[v * gs + co];
-  __shared__ double red[256];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
+  if (i < nw) {
+    const int co = i % cout, r = i / cout;
+    const int ci = r % cin, tap = r / cin;
+    const int64_t stride = (int64_t)taps * cinp * coutp, at = ((int64_t)tap * cinp + ci) * coutp + co;
+    float f = 0.f;
+    for (int c = seg; c < ntile; c += 8) f += part[c * stride + at];
+    s = f;
+  } else if (i < nw + cout) {
+    for (int c = seg; c < ntile; c += 8) s += gbp[(int64_t)c * coutp + i - nw];
   }
-  if (threadIdx.x == 0) gb[co] = (float)red[0];
+  red[seg][threadIdx.x & 31] = s;
+  __syncthreads();
+  if (seg == 0 && i < nw + cout) {
+    for (int q = 1; q < 8; ++q) s += red[q][threadIdx.x & 31];
+    if (i < nw) gw[i] = (float)s;
+    else gb[i - nw] = (float)s;
+  }
 }
 
 // g *= (out > 0)
@@ -888,8 +1024,9 @@ Err tc_smem_optin() {
 }
 
 // y = conv(x) for layer L; x has xs channels (uses the first cin), y gets ys channels (writes first cout)
+// (mask: x counts as zero where mask is not positive)
 Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y, int ys, bool relu, dda::nn::Dims d,
-         int B, bool transposed) {
+         int B, bool transposed, const float* mask = nullptr) {
   const int64_t V = (int64_t)B * d.nvox();
   const int blocks = (int)((V + dda::nn::kVoxPerCta - 1) / dda::nn::kVoxPerCta);
   const int kc_n = transposed ? L.cin_t_kc : L.kc_n;
@@ -912,7 +1049,7 @@ Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y
         n->xb_bytes = need;
       }
       const int64_t items = V * (cpad / 8);
-      dda::nn::k_to_bf16<<<dda::nn::blocks_for(items), 256, 0, n->stream>>>(x, xs, cin, cpad, d.nvox(), B, n->xb);
+      dda::nn::k_to_bf16<<<dda::nn::blocks_for(items), 256, 0, n->stream>>>(x, mask, xs, cin, cpad, d.nvox(), B, n->xb);
       DDA_CU(cudaGetLastError());
       CUtensorMap tmap;
       DDA_TRY(encode_act_map(&tmap, n->xb, cpad, d, B, tl));
@@ -935,6 +1072,10 @@ Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y
       dda::add_launches(2);
       return Err::Ok();
     }
+  }
+  if (mask) {  // the mma.sync kernel reads x as it is
+    dda::nn::k_relu_bwd<<<dda::nn::blocks_for(V * xs), 256, 0, n->stream>>>(const_cast<float*>(x), mask, V * xs);
+    dda::add_launches(1);
   }
   switch (nt_n) {
 #define CASE(NT)                                                                                                   \
@@ -962,31 +1103,68 @@ Err grow_ws(dda_unet* n, float** p, size_t* cap, size_t bytes) {
   return Err::Ok();
 }
 
-// weight and bias gradients of layer L from input x (xs channels) and output gradient gy (gs channels)
-Err wgrad(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, const float* gy, int gs, dda::nn::Dims d,
-          int B) {
-  const int64_t V = (int64_t)B * d.nvox();
-  const int nchunk = (int)((V + dda::nn::kWgradChunk - 1) / dda::nn::kWgradChunk);
-  const size_t need = sizeof(float) * (size_t)nchunk * L.taps * L.kc_n * 16 * L.nt_n * 8;
-  DDA_TRY(grow_ws(n, &n->part, &n->part_bytes, need));
-  dim3 grid(nchunk, L.taps, L.kc_n);
+// Tile of the weight gradient: the least modelled time over x splits of at most 32 voxels and (Ty, Tz):
+// per CTA a fixed 2 us, the staged rows and the MMAs of its K voxels; two CTAs per SM; plus the partials'
+// traffic at 4 TB/s.
+dda::nn::WgTile wg_tile(const dda::nn::Dims& d, int B, int taps, int kc_n, int NT) {
+  const int hal = taps == dda::nn::kTaps ? 1 : 0;
+  dda::nn::WgTile best{};
+  double bt = 1e300;
+  const int ntx = (d.X + 31) / 32, Tx = (d.X + ntx - 1) / ntx;
+  for (int Tz = 1; Tz <= std::min(d.Z, 8); ++Tz)
+    for (int Ty = 1; Ty <= std::min(d.Y, 32); ++Ty) {
+      dda::nn::WgTile t{};
+      t.Tx = Tx; t.Ty = Ty; t.Tz = Tz;
+      t.ntx = ntx; t.nty = ceil_div(d.Y, Ty); t.ntz = ceil_div(d.Z, Tz);
+      t.K = Tx * Ty * Tz;
+      if (t.K > 1024) break;
+      t.Kpad = (t.K + 15) / 16 * 16;
+      t.rows = (Tx + 2 * hal) * (Ty + 2 * hal) * (Tz + 2 * hal);
+      const size_t sm = dda::nn::wg_smem(t, NT);
+      if (sm > 110 * 1024) break;
+      const double ntile = (double)t.ntx * t.nty * t.ntz * B;
+      const double us = 2.0 + 0.002 * t.rows + 0.0012 * t.Kpad * (NT + 2);
+      const double total = std::ceil(ntile * kc_n / 304.0) * us + ntile * taps * kc_n * 16.0 * NT * 64.0 / 4e6;
+      if (total < bt) { bt = total; best = t; }
+    }
+  return best;
+}
+
+// weight and bias gradients of layer L from input x (xs channels) and output gradient gy (gs channels),
+// masked by (mask > 0) when given
+Err wgrad(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, const float* gy, const float* mask, int gs,
+          dda::nn::Dims d, int B) {
+  const dda::nn::WgTile t = wg_tile(d, B, L.taps, L.kc_n, L.nt_n);
+  const int64_t ntile = (int64_t)t.ntx * t.nty * t.ntz * B;
+  if (t.K == 0 || ntile > (1 << 30)) return Err::make(DDA_EUNSUPPORTED, "no weight-gradient tile for this grid");
+  const int cinp = L.kc_n * 16, coutp = L.nt_n * 8;
+  const size_t pf = (size_t)ntile * L.taps * cinp * coutp;
+  DDA_TRY(grow_ws(n, &n->part, &n->part_bytes, sizeof(float) * pf + sizeof(double) * (size_t)ntile * coutp));
+  double* gbp = reinterpret_cast<double*>(n->part + pf);  // pf is a multiple of 128
+  const dim3 grid((unsigned)ntile, L.kc_n);
+  const size_t sm = dda::nn::wg_smem(t, L.nt_n);
   switch (L.nt_n) {
-#define CASE(NT)                                                                                                    \
-  case NT:                                                                                                          \
-    dda::nn::k_wgrad<NT><<<grid, dda::nn::kConvThreads, 0, n->stream>>>(x, xs, L.cin, gy, gs, L.cout, L.taps, d, V, \
-                                                                        n->part, L.kc_n);                           \
-    break;
+#define CASE(NT)                                                                                                     \
+  case NT: {                                                                                                         \
+    static std::atomic<bool> done{false};                                                                            \
+    if (!done) {                                                                                                     \
+      DDA_CU(cudaFuncSetAttribute(dda::nn::k_wgrad<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024));   \
+      done = true;                                                                                                   \
+    }                                                                                                                \
+    dda::nn::k_wgrad<NT><<<grid, dda::nn::kWgT, sm, n->stream>>>(x, xs, L.cin, gy, mask, gs, L.cout, L.taps, d, t,   \
+                                                                 n->part, gbp, L.kc_n);                              \
+    break;                                                                                                           \
+  }
     CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
 #undef CASE
     default: return Err::make(DDA_EUNSUPPORTED, "layer wider than 64 channels");
   }
   DDA_CU(cudaGetLastError());
-  const int tot = L.taps * L.cin * L.cout;
-  dda::nn::k_wgrad_sum<<<dda::nn::blocks_for(tot), 256, 0, n->stream>>>(n->part, nchunk, L.taps, L.kc_n * 16,
-                                                                        L.nt_n * 8, L.cin, L.cout, n->g + L.woff);
-  dda::nn::k_colsum<<<L.cout, 256, 0, n->stream>>>(gy, gs, L.cout, V, n->g + L.boff);
+  const int tot = L.taps * L.cin * L.cout + L.cout;
+  dda::nn::k_wgrad_sum<<<(tot + 31) / 32, 256, 0, n->stream>>>(n->part, gbp, (int)ntile, L.taps, cinp, coutp, L.cin,
+                                                              L.cout, n->g + L.woff, n->g + L.boff);
   DDA_CU(cudaGetLastError());
-  dda::add_launches(3);
+  dda::add_launches(2);
   return Err::Ok();
 }
 
@@ -1067,17 +1245,14 @@ Err forward_pass(dda_unet* n, const Acts& a, int B, dda::nn::Dims d1) {
 }
 
 // conv backward for layer li: output activation `out` (for the ReLU mask), its gradient g_out (gs channels,
-// modified in place by the mask), input activation x (xs channels); writes the input gradient to gx (gxs ch.)
+// taken as zero where out is not positive), input activation x (xs channels); writes the input gradient to
+// gx (gxs ch.)
 Err conv_back(dda_unet* n, int li, const float* x, int xs, const float* out, float* g_out, int gs, float* gx, int gxs,
               dda::nn::Dims d, int B, bool relu) {
   const auto& L = n->layers[li];
-  const int64_t V = (int64_t)B * d.nvox();
-  if (relu) {
-    dda::nn::k_relu_bwd<<<dda::nn::blocks_for(V * gs), 256, 0, n->stream>>>(g_out, out, V * gs);
-    dda::add_launches(1);
-  }
-  DDA_TRY(wgrad(n, L, x, xs, g_out, gs, d, B));
-  if (gx) DDA_TRY(conv(n, L, g_out, gs, gx, gxs, false, d, B, true));
+  const float* mask = relu ? out : nullptr;
+  DDA_TRY(wgrad(n, L, x, xs, g_out, mask, gs, d, B));
+  if (gx) DDA_TRY(conv(n, L, g_out, gs, gx, gxs, false, d, B, true, mask));
   return Err::Ok();
 }
 
