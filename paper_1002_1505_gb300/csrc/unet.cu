@@ -173,7 +173,8 @@ __global__ void __launch_bounds__(kConvThreads) k_conv(const float* __restrict__
 // as two 8-channel halves in which staged voxel s = (zz * (Ty+2) + yy) * (Tx+2) + xx sits at byte
 // 16 s.  A row of a plane is contiguous, so the box's inner extent is 16 (Tx+2) bytes, up to 512
 // (with channels innermost in one tensor it was 16 bytes a voxel, and the copies set the pace:
-// 12 -> 12 channels on 2 x 64 x 48 x 32 in 71 us, now 36).  In that layout the rows of an
+// 12 -> 12 channels on 2 x 64 x 48 x 32 in 71 us, with planes 36, with the lean issue loop and the tile
+// model below 23).  In that layout the rows of an
 // MMA's A operand are 16 bytes apart, so the K-major no-swizzle descriptor with an 8-row stride of
 // 128 bytes addresses 128 consecutive staged voxels from any start, and the operand of tap
 // (dz, dy, dx) is the output rows' operand moved by dz (Ty+2)(Tx+2) + dy (Tx+2) + dx rows: one
@@ -265,12 +266,25 @@ struct TcTile {
 
 __host__ __device__ inline uint32_t tc_act_bytes(const TcTile& t) { return 2u * (uint32_t)t.rows_alloc * 16u; }
 
-// wpk: per (chunk, tap) NP x 16 bf16 in the B-tile layout, chunks outermost
+// where a convolution's results go: FP32 channels-last y (ys per voxel, the first cout written; may be
+// null) and / or bfloat16 planes of 8 channels (planes p0 .. p0 + ceil8(cout) of g8 per sample; may be
+// null), the latter zeroed where mask (FP32, ys per voxel; may be null) is not positive
+struct ConvOut {
+  float* y;
+  int ys;
+  uint4* planes;
+  int g8, p0, np;  // np: planes written
+  const float* mask;
+};
+
+// wpk: per (chunk, tap) NP x 16 bf16 in the B-tile layout, chunks outermost.  Thread 32 keeps the chunk
+// buffers filled, thread 0 issues the MMAs: their descriptors differ only in the row (16-byte units in
+// the address field), so one issue costs a few instructions.
 template <int NP>
 __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ CUtensorMap tmap,
                                                         const uint4* __restrict__ wpk, int kc_n, bool flip,
-                                                        const float* __restrict__ bias, float* __restrict__ y, int ys,
-                                                        int cout, bool relu, Dims d, TcTile tl,
+                                                        const float* __restrict__ bias, ConvOut out, int cout,
+                                                        bool relu, Dims d, TcTile tl,
                                                         unsigned int* __restrict__ fault) {
   static_assert(NP % 16 == 0 && NP >= 16 && NP <= 128, "N must be a multiple of 16 in [16, 128]");
   extern __shared__ __align__(1024) unsigned char smem_tc[];
@@ -287,41 +301,49 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
   const uint32_t w_bytes = (uint32_t)kTaps * NP * 32u;
   const uint32_t box_bytes = 16u * (uint32_t)(tl.sx * tl.sy * tl.sz);
   const int plane = tl.sx * tl.sy;
-  if (warp == 0) tc::alloc(tmem_slot, tl.ncol);
-  if (tid == 0) {
+  if (tid == 32) {
     for (int i = 0; i < 5; ++i) bulk::mbar_init(&full[i], 1);
   }
+  if (warp == 0) tc::alloc(tmem_slot, tl.ncol);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = *tmem_slot;
   bool ok = true;
-  if (tid == 0) {
-    uint32_t fph[2] = {0u, 0u}, eph[2] = {0u, 0u};
+  if (tid == 32) {
     for (int kc = 0; kc < kc_n; ++kc) {
       const int s = (tl.stages == 2) ? (kc & 1) : 0;
       unsigned char* act = buf0 + (size_t)s * tl.stage_bytes;
-      unsigned char* wb = act + act_bytes;
-      if (kc >= tl.stages) {  // the MMAs of chunk kc - stages have read this buffer
-        ok = bulk::mbar_wait(&empty[s], eph[s], kTcMaxPolls, fault) && ok;
-        eph[s] ^= 1u;
-      }
+      if (kc >= tl.stages)  // the MMAs of chunk kc - stages have read this buffer
+        bulk::mbar_wait(&empty[s], (uint32_t)(kc / tl.stages - 1) & 1u, kTcMaxPolls, fault);
       bulk::mbar_arrive_expect_tx(&full[s], 2u * box_bytes + w_bytes);
       const int pl = (b * kc_n + kc) * 2;  // the chunk's two planes of 8 channels
       tc::tma_load_4d(act, &tmap, 8 * (tx0 - 1), ty0 - 1, tz0 - 1, pl, &full[s]);
       tc::tma_load_4d(act + half_bytes, &tmap, 8 * (tx0 - 1), ty0 - 1, tz0 - 1, pl + 1, &full[s]);
-      bulk::load_g2s(wb, wpk + (int64_t)kc * kTaps * NP * 2, w_bytes, &full[s]);
-      ok = bulk::mbar_wait(&full[s], fph[s], kTcMaxPolls, fault) && ok;
-      fph[s] ^= 1u;
+      bulk::load_g2s(act + act_bytes, wpk + (int64_t)kc * kTaps * NP * 2, w_bytes, &full[s]);
+    }
+  }
+  if (tid == 0) {
+    const int sg = flip ? -1 : 1;
+    for (int kc = 0; kc < kc_n; ++kc) {
+      const int s = (tl.stages == 2) ? (kc & 1) : 0;
+      unsigned char* act = buf0 + (size_t)s * tl.stage_bytes;
+      ok = bulk::mbar_wait(&full[s], (uint32_t)(kc / tl.stages) & 1u, kTcMaxPolls, fault) && ok;
       tc::fence_after();
-      for (int mt = 0; mt < tl.n_mt; ++mt)
-        for (int t = 0; t < kTaps; ++t) {
-          const int tt = flip ? (kTaps - 1 - t) : t;
-          const int off = (tt / 9 - 1) * plane + ((tt / 3) % 3 - 1) * tl.sx + (tt % 3 - 1);
-          const uint32_t row = (uint32_t)(tl.q_first + mt * 128 + off);
-          tc::mma(tmem + (uint32_t)(mt * NP), tc::desc(act + (size_t)row * 16u, half_bytes, 128),
-                  tc::desc(wb + (size_t)t * NP * 32u, 128, 256), tc::idesc_bf16(NP), (kc > 0 || t > 0) ? 1u : 0u);
-        }
+      const uint64_t a0 = tc::desc(act, half_bytes, 128), b0 = tc::desc(act + act_bytes, 128, 256);
+      for (int mt = 0; mt < tl.n_mt; ++mt) {
+        const uint64_t am = a0 + (uint32_t)(tl.q_first + mt * 128);
+        const uint32_t dt = tmem + (uint32_t)(mt * NP);
+        uint64_t bt = b0;
+        for (int dz = -sg; dz != 2 * sg; dz += sg)
+          for (int dy = -sg; dy != 2 * sg; dy += sg) {
+            const uint64_t ar = am + (int64_t)(dz * plane + dy * tl.sx);
+            tc::mma(dt, ar - (int64_t)sg, bt, tc::idesc_bf16(NP), (kc > 0 || dz != -sg || dy != -sg) ? 1u : 0u);
+            tc::mma(dt, ar, bt + 2 * NP, tc::idesc_bf16(NP), 1u);
+            tc::mma(dt, ar + (int64_t)sg, bt + 4 * NP, tc::idesc_bf16(NP), 1u);
+            bt += 6 * NP;
+          }
+      }
       tc::commit(&empty[s]);
     }
     tc::commit(done);
@@ -329,7 +351,9 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
   ok = bulk::mbar_wait(done, 0u, kTcMaxPolls, fault) && ok;
   tc::fence_after();
   const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-  const bool vec = ys % 4 == 0 && cout % 4 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0;
+  const int ys = out.ys;
+  const bool vec = ys % 4 == 0 && cout % 4 == 0 && (reinterpret_cast<uintptr_t>(out.y) & 15) == 0;
+  const int64_t nvox = d.nvox();
   for (int mt = 0; mt < tl.n_mt; ++mt) {
     const int q = tl.q_first + mt * 128 + tid;
     const int zz = q / plane, r = q - zz * plane;
@@ -337,7 +361,10 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
     const int z = tz0 + zz - 1, yv = ty0 + yy - 1, x = tx0 + xx - 1;
     const bool valid = ok && zz >= 1 && zz <= tl.Tz && yy >= 1 && yy <= tl.Ty && xx >= 1 && xx <= tl.Tx && z < d.Z &&
                        yv < d.Y && x < d.X;
-    float* yo = y + ((((int64_t)b * d.Z + (valid ? z : 0)) * d.Y + (valid ? yv : 0)) * d.X + (valid ? x : 0)) * ys;
+    const int64_t vox = valid ? ((int64_t)z * d.Y + yv) * d.X + x : 0;
+    float* yo = out.y + (b * nvox + vox) * ys;
+    uint4* po = out.planes + ((int64_t)b * out.g8 + out.p0) * nvox + vox;
+    const float* mo = out.mask + (b * nvox + vox) * ys;
 #pragma unroll
     for (int c0 = 0; c0 < NP; c0 += 16) {
       float acc[16];
@@ -351,15 +378,30 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_tc(const __grid_constant__ 
             if (relu) acc[j] = fmaxf(acc[j], 0.f);
           }
         }
-        if (vec) {
+        if (out.y) {
+          if (vec) {
 #pragma unroll
-          for (int j = 0; j < 16; j += 4)
-            if (c0 + j < cout)
-              *reinterpret_cast<float4*>(yo + c0 + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
-        } else {
+            for (int j = 0; j < 16; j += 4)
+              if (c0 + j < cout)
+                *reinterpret_cast<float4*>(yo + c0 + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+          } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (c0 + j < cout) yo[c0 + j] = acc[j];
+            for (int j = 0; j < 16; ++j)
+              if (c0 + j < cout) yo[c0 + j] = acc[j];
+          }
+        }
+        if (out.planes) {
+          if (out.mask) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (c0 + j < cout && !(__ldg(mo + c0 + j) > 0.f)) acc[j] = 0.f;
+          }
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (c0 / 8 + h < out.np)
+              po[(int64_t)(c0 / 8 + h) * nvox] =
+                  make_uint4(pack_bf16(acc[8 * h], acc[8 * h + 1]), pack_bf16(acc[8 * h + 2], acc[8 * h + 3]),
+                             pack_bf16(acc[8 * h + 4], acc[8 * h + 5]), pack_bf16(acc[8 * h + 6], acc[8 * h + 7]));
         }
       }
     }
@@ -458,7 +500,8 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
 }
 
 template <int NT>
-__global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int xs, int cin,
+__global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int xs, const uint4* __restrict__ xp,
+                                               int cin,
                                                const float* __restrict__ gy, const float* __restrict__ mask, int gs,
                                                int cout, int taps, Dims d, WgTile tl, float* __restrict__ part,
                                                double* __restrict__ gbp, int kc_n) {
@@ -486,10 +529,18 @@ __global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int
     const int xx = r % sx, q = r / sx;
     const int yy = q % sy, zz = q / sy;
     const int gx = x0 + xx - hal, gyy = y0 + yy - hal, gz = z0 + zz - hal;
-    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (gx >= 0 && gx < d.X && gyy >= 0 && gyy < d.Y && gz >= 0 && gz < d.Z)
-      load8(x + (vb + ((int64_t)gz * d.Y + gyy) * d.X + gx) * xs, kc * 16 + h * 8, cin, xv, f);
-    *reinterpret_cast<uint4*>(xt + (size_t)r * kWgXS + h * 16) = pack8(f);
+    uint4 val = make_uint4(0u, 0u, 0u, 0u);
+    if (gx >= 0 && gx < d.X && gyy >= 0 && gyy < d.Y && gz >= 0 && gz < d.Z) {
+      const int64_t v = ((int64_t)gz * d.Y + gyy) * d.X + gx;
+      if (xp) {  // already rounded, in planes of 8 channels
+        val = __ldg(xp + ((int64_t)b * 2 * kc_n + kc * 2 + h) * d.nvox() + v);
+      } else {
+        float f[8];
+        load8(x + (vb + v) * xs, kc * 16 + h * 8, cin, xv, f);
+        val = pack8(f);
+      }
+    }
+    *reinterpret_cast<uint4*>(xt + (size_t)r * kWgXS + h * 16) = val;
   }
   // output gradient: thread = (voxel group, 8-channel column)
   const bool gv = gs % 4 == 0 && (reinterpret_cast<uintptr_t>(gy) & 15) == 0 &&
@@ -731,6 +782,65 @@ __global__ void k_copy_ch(const float* __restrict__ src, int sc, int soff, float
   }
 }
 
+// 2x2x2 average pooling of FP32 channels-last x (C channels, twice the dims d) into bfloat16 planes of 8
+// channels (g8 per sample, zeros above C); the same sums as k_pool.  One thread per 8 channels of a voxel.
+__global__ void k_pool_planes(const float* __restrict__ x, uint4* __restrict__ out, int C, int g8, Dims d, int B) {
+  const int64_t nv = d.nvox(), total = nv * g8 * B;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t p = i / nv, v = i - p * nv;
+    const int c = (int)(p % g8) * 8;
+    const int64_t b = p / g8;
+    const int xx = (int)(v % d.X), yy = (int)(v / d.X % d.Y), zz = (int)(v / d.X / d.Y);
+    const int X2 = 2 * d.X, Y2 = 2 * d.Y, Z2 = 2 * d.Z;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int q = 0; q < 8; ++q) {
+      const int z = 2 * zz + (q >> 2), y2 = 2 * yy + ((q >> 1) & 1), x2 = 2 * xx + (q & 1);
+      float f[8];
+      load8(x + (((b * Z2 + z) * Y2 + y2) * X2 + x2) * C, c, C, C % 4 == 0, f);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) s[j] += f[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] *= 0.125f;
+    out[i] = pack8(s);
+  }
+}
+
+// nearest x2 upsampling between planes: planes [0, n) of dst (g8 per sample, dims d) from src (sg8 per
+// sample, half the dims), and zeros in planes [z0, g8) of dst
+__global__ void k_up_planes(const uint4* __restrict__ src, int sg8, int n, uint4* __restrict__ dst, int g8, int z0,
+                            Dims d, int B) {
+  const int64_t nv = d.nvox();
+  const int np = n + g8 - z0;
+  const int Xc = d.X / 2, Yc = d.Y / 2, Zc = d.Z / 2;
+  const int64_t nvc = (int64_t)Xc * Yc * Zc, total = nv * np * B;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t q = i / nv, v = i - q * nv;
+    const int p = (int)(q % np);
+    const int64_t b = q / np;
+    uint4 val = make_uint4(0u, 0u, 0u, 0u);
+    if (p < n) {
+      const int x = (int)(v % d.X), y = (int)(v / d.X % d.Y), z = (int)(v / d.X / d.Y);
+      val = __ldg(src + (b * sg8 + p) * nvc + ((int64_t)(z / 2) * Yc + y / 2) * Xc + x / 2);
+    }
+    dst[(b * g8 + (p < n ? p : z0 + p - n)) * nv + v] = val;
+  }
+}
+
+// partial sums of the mask, one per CTA
+__global__ void k_mask_sum(const float* __restrict__ mask, int64_t V, double* __restrict__ part) {
+  double s = 0.0;
+  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < V; v += (int64_t)gridDim.x * blockDim.x) s += mask[v];
+  __shared__ double red[256];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+}
+
 // masked MSE: loss partials and gradient g = 2 m (y - t) / (count * C)
 __global__ void k_loss(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask, int C,
                        int64_t V, double inv_cnt, float* __restrict__ g, double* __restrict__ part) {
@@ -872,9 +982,11 @@ struct dda_unet {
   size_t part_bytes = 0;
   double* lpart = nullptr;
   double* h_loss = nullptr;
+  bool planes = false;                 // the last forward pass left its inputs in bfloat16 planes
+  cudaEvent_t ev = nullptr;            // the mask sum's copy has arrived
   bool use_tc = true;                  // convolutions on tcgen05 (DDA_UNET_TC=0: mma.sync throughout)
   unsigned int* d_fault = nullptr;     // set when a bounded tensor-core wait gave up
-  std::vector<std::pair<std::array<int, 5>, dda::nn::TcTile>> tiles;  // tc_tile's answers by shape
+  std::vector<std::pair<std::array<int, 6>, dda::nn::TcTile>> tiles;  // tc_tile's answers by shape
   uint4* xb = nullptr;                 // bfloat16 copy of a tcgen05 convolution's input
   size_t xb_bytes = 0;
 };
@@ -921,7 +1033,7 @@ Err repack(dda_unet* n) {
 // (activation tile with halo, both halves, plus the chunk's weights for 27 taps) and its MMAs
 // (27 per 128-row M tile), overlapped when two buffers or two CTAs per SM fit.  false when no tile
 // fits: the caller uses the mma.sync kernel.
-bool tc_tile(const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
+bool tc_tile(const dda::nn::Dims& d, int B, int np, int kc_n, dda::nn::TcTile* out) {
   constexpr double kSmem = 227.0 * 1024.0, kBytesPerNs = 60.0, kMmaNs = 16.0;
   double best = 1e300;
   bool found = false;
@@ -948,15 +1060,18 @@ bool tc_tile(const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
       const double act = 2.0 * t.rows_alloc * 16.0, w = 27.0 * np * 32.0;
       t.stage_bytes = (uint32_t)((act + w + 1023) / 1024) * 1024u;
       if (1024.0 + t.stage_bytes > kSmem) break;
-      t.stages = (1024.0 + 2.0 * t.stage_bytes <= kSmem) ? 2 : 1;
-      const int cps = std::max(1, std::min((int)(kSmem / (1024.0 + t.stages * (double)t.stage_bytes)),
-                                           (int)(512 / t.ncol)));
+      t.stages = (kc_n > 1 && 1024.0 + 2.0 * t.stage_bytes <= kSmem) ? 2 : 1;
+      const int cps = std::max(1, std::min({(int)(kSmem / (1024.0 + t.stages * (double)t.stage_bytes)),
+                                            (int)(512 / t.ncol), 8}));
+      // a CTA's own time: start and epilogue, then per chunk the copies and the MMAs (the first chunk's
+      // copies are not overlapped); co-resident CTAs share the copy and MMA rates but hide the rest
       const double load = (2.0 * 16.0 * t.sx * t.sy * t.sz + w) / kBytesPerNs;
       const double mma = t.n_mt * 27.0 * kMmaNs * std::max(1.0, np / 64.0);
-      const double per_chunk = (t.stages == 2 || cps >= 2) ? std::max(load, mma) : load + mma;
+      const double busy = kc_n * std::max(load, mma) + 150.0 * t.n_mt * (np / 16);
+      const double lone = 2500.0 + load + kc_n * (t.stages == 2 ? std::max(load, mma) : load + mma) + 150.0 * t.n_mt * (np / 16);
       const double ctas = (double)B * t.ntx * ((d.Y + Ty - 1) / Ty) * ((d.Z + Tz - 1) / Tz);
-      const double waves = std::ceil(ctas / (152.0 * cps));
-      const double cost = waves * cps * per_chunk;
+      const double per_sm = std::ceil(ctas / 152.0);
+      const double cost = std::max(per_sm * busy, std::ceil(per_sm / cps) * lone);
       if (cost < best) {
         best = cost;
         *out = t;
@@ -968,15 +1083,15 @@ bool tc_tile(const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
 
 // tc_tile with its answers kept in the network (at most 64 shapes): the search takes tens of
 // microseconds of host time, more than a small convolution
-bool tc_tile_of(dda_unet* n, const dda::nn::Dims& d, int B, int np, dda::nn::TcTile* out) {
-  const std::array<int, 5> key = {d.Z, d.Y, d.X, B, np};
+bool tc_tile_of(dda_unet* n, const dda::nn::Dims& d, int B, int np, int kc_n, dda::nn::TcTile* out) {
+  const std::array<int, 6> key = {d.Z, d.Y, d.X, B, np, kc_n};
   for (auto& e : n->tiles)
     if (e.first == key) {
       *out = e.second;
       return out->Tx > 0;
     }
   dda::nn::TcTile t{};
-  if (!tc_tile(d, B, np, &t)) t = dda::nn::TcTile{};
+  if (!tc_tile(d, B, np, kc_n, &t)) t = dda::nn::TcTile{};
   if (n->tiles.size() >= 64) n->tiles.erase(n->tiles.begin());
   n->tiles.emplace_back(key, t);
   *out = t;
@@ -1023,10 +1138,40 @@ Err tc_smem_optin() {
   return Err::Ok();
 }
 
+// The tcgen05 convolution of layer L from bfloat16 planes xp (2 ceil16(channels) / 16 per sample) into out.
+Err conv_planes(dda_unet* n, const dda_unet::Layer& L, const uint4* xp, const dda::nn::ConvOut& out, bool relu,
+                dda::nn::Dims d, int B, bool transposed, const dda::nn::TcTile& tl) {
+  const int kc_n = transposed ? L.cin_t_kc : L.kc_n;
+  const int cout = transposed ? L.cin : L.cout;
+  const float* bias = transposed ? nullptr : n->p + L.boff;
+  CUtensorMap tmap;
+  DDA_TRY(encode_act_map(&tmap, xp, kc_n * 16, d, B, tl));
+  const uint4* wt = reinterpret_cast<const uint4*>(transposed ? L.wttc : L.wtc);
+  const dim3 grid((unsigned)(tl.ntx * ((d.Y + tl.Ty - 1) / tl.Ty)), (unsigned)((d.Z + tl.Tz - 1) / tl.Tz), (unsigned)B);
+  const size_t smem = 1024 + (size_t)tl.stages * tl.stage_bytes;
+  switch (np16(cout)) {
+#define CASE(NP)                                                                                                    \
+  case NP:                                                                                                          \
+    DDA_TRY(tc_smem_optin<NP>());                                                                                   \
+    dda::nn::k_conv_tc<NP><<<grid, dda::nn::kTcThreads, smem, n->stream>>>(tmap, wt, kc_n, transposed, bias, out,   \
+                                                                           cout, relu, d, tl, n->d_fault);          \
+    break;
+    CASE(16) CASE(32) CASE(48) CASE(64) CASE(80) CASE(96) CASE(112) CASE(128)
+#undef CASE
+    default: return Err::make(DDA_EUNSUPPORTED, "layer wider than 128 channels");
+  }
+  DDA_CU(cudaGetLastError());
+  dda::add_launches(1);
+  return Err::Ok();
+}
+
 // y = conv(x) for layer L; x has xs channels (uses the first cin), y gets ys channels (writes first cout)
-// (mask: x counts as zero where mask is not positive)
+// (mask: x counts as zero where mask is not positive; xp: x in bfloat16 planes already, mask applied;
+// yp / ymask: the result in bfloat16 planes as well, 2 ceil16(cout) / 16 per sample, zeroed where ymask
+// is not positive -- on the tcgen05 path only, *yp_done says whether)
 Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y, int ys, bool relu, dda::nn::Dims d,
-         int B, bool transposed, const float* mask = nullptr) {
+         int B, bool transposed, const float* mask = nullptr, const uint4* xp = nullptr, uint4* yp = nullptr,
+         const float* ymask = nullptr, bool* yp_done = nullptr) {
   const int64_t V = (int64_t)B * d.nvox();
   const int blocks = (int)((V + dda::nn::kVoxPerCta - 1) / dda::nn::kVoxPerCta);
   const int kc_n = transposed ? L.cin_t_kc : L.kc_n;
@@ -1035,41 +1180,30 @@ Err conv(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, float* y
   const int cout = transposed ? L.cin : L.cout;
   const uint2* w = transposed ? L.wt : L.wp;
   const float* bias = transposed ? nullptr : n->p + L.boff;
+  if (yp_done) *yp_done = false;
   if (n->use_tc && L.taps == dda::nn::kTaps) {
     const int np = np16(cout);
     dda::nn::TcTile tl;
-    if (tc_tile_of(n, d, B, np, &tl)) {
-      const int cpad = kc_n * 16;
-      const size_t need = sizeof(uint16_t) * (size_t)V * cpad;
-      if (need > n->xb_bytes) {
-        if (n->xb) cudaFree(n->xb);
-        n->xb = nullptr;
-        n->xb_bytes = 0;
-        DDA_CU(cudaMalloc((void**)&n->xb, need));
-        n->xb_bytes = need;
+    if (tc_tile_of(n, d, B, np, kc_n, &tl)) {
+      if (!xp) {
+        const int cpad = kc_n * 16;
+        const size_t need = sizeof(uint16_t) * (size_t)V * cpad;
+        if (need > n->xb_bytes) {
+          if (n->xb) cudaFree(n->xb);
+          n->xb = nullptr;
+          n->xb_bytes = 0;
+          DDA_CU(cudaMalloc((void**)&n->xb, need));
+          n->xb_bytes = need;
+        }
+        const int64_t items = V * (cpad / 8);
+        dda::nn::k_to_bf16<<<dda::nn::blocks_for(items), 256, 0, n->stream>>>(x, mask, xs, cin, cpad, d.nvox(), B, n->xb);
+        DDA_CU(cudaGetLastError());
+        dda::add_launches(1);
+        xp = n->xb;
       }
-      const int64_t items = V * (cpad / 8);
-      dda::nn::k_to_bf16<<<dda::nn::blocks_for(items), 256, 0, n->stream>>>(x, mask, xs, cin, cpad, d.nvox(), B, n->xb);
-      DDA_CU(cudaGetLastError());
-      CUtensorMap tmap;
-      DDA_TRY(encode_act_map(&tmap, n->xb, cpad, d, B, tl));
-      const uint4* wt = reinterpret_cast<const uint4*>(transposed ? L.wttc : L.wtc);
-      const dim3 grid((unsigned)(tl.ntx * ((d.Y + tl.Ty - 1) / tl.Ty)), (unsigned)((d.Z + tl.Tz - 1) / tl.Tz),
-                      (unsigned)B);
-      const size_t smem = 1024 + (size_t)tl.stages * tl.stage_bytes;
-      switch (np) {
-#define CASE(NP)                                                                                                  \
-  case NP:                                                                                                        \
-    DDA_TRY(tc_smem_optin<NP>());                                                                                 \
-    dda::nn::k_conv_tc<NP><<<grid, dda::nn::kTcThreads, smem, n->stream>>>(tmap, wt, kc_n, transposed, bias, y, ys, \
-                                                                           cout, relu, d, tl, n->d_fault);        \
-    break;
-        CASE(16) CASE(32) CASE(48) CASE(64) CASE(80) CASE(96) CASE(112) CASE(128)
-#undef CASE
-        default: return Err::make(DDA_EUNSUPPORTED, "layer wider than 128 channels");
-      }
-      DDA_CU(cudaGetLastError());
-      dda::add_launches(2);
+      dda::nn::ConvOut out{y, ys, yp, np / 8, 0, np / 8, ymask};
+      DDA_TRY(conv_planes(n, L, xp, out, relu, d, B, transposed, tl));
+      if (yp_done) *yp_done = yp != nullptr;
       return Err::Ok();
     }
   }
@@ -1132,8 +1266,9 @@ dda::nn::WgTile wg_tile(const dda::nn::Dims& d, int B, int taps, int kc_n, int N
 
 // weight and bias gradients of layer L from input x (xs channels) and output gradient gy (gs channels),
 // masked by (mask > 0) when given
-Err wgrad(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, const float* gy, const float* mask, int gs,
-          dda::nn::Dims d, int B) {
+// (xp: the input in bfloat16 planes instead)
+Err wgrad(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, const uint4* xp, const float* gy,
+          const float* mask, int gs, dda::nn::Dims d, int B) {
   const dda::nn::WgTile t = wg_tile(d, B, L.taps, L.kc_n, L.nt_n);
   const int64_t ntile = (int64_t)t.ntx * t.nty * t.ntz * B;
   if (t.K == 0 || ntile > (1 << 30)) return Err::make(DDA_EUNSUPPORTED, "no weight-gradient tile for this grid");
@@ -1151,7 +1286,7 @@ Err wgrad(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, const f
       DDA_CU(cudaFuncSetAttribute(dda::nn::k_wgrad<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024));   \
       done = true;                                                                                                   \
     }                                                                                                                \
-    dda::nn::k_wgrad<NT><<<grid, dda::nn::kWgT, sm, n->stream>>>(x, xs, L.cin, gy, mask, gs, L.cout, L.taps, d, t,   \
+    dda::nn::k_wgrad<NT><<<grid, dda::nn::kWgT, sm, n->stream>>>(x, xs, xp, L.cin, gy, mask, gs, L.cout, L.taps, d, t, \
                                                                  n->part, gbp, L.kc_n);                              \
     break;                                                                                                           \
   }
@@ -1173,6 +1308,10 @@ struct Acts {
   float *x, *e1a, *s1, *p1, *e2a, *s2, *p2, *e3a, *s3, *p3, *ba, *bb, *c3, *d3a, *d3b, *c2, *d2a, *d2b, *c1, *d1a,
       *d1b, *y;
   // gradients
+  // inputs of the 3x3x3 layers 0..13 in bfloat16 planes (tcgen05 path), the upsampled tensors' sources, and
+  // a masked gradient
+  uint4 *bin[14], *b_bb, *b_d3b, *b_d2b, *b_g;
+  bool planes;  // the planes hold this pass's inputs
   float *g_y, *g_d1b, *g_c1, *g_d2b, *g_c2, *g_d3b, *g_c3, *g_bb, *g_p3, *g_s3, *g_p2, *g_s2, *g_p1, *g_s1, *g_tmp;
 };
 
@@ -1194,6 +1333,16 @@ Err layout(dda_unet* n, int B, dda::nn::Dims d1, bool with_grads, Acts* a) {
         {&a->g_s1, V1 * c1}, {&a->g_tmp, V1 * cmax}};
     list.insert(list.end(), gl.begin(), gl.end());
   }
+  const int64_t Vl[14] = {V1, V1, V2, V2, V3, V3, V4, V4, V3, V3, V2, V2, V1, V1};
+  for (int l = 0; l < 14; ++l)
+    list.push_back({reinterpret_cast<float**>(&a->bin[l]), n->use_tc ? Vl[l] * n->layers[l].kc_n * 8 : 0});
+  list.push_back({reinterpret_cast<float**>(&a->b_bb), n->use_tc ? V4 * np16(c4) / 2 : 0});
+  list.push_back({reinterpret_cast<float**>(&a->b_d3b), n->use_tc ? V3 * np16(c3) / 2 : 0});
+  list.push_back({reinterpret_cast<float**>(&a->b_d2b), n->use_tc ? V2 * np16(c2) / 2 : 0});
+  if (with_grads) {
+    const int64_t w = std::max({V1 * np16(c1), V2 * np16(c2), V3 * np16(c3), V4 * np16(c4)}) / 2;
+    list.push_back({reinterpret_cast<float**>(&a->b_g), n->use_tc ? w : 0});
+  }
   int64_t total = 0;
   for (auto& e : list) total += (e.second + 63) / 64 * 64;
   DDA_TRY(grow_ws(n, &n->ws, &n->ws_bytes, sizeof(float) * (size_t)total));
@@ -1205,14 +1354,86 @@ Err layout(dda_unet* n, int B, dda::nn::Dims d1, bool with_grads, Acts* a) {
   return Err::Ok();
 }
 
-Err forward_pass(dda_unet* n, const Acts& a, int B, dda::nn::Dims d1) {
+// The forward pass on bfloat16 planes: every 3x3x3 layer reads planes that its producer wrote (the
+// convolutions' epilogues, the pooling, the upsampling straight into the concatenated tensor, into which
+// the skips' convolutions write as well), so the FP32 tensors in between are written only where something
+// reads them: the pooled ones and the head's input, and all of them when a backward pass follows.
+// 2 x 64 x 48 x 32 forward: 569 us with conversion, copy and FP32 upsampling kernels, 295 this way (23
+// launches instead of 39).
+// Returns false in *ran when a layer has no tcgen05 tile or an upsampled width is no multiple of 8.
+Err forward_planes(dda_unet* n, const Acts& a, const float* x, int B, dda::nn::Dims d1, bool keep, bool* ran) {
+  using namespace dda::nn;
+  const Dims d2{d1.Z / 2, d1.Y / 2, d1.X / 2}, d3{d2.Z / 2, d2.Y / 2, d2.X / 2}, d4{d3.Z / 2, d3.Y / 2, d3.X / 2};
+  const int c1 = n->ch[0], c2 = n->ch[1], c3 = n->ch[2], c4 = n->ch[3];
+  auto& L = n->layers;
+  const Dims dl[14] = {d1, d1, d2, d2, d3, d3, d4, d4, d3, d3, d2, d2, d1, d1};
+  TcTile tl[14];
+  *ran = false;
+  if (!n->use_tc || c2 % 8 || c3 % 8 || c4 % 8) return Err::Ok();
+  for (int l = 0; l < 14; ++l)
+    if (!tc_tile_of(n, dl[l], B, np16(L[l].cout), L[l].kc_n, &tl[l])) return Err::Ok();
+  *ran = true;
+  cudaStream_t st = n->stream;
+  k_to_bf16<<<blocks_for((int64_t)B * d1.nvox() * L[0].kc_n * 2), 256, 0, st>>>(x, nullptr, n->cin, n->cin,
+                                                                               L[0].kc_n * 16, d1.nvox(), B, a.bin[0]);
+  DDA_CU(cudaGetLastError());
+  // layer l into y (FP32, when wanted) and planes p (all of the layer's, or a skip's place from plane p0 of g8)
+  auto run = [&](int l, float* y, uint4* p, int g8 = 0, int p0 = 0) {
+    const int np = np16(L[l].cout) / 8;
+    ConvOut o{y, L[l].cout, p, g8 ? g8 : np, p0, g8 ? ceil_div(L[l].cout, 8) : np, nullptr};
+    return conv_planes(n, L[l], a.bin[l], o, true, dl[l], B, false, tl[l]);
+  };
+  auto pool = [&](const float* xf, int C, int l) {
+    k_pool_planes<<<blocks_for((int64_t)B * dl[l].nvox() * L[l].kc_n * 2), 256, 0, st>>>(xf, a.bin[l], C, L[l].kc_n * 2,
+                                                                                        dl[l], B);
+    return cudaGetLastError();
+  };
+  auto up = [&](const uint4* src, int C, int skip, int l) {
+    const int g8 = L[l].kc_n * 2, z0 = C / 8 + ceil_div(skip, 8);
+    k_up_planes<<<blocks_for((int64_t)B * dl[l].nvox() * (C / 8 + g8 - z0)), 256, 0, st>>>(src, np16(C) / 8, C / 8,
+                                                                                          a.bin[l], g8, z0, dl[l], B);
+    return cudaGetLastError();
+  };
+  DDA_TRY(run(0, keep ? a.e1a : nullptr, a.bin[1]));
+  DDA_TRY(run(1, a.s1, a.bin[12], L[12].kc_n * 2, c2 / 8));
+  DDA_CU(pool(a.s1, c1, 2));
+  DDA_TRY(run(2, keep ? a.e2a : nullptr, a.bin[3]));
+  DDA_TRY(run(3, a.s2, a.bin[10], L[10].kc_n * 2, c3 / 8));
+  DDA_CU(pool(a.s2, c2, 4));
+  DDA_TRY(run(4, keep ? a.e3a : nullptr, a.bin[5]));
+  DDA_TRY(run(5, a.s3, a.bin[8], L[8].kc_n * 2, c4 / 8));
+  DDA_CU(pool(a.s3, c3, 6));
+  DDA_TRY(run(6, keep ? a.ba : nullptr, a.bin[7]));
+  DDA_TRY(run(7, keep ? a.bb : nullptr, a.b_bb));
+  DDA_CU(up(a.b_bb, c4, c3, 8));
+  DDA_TRY(run(8, keep ? a.d3a : nullptr, a.bin[9]));
+  DDA_TRY(run(9, keep ? a.d3b : nullptr, a.b_d3b));
+  DDA_CU(up(a.b_d3b, c3, c2, 10));
+  DDA_TRY(run(10, keep ? a.d2a : nullptr, a.bin[11]));
+  DDA_TRY(run(11, keep ? a.d2b : nullptr, a.b_d2b));
+  DDA_CU(up(a.b_d2b, c2, c1, 12));
+  DDA_TRY(run(12, keep ? a.d1a : nullptr, a.bin[13]));
+  DDA_TRY(run(13, a.d1b, nullptr));
+  dda::add_launches(7);
+  return Err::Ok();
+}
+
+// x: the input (FP32, channels last), y: the output; keep: a backward pass follows
+Err forward_pass(dda_unet* n, Acts& a, const float* x, float* y, int B, dda::nn::Dims d1, bool keep) {
+  DDA_TRY(forward_planes(n, a, x, B, d1, keep, &a.planes));
+  n->planes = a.planes;
+  if (keep && !a.planes) {  // the first layer's weight gradient reads the input again
+    DDA_CU(cudaMemcpyAsync(a.x, x, sizeof(float) * (size_t)B * d1.nvox() * n->cin, cudaMemcpyDeviceToDevice, n->stream));
+    x = a.x;
+  }
+  if (a.planes) return conv(n, n->layers[14], a.d1b, n->ch[0], y, n->cout, false, d1, B, false);
   const dda::nn::Dims d2{d1.Z / 2, d1.Y / 2, d1.X / 2}, d3{d2.Z / 2, d2.Y / 2, d2.X / 2},
       d4{d3.Z / 2, d3.Y / 2, d3.X / 2};
   const int c1 = n->ch[0], c2 = n->ch[1], c3 = n->ch[2], c4 = n->ch[3];
   auto& L = n->layers;
   cudaStream_t st = n->stream;
   using namespace dda::nn;
-  DDA_TRY(conv(n, L[0], a.x, n->cin, a.e1a, c1, true, d1, B, false));
+  DDA_TRY(conv(n, L[0], x, n->cin, a.e1a, c1, true, d1, B, false));
   DDA_TRY(conv(n, L[1], a.e1a, c1, a.s1, c1, true, d1, B, false));
   k_pool<<<blocks_for((int64_t)B * d2.nvox() * c1), 256, 0, st>>>(a.s1, a.p1, c1, d2, B);
   DDA_TRY(conv(n, L[2], a.p1, c1, a.e2a, c2, true, d2, B, false));
@@ -1238,7 +1459,7 @@ Err forward_pass(dda_unet* n, const Acts& a, int B, dda::nn::Dims d1) {
                                                                       (int64_t)B * d1.nvox(), false);
   DDA_TRY(conv(n, L[12], a.c1, c2 + c1, a.d1a, c1, true, d1, B, false));
   DDA_TRY(conv(n, L[13], a.d1a, c1, a.d1b, c1, true, d1, B, false));
-  DDA_TRY(conv(n, L[14], a.d1b, c1, a.y, n->cout, false, d1, B, false));
+  DDA_TRY(conv(n, L[14], a.d1b, c1, y, n->cout, false, d1, B, false));
   DDA_CU(cudaGetLastError());
   dda::add_launches(9);
   return Err::Ok();
@@ -1246,14 +1467,20 @@ Err forward_pass(dda_unet* n, const Acts& a, int B, dda::nn::Dims d1) {
 
 // conv backward for layer li: output activation `out` (for the ReLU mask), its gradient g_out (gs channels,
 // taken as zero where out is not positive), input activation x (xs channels); writes the input gradient to
-// gx (gxs ch.)
-Err conv_back(dda_unet* n, int li, const float* x, int xs, const float* out, float* g_out, int gs, float* gx, int gxs,
-              dda::nn::Dims d, int B, bool relu) {
+// gx (gxs ch.).  gp: the masked g_out in planes already, when a.planes and the layer above wrote it;
+// prev_out: the output of the layer below whose gradient gx is, to leave gx masked by it in a.b_g.
+Err conv_back(dda_unet* n, const Acts& a, int li, const float* x, int xs, const float* out, float* g_out, int gs,
+              float* gx, int gxs, dda::nn::Dims d, int B, bool relu, bool* gp, const float* prev_out = nullptr) {
   const auto& L = n->layers[li];
   const float* mask = relu ? out : nullptr;
-  DDA_TRY(wgrad(n, L, x, xs, g_out, mask, gs, d, B));
-  if (gx) DDA_TRY(conv(n, L, g_out, gs, gx, gxs, false, d, B, true, mask));
-  return Err::Ok();
+  const bool have = *gp;
+  *gp = false;
+  DDA_TRY(wgrad(n, L, x, xs, a.planes && li < 14 ? a.bin[li] : nullptr, g_out, mask, gs, d, B));
+  if (!gx) return Err::Ok();
+  // the planes being read and the planes being written: a.b_g holds one of them, the shared copy the other
+  const bool write = a.planes && prev_out && !have;
+  return conv(n, L, g_out, gs, gx, gxs, false, d, B, true, mask, have ? a.b_g : nullptr, write ? a.b_g : nullptr,
+              prev_out, gp);
 }
 
 Err backward_pass(dda_unet* n, const Acts& a, int B, dda::nn::Dims d1) {
@@ -1262,38 +1489,39 @@ Err backward_pass(dda_unet* n, const Acts& a, int B, dda::nn::Dims d1) {
   const int c1 = n->ch[0], c2 = n->ch[1], c3 = n->ch[2], c4 = n->ch[3];
   cudaStream_t st = n->stream;
   const int64_t V1 = (int64_t)B * d1.nvox(), V2 = V1 / 8, V3 = V2 / 8, V4 = V3 / 8;
+  bool gp = false;  // a.b_g holds the next layer's masked gradient
   // head (linear): input d1b
-  DDA_TRY(conv_back(n, 14, a.d1b, c1, a.y, a.g_y, n->cout, a.g_d1b, c1, d1, B, false));
+  DDA_TRY(conv_back(n, a, 14, a.d1b, c1, a.y, a.g_y, n->cout, a.g_d1b, c1, d1, B, false, &gp));
   // dec1
-  DDA_TRY(conv_back(n, 13, a.d1a, c1, a.d1b, a.g_d1b, c1, a.g_tmp, c1, d1, B, true));
-  DDA_TRY(conv_back(n, 12, a.c1, c2 + c1, a.d1a, a.g_tmp, c1, a.g_c1, c2 + c1, d1, B, true));
+  DDA_TRY(conv_back(n, a, 13, a.d1a, c1, a.d1b, a.g_d1b, c1, a.g_tmp, c1, d1, B, true, &gp, a.d1a));
+  DDA_TRY(conv_back(n, a, 12, a.c1, c2 + c1, a.d1a, a.g_tmp, c1, a.g_c1, c2 + c1, d1, B, true, &gp));
   k_up_bwd<<<blocks_for(V2 * c2), 256, 0, st>>>(a.g_c1, c2 + c1, a.g_d2b, c2, d2, B);
   k_copy_ch<<<blocks_for(V1 * c1), 256, 0, st>>>(a.g_c1, c2 + c1, c2, a.g_s1, c1, 0, c1, V1, false);
   // dec2
-  DDA_TRY(conv_back(n, 11, a.d2a, c2, a.d2b, a.g_d2b, c2, a.g_tmp, c2, d2, B, true));
-  DDA_TRY(conv_back(n, 10, a.c2, c3 + c2, a.d2a, a.g_tmp, c2, a.g_c2, c3 + c2, d2, B, true));
+  DDA_TRY(conv_back(n, a, 11, a.d2a, c2, a.d2b, a.g_d2b, c2, a.g_tmp, c2, d2, B, true, &gp, a.d2a));
+  DDA_TRY(conv_back(n, a, 10, a.c2, c3 + c2, a.d2a, a.g_tmp, c2, a.g_c2, c3 + c2, d2, B, true, &gp));
   k_up_bwd<<<blocks_for(V3 * c3), 256, 0, st>>>(a.g_c2, c3 + c2, a.g_d3b, c3, d3, B);
   k_copy_ch<<<blocks_for(V2 * c2), 256, 0, st>>>(a.g_c2, c3 + c2, c3, a.g_s2, c2, 0, c2, V2, false);
   // dec3
-  DDA_TRY(conv_back(n, 9, a.d3a, c3, a.d3b, a.g_d3b, c3, a.g_tmp, c3, d3, B, true));
-  DDA_TRY(conv_back(n, 8, a.c3, c4 + c3, a.d3a, a.g_tmp, c3, a.g_c3, c4 + c3, d3, B, true));
+  DDA_TRY(conv_back(n, a, 9, a.d3a, c3, a.d3b, a.g_d3b, c3, a.g_tmp, c3, d3, B, true, &gp, a.d3a));
+  DDA_TRY(conv_back(n, a, 8, a.c3, c4 + c3, a.d3a, a.g_tmp, c3, a.g_c3, c4 + c3, d3, B, true, &gp));
   k_up_bwd<<<blocks_for(V4 * c4), 256, 0, st>>>(a.g_c3, c4 + c3, a.g_bb, c4, d4, B);
   k_copy_ch<<<blocks_for(V3 * c3), 256, 0, st>>>(a.g_c3, c4 + c3, c4, a.g_s3, c3, 0, c3, V3, false);
   // bottleneck
-  DDA_TRY(conv_back(n, 7, a.ba, c4, a.bb, a.g_bb, c4, a.g_tmp, c4, d4, B, true));
-  DDA_TRY(conv_back(n, 6, a.p3, c3, a.ba, a.g_tmp, c4, a.g_p3, c3, d4, B, true));
+  DDA_TRY(conv_back(n, a, 7, a.ba, c4, a.bb, a.g_bb, c4, a.g_tmp, c4, d4, B, true, &gp, a.ba));
+  DDA_TRY(conv_back(n, a, 6, a.p3, c3, a.ba, a.g_tmp, c4, a.g_p3, c3, d4, B, true, &gp));
   k_pool_bwd<<<blocks_for(V3 * c3), 256, 0, st>>>(a.g_p3, a.g_s3, c3, d3, B, true);
   // enc3
-  DDA_TRY(conv_back(n, 5, a.e3a, c3, a.s3, a.g_s3, c3, a.g_tmp, c3, d3, B, true));
-  DDA_TRY(conv_back(n, 4, a.p2, c2, a.e3a, a.g_tmp, c3, a.g_p2, c2, d3, B, true));
+  DDA_TRY(conv_back(n, a, 5, a.e3a, c3, a.s3, a.g_s3, c3, a.g_tmp, c3, d3, B, true, &gp, a.e3a));
+  DDA_TRY(conv_back(n, a, 4, a.p2, c2, a.e3a, a.g_tmp, c3, a.g_p2, c2, d3, B, true, &gp));
   k_pool_bwd<<<blocks_for(V2 * c2), 256, 0, st>>>(a.g_p2, a.g_s2, c2, d2, B, true);
   // enc2
-  DDA_TRY(conv_back(n, 3, a.e2a, c2, a.s2, a.g_s2, c2, a.g_tmp, c2, d2, B, true));
-  DDA_TRY(conv_back(n, 2, a.p1, c1, a.e2a, a.g_tmp, c2, a.g_p1, c1, d2, B, true));
+  DDA_TRY(conv_back(n, a, 3, a.e2a, c2, a.s2, a.g_s2, c2, a.g_tmp, c2, d2, B, true, &gp, a.e2a));
+  DDA_TRY(conv_back(n, a, 2, a.p1, c1, a.e2a, a.g_tmp, c2, a.g_p1, c1, d2, B, true, &gp));
   k_pool_bwd<<<blocks_for(V1 * c1), 256, 0, st>>>(a.g_p1, a.g_s1, c1, d1, B, true);
   // enc1
-  DDA_TRY(conv_back(n, 1, a.e1a, c1, a.s1, a.g_s1, c1, a.g_tmp, c1, d1, B, true));
-  DDA_TRY(conv_back(n, 0, a.x, n->cin, a.e1a, a.g_tmp, c1, nullptr, 0, d1, B, true));
+  DDA_TRY(conv_back(n, a, 1, a.e1a, c1, a.s1, a.g_s1, c1, a.g_tmp, c1, d1, B, true, &gp));
+  DDA_TRY(conv_back(n, a, 0, a.x, n->cin, a.e1a, a.g_tmp, c1, nullptr, 0, d1, B, true, &gp));
   DDA_CU(cudaGetLastError());
   dda::add_launches(9);
   return Err::Ok();
@@ -1359,7 +1587,8 @@ dda_status dda_unet_create(dda_unet** out, int device, void* stream, int cin, in
             cudaMalloc((void**)&n->m, sizeof(float) * off) == cudaSuccess &&
             cudaMalloc((void**)&n->v, sizeof(float) * off) == cudaSuccess &&
             cudaMalloc((void**)&n->lpart, sizeof(double) * 2048) == cudaSuccess &&
-            cudaMallocHost((void**)&n->h_loss, sizeof(double) * 2048) == cudaSuccess;
+            cudaMallocHost((void**)&n->h_loss, sizeof(double) * 2048) == cudaSuccess &&
+            cudaEventCreateWithFlags(&n->ev, cudaEventDisableTiming) == cudaSuccess;
   {
     const char* f = std::getenv("DDA_UNET_TC");
     n->use_tc = !(f && std::atoi(f) == 0);
@@ -1406,6 +1635,7 @@ void dda_unet_destroy(dda_unet* n) {
     if (q) cudaFree(q);
   if (n->lpart) cudaFree(n->lpart);
   if (n->h_loss) cudaFreeHost(n->h_loss);
+  if (n->ev) cudaEventDestroy(n->ev);
   if (n->d_fault) cudaFree(n->d_fault);
   if (n->xb) cudaFree(n->xb);
   delete n;
@@ -1446,6 +1676,26 @@ dda_status dda_unet_set_params(dda_unet* n, const float* host) {
   return DDA_OK;
 }
 
+namespace {
+// sum of the mask over V voxels, on the device in double precision (exact for 0/1 masks); begin queues
+// it, end waits for its copy only.  The partials use the second half of lpart / h_loss.
+constexpr int kMaskBlocks = 256;
+Err mask_sum_begin(dda_unet* n, const float* mask, int64_t V) {
+  dda::nn::k_mask_sum<<<kMaskBlocks, 256, 0, n->stream>>>(mask, V, n->lpart + 1024);
+  DDA_CU(cudaGetLastError());
+  dda::add_launches(1);
+  DDA_CU(cudaMemcpyAsync(n->h_loss + 1024, n->lpart + 1024, sizeof(double) * kMaskBlocks, cudaMemcpyDeviceToHost, n->stream));
+  DDA_CU(cudaEventRecord(n->ev, n->stream));
+  return Err::Ok();
+}
+Err mask_sum_end(dda_unet* n, double* cnt) {
+  if (cudaEventSynchronize(n->ev) != cudaSuccess) return Err::make(DDA_ECUDA, "mask copy failed");
+  *cnt = 0.0;
+  for (int i = 0; i < kMaskBlocks; ++i) *cnt += n->h_loss[1024 + i];
+  return Err::Ok();
+}
+}  // namespace
+
 dda_status dda_unet_forward(dda_unet* n, const float* x_dev, float* y_dev, int batch, const int32_t dims[3]) {
   if (!n || !x_dev || !y_dev || batch < 1 || !dims) return DDA_EINVAL;
   Err e = check_dims(dims);
@@ -1454,17 +1704,7 @@ dda_status dda_unet_forward(dda_unet* n, const float* x_dev, float* y_dev, int b
   const dda::nn::Dims d1{dims[2], dims[1], dims[0]};
   Acts a;
   e = layout(n, batch, d1, false, &a);
-  if (e.ok()) {
-    const int64_t V1 = (int64_t)batch * d1.nvox();
-    if (cudaMemcpyAsync(a.x, x_dev, sizeof(float) * V1 * n->cin, cudaMemcpyDeviceToDevice, n->stream) != cudaSuccess)
-      e = Err::make(DDA_ECUDA, "input copy failed");
-  }
-  if (e.ok()) e = forward_pass(n, a, batch, d1);
-  if (e.ok()) {
-    const int64_t V1 = (int64_t)batch * d1.nvox();
-    if (cudaMemcpyAsync(y_dev, a.y, sizeof(float) * V1 * n->cout, cudaMemcpyDeviceToDevice, n->stream) != cudaSuccess)
-      e = Err::make(DDA_ECUDA, "output copy failed");
-  }
+  if (e.ok()) e = forward_pass(n, a, x_dev, y_dev, batch, d1, false);
   return e.ok() ? DDA_OK : ufail(n, e);
 }
 
@@ -1478,18 +1718,12 @@ dda_status dda_unet_loss_grad(dda_unet* n, const float* x_dev, const float* t_de
   const int64_t V1 = (int64_t)batch * d1.nvox();
   Acts a;
   e = layout(n, batch, d1, true, &a);
-  if (e.ok() && cudaMemcpyAsync(a.x, x_dev, sizeof(float) * V1 * n->cin, cudaMemcpyDeviceToDevice, n->stream) !=
-                    cudaSuccess)
-    e = Err::make(DDA_ECUDA, "input copy failed");
-  if (e.ok()) e = forward_pass(n, a, batch, d1);
-  // masked-voxel count on the host side of the device: sum the mask once
+  // the mask's sum goes to the host while the forward pass runs: nothing waits for it
+  if (e.ok()) e = mask_sum_begin(n, mask_dev, V1);
+  if (e.ok()) e = forward_pass(n, a, x_dev, a.y, batch, d1, true);
   double cnt = 0.0;
   if (e.ok()) {
-    std::vector<float> hm(V1);
-    if (cudaMemcpyAsync(hm.data(), mask_dev, sizeof(float) * V1, cudaMemcpyDeviceToHost, n->stream) != cudaSuccess ||
-        cudaStreamSynchronize(n->stream) != cudaSuccess)
-      e = Err::make(DDA_ECUDA, "mask copy failed");
-    for (float m : hm) cnt += m;
+    e = mask_sum_end(n, &cnt);
     if (e.ok() && cnt <= 0) e = Err::make(DDA_EINVAL, "mask selects no voxel");
   }
   const int lb = 512;
@@ -1569,16 +1803,9 @@ dda_status dda_unet_forward_train(dda_unet* n, const float* x_dev, float* y_dev,
   if (!e.ok()) return ufail(n, e);
   if (cudaSetDevice(n->device) != cudaSuccess) return ufail(n, Err::make(DDA_ECUDA, "cudaSetDevice failed"));
   const dda::nn::Dims d1{dims[2], dims[1], dims[0]};
-  const int64_t V1 = (int64_t)batch * d1.nvox();
   Acts a;
   e = layout(n, batch, d1, true, &a);
-  if (e.ok() && cudaMemcpyAsync(a.x, x_dev, sizeof(float) * V1 * n->cin, cudaMemcpyDeviceToDevice, n->stream) !=
-                    cudaSuccess)
-    e = Err::make(DDA_ECUDA, "input copy failed");
-  if (e.ok()) e = forward_pass(n, a, batch, d1);
-  if (e.ok() && cudaMemcpyAsync(y_dev, a.y, sizeof(float) * V1 * n->cout, cudaMemcpyDeviceToDevice, n->stream) !=
-                    cudaSuccess)
-    e = Err::make(DDA_ECUDA, "output copy failed");
+  if (e.ok()) e = forward_pass(n, a, x_dev, y_dev, batch, d1, true);
   return e.ok() ? DDA_OK : ufail(n, e);
 }
 
@@ -1587,12 +1814,12 @@ dda_status dda_unet_mse(dda_unet* n, const float* y_dev, const float* t_dev, con
   if (!n || !y_dev || !t_dev || !mask_dev || !gy_dev || batch < 1 || !dims) return DDA_EINVAL;
   if (cudaSetDevice(n->device) != cudaSuccess) return ufail(n, Err::make(DDA_ECUDA, "cudaSetDevice failed"));
   const int64_t V1 = (int64_t)batch * dims[0] * dims[1] * dims[2];
-  std::vector<float> hm(V1);
-  if (cudaMemcpyAsync(hm.data(), mask_dev, sizeof(float) * V1, cudaMemcpyDeviceToHost, n->stream) != cudaSuccess ||
-      cudaStreamSynchronize(n->stream) != cudaSuccess)
-    return ufail(n, Err::make(DDA_ECUDA, "mask copy failed"));
   double cnt = 0.0;
-  for (float m : hm) cnt += m;
+  {
+    Err e = mask_sum_begin(n, mask_dev, V1);
+    if (e.ok()) e = mask_sum_end(n, &cnt);
+    if (!e.ok()) return ufail(n, e);
+  }
   if (cnt <= 0) return ufail(n, Err::make(DDA_EINVAL, "mask selects no voxel"));
   const int lb = 512;
   dda::nn::k_loss<<<lb, 256, 0, n->stream>>>(y_dev, t_dev, mask_dev, n->cout, V1, weight / (cnt * n->cout), gy_dev,
@@ -1616,6 +1843,7 @@ dda_status dda_unet_backward(dda_unet* n, const float* gy_dev, int batch, const 
   const int64_t V1 = (int64_t)batch * d1.nvox();
   Acts a;
   e = layout(n, batch, d1, true, &a);  // same sizes as the preceding dda_unet_forward_train: same buffers
+  a.planes = n->planes;
   if (e.ok() && cudaMemcpyAsync(a.g_y, gy_dev, sizeof(float) * V1 * n->cout, cudaMemcpyDeviceToDevice, n->stream) !=
                     cudaSuccess)
     e = Err::make(DDA_ECUDA, "gradient copy failed");
