@@ -14,31 +14,55 @@
 namespace dda {
 namespace kred {
 
-// a thread's running sum of float products carried as a double-float pair
-// (products split exactly with one FMA, added with the two-sum)
-struct AccF {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void fma(float a, float b) {
-    const float p = __fmul_rn(a, b);
-    const float pe = __fmaf_rn(a, b, -p);
-    const float t = __fadd_rn(hi, p);
-    const float z = __fsub_rn(t, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z));
+// Two running sums of float products side by side, each carried as a double-float pair (products split
+// exactly with one FMA, added with the two-sum), on the packed FP32 instructions: conj(a) b as (re, im),
+// or the two squares of |a|^2.
+struct AccF2 {
+  float2 hi = {0.f, 0.f}, lo = {0.f, 0.f};
+  __device__ __forceinline__ void fma(float2 a, float2 b) {
+    auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+    const float2 p = __fmul2_rn(a, b);
+    const float2 pe = __ffma2_rn(a, b, neg(p));
+    const float2 t = __fadd2_rn(hi, p);
+    const float2 z = __fadd2_rn(t, neg(hi));
+    const float2 e = __fadd2_rn(__fadd2_rn(hi, neg(__fadd2_rn(t, neg(z)))), __fadd2_rn(p, neg(z)));
     hi = t;
-    lo = __fadd_rn(lo, __fadd_rn(e, pe));
+    lo = __fadd2_rn(lo, __fadd2_rn(e, pe));
   }
-  __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
-// re + i im += conj(a) b
-__device__ __forceinline__ void acc_cdot(AccF& re, AccF& im, float2 a, float2 b) {
-  re.fma(a.x, b.x);
-  re.fma(a.y, b.y);
-  im.fma(a.x, b.y);
-  im.fma(-a.y, b.x);
+__device__ __forceinline__ void acc_cdot(AccF2& c, float2 a, float2 b) {
+  c.fma(make_float2(a.x, a.x), b);
+  c.fma(make_float2(a.y, a.y), make_float2(b.y, -b.x));
 }
-__device__ __forceinline__ void acc_nrm(AccF& s, float2 a) {
-  s.fma(a.x, a.x);
-  s.fma(a.y, a.y);
+__device__ __forceinline__ void acc_nrm(AccF2& s, float2 a) { s.fma(a, a); }
+
+// (h, l) += (h2, l2), sums carried as double-float pairs
+__device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2) {
+  const float s = __fadd_rn(h, h2), z = __fsub_rn(s, h);
+  l = __fadd_rn(__fadd_rn(l, l2), __fadd_rn(__fsub_rn(h, __fsub_rn(s, z)), __fsub_rn(h2, z)));
+  h = s;
+}
+
+// Block sum of NS pairs, blockDim.x = 256: the warps' sums stay in pairs (an FP64 shuffle tree of three
+// values costs a CTA of eight warps 1900 issue cycles at 1/64 of the FP32 rate, this one 300), then one
+// warp adds the eight warps' sums of all values in FP64; result in out (doubles, NS <= 4).
+template <int NS>
+__device__ __forceinline__ void block_sum_pairs(float (&h)[NS], float (&l)[NS], double* out) {
+  __shared__ double red[NS * 8];
+#pragma unroll
+  for (int s = 0; s < NS; ++s)
+    for (int o = 16; o > 0; o >>= 1)
+      pair_add(h[s], l[s], __shfl_down_sync(0xffffffffu, h[s], o), __shfl_down_sync(0xffffffffu, l[s], o));
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0)
+#pragma unroll
+    for (int s = 0; s < NS; ++s) red[s * 8 + w] = (double)h[s] + (double)l[s];
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double x = threadIdx.x < NS * 8 ? red[threadIdx.x] : 0.0;
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o, 8);
+    if (threadIdx.x % 8 == 0 && threadIdx.x < NS * 8) out[threadIdx.x / 8] = x;
+  }
 }
 
 // Block sum of v (all threads call; blockDim.x a multiple of 32, at most 1024); result in out (thread 0 writes).
@@ -63,14 +87,14 @@ __device__ __forceinline__ void block_sum(double (&v)[NS], double* out) {
   }
 }
 
-// Store this CTA's block sum of acc in slot `slot` of RHS b (nblk slots per RHS, kRedSlots
+// Store this CTA's block sum of the pairs (h, l) in slot `slot` of RHS b (nblk slots per RHS, kRedSlots
 // doubles each).  Returns true in every thread of the last CTA of b to arrive, with b's totals
 // in tot; that CTA also resets b's counter to zero.  All threads of the CTA must call it.
 template <int NS>
-__device__ __forceinline__ bool last_cta_totals(double (&acc)[NS], double* part, unsigned int* count, int b,
-                                                int slot, int nblk, double (&tot)[NS]) {
+__device__ __forceinline__ bool last_cta_totals(float (&h)[NS], float (&l)[NS], double* part, unsigned int* count,
+                                                int b, int slot, int nblk, double (&tot)[NS]) {
   double* mine = part + ((int64_t)b * nblk + slot) * kRedSlots;
-  block_sum<NS>(acc, mine);
+  block_sum_pairs<NS>(h, l, mine);
   __shared__ unsigned int s_last;
   if (threadIdx.x == 0) {
     __threadfence();

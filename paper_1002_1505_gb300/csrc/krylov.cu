@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "dda_internal.h"
+#include "kred.cuh"
 
 namespace dda {
 
@@ -301,12 +302,14 @@ __global__ void k_bicg_xr(KrylovVecs<C> kv, KState* ks, RedBuf rb, int64_t n3) {
   const int b = blockIdx.y;
   const KState k = ks[b];
   double acc[3] = {0.0, 0.0, 0.0};
+  float sh[3] = {0.f, 0.f, 0.f}, sl[3] = {0.f, 0.f, 0.f};
   if (k.done == 0 || k.done == 3) {
     using R = typename RealOf<C>::t;
     const C al = mk((R)k.alpha.x, (R)k.alpha.y), om = mk((R)k.omega.x, (R)k.omega.y);
     const bool half = (k.done == 3);
     const int64_t o = (int64_t)b * n3;
-    Acc<C> re, im, rr;
+    [[maybe_unused]] Acc<C> re, im, rr;
+    [[maybe_unused]] kred::AccF2 dot, nrm;
     VEC_LOOP(n3) {
       const C sv = kv.s[o + i];
       C xv = cadd(kv.x[o + i], cmul(al, kv.p[o + i]));
@@ -317,15 +320,31 @@ __global__ void k_bicg_xr(KrylovVecs<C> kv, KState* ks, RedBuf rb, int64_t n3) {
       }
       kv.x[o + i] = xv;
       kv.r[o + i] = rv;
-      acc_cdot(re, im, kv.rhat[o + i], rv);
-      acc_nrm(rr, rv);
+      if constexpr (std::is_same<C, float2>::value) {
+        kred::acc_cdot(dot, kv.rhat[o + i], rv);
+        kred::acc_nrm(nrm, rv);
+      } else {
+        acc_cdot(re, im, kv.rhat[o + i], rv);
+        acc_nrm(rr, rv);
+      }
     }
-    acc[0] = re.get();
-    acc[1] = im.get();
-    acc[2] = rr.get();
+    if constexpr (std::is_same<C, float2>::value) {
+      sh[0] = dot.hi.x; sh[1] = dot.hi.y; sh[2] = nrm.hi.x;
+      sl[0] = dot.lo.x; sl[1] = dot.lo.y; sl[2] = nrm.lo.x;
+      kred::pair_add(sh[2], sl[2], nrm.hi.y, nrm.lo.y);
+    } else {
+      acc[0] = re.get();
+      acc[1] = im.get();
+      acc[2] = rr.get();
+    }
   }
   double t[3];
-  if (last_block_totals<3>(acc, rb, b, t) && threadIdx.x == 0) {
+  bool last;
+  if constexpr (std::is_same<C, float2>::value)
+    last = kred::last_cta_totals<3>(sh, sl, rb.part, rb.count, b, blockIdx.x, rb.nblk, t);
+  else
+    last = last_block_totals<3>(acc, rb, b, t);
+  if (last && threadIdx.x == 0) {
     KState& k = ks[b];
     if (k.done == 3) { k.done = 1; k.it += 1; return; }
     if (k.done) return;

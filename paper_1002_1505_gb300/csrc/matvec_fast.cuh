@@ -180,7 +180,7 @@ __device__ __forceinline__ void x_fwd_body(const Geom& g, const MvData<C>& d, co
   if (rhs_done(d, b)) return;
   copy_tw(tw, d.twx, PX);
   [[maybe_unused]] C k1 = czero<C>(), k2 = czero<C>();  // (beta, omega) or (alpha, -)
-  [[maybe_unused]] kred::AccF ss;
+  [[maybe_unused]] kred::AccF2 ss;
   if constexpr (MODE == kFuseP) {
     const KState k = ksw[b];
     k1 = mk((float)k.beta.x, (float)k.beta.y);
@@ -206,6 +206,19 @@ __device__ __forceinline__ void x_fwd_body(const Geom& g, const MvData<C>& d, co
       w.next(g.nx);
     }
     C vals[kXU];
+    // the vectors' values first: the stores below would otherwise order every element's loads behind
+    // the previous element's store
+    [[maybe_unused]] C ra[MODE == kFuseNone ? 1 : kXU], va[MODE == kFuseNone ? 1 : kXU], pa[MODE == kFuseP ? kXU : 1];
+    if constexpr (MODE != kFuseNone) {
+#pragma unroll
+      for (int u = 0; u < kXU; ++u) {
+        const int64_t o = ((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u];
+        const bool in_target = idxs[u] >= 0;
+        ra[u] = in_target ? kf->r[o] : czero<C>();
+        va[u] = in_target ? kf->v[o] : czero<C>();
+        if constexpr (MODE == kFuseP) pa[u] = in_target ? kf->p[o] : czero<C>();
+      }
+    }
 #pragma unroll
     for (int u = 0; u < kXU; ++u) {
       const int cl = rs[u] / TY;
@@ -217,10 +230,10 @@ __device__ __forceinline__ void x_fwd_body(const Geom& g, const MvData<C>& d, co
           v = io_get<C>(p[o]);
           if (conj) v = conjc(v);
         } else if constexpr (MODE == kFuseP) {
-          v = cadd(kf->r[o], cmul(k1, csub(kf->p[o], cmul(k2, kf->v[o]))));
+          v = cadd(ra[u], cmul(k1, csub(pa[u], cmul(k2, va[u]))));
           kf->p[o] = v;
         } else {
-          v = csub(kf->r[o], cmul(k1, kf->v[o]));
+          v = csub(ra[u], cmul(k1, va[u]));
           kf->s[o] = v;
           kred::acc_nrm(ss, v);
         }
@@ -271,9 +284,10 @@ __device__ __forceinline__ void x_fwd_body(const Geom& g, const MvData<C>& d, co
     }
   }
   if constexpr (MODE == kFuseS) {
-    double acc[1] = {ss.get()};
+    float ah[1] = {ss.hi.x}, al[1] = {ss.lo.x};
+    kred::pair_add(ah[0], al[0], ss.hi.y, ss.lo.y);
     double tot[1];
-    if (kred::last_cta_totals<1>(acc, rbx->part, rbx->count, b, x_slot<NC>(), x_slots<NC>(), tot) &&
+    if (kred::last_cta_totals<1>(ah, al, rbx->part, rbx->count, b, x_slot<NC>(), x_slots<NC>(), tot) &&
         threadIdx.x == 0) {
       KState& k = ksw[b];
       if (!k.done && tot[0] <= k.tol2) { k.done = 3; k.rr = tot[0]; }  // converged on the half step
@@ -352,7 +366,7 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
   }
   __syncthreads();
   const C* ia = d.ia + (int64_t)(rhs0 + b) * g.ncomp * 3;
-  [[maybe_unused]] kred::AccF re, im, tt;
+  [[maybe_unused]] kred::AccF2 dot, tt;
   // kXU elements per thread per round, site indices first, then the input values (independent loads
   // in flight: 256 x 256 x 320, 32 RHS 1.81 -> 1.69 ms); as in the forward gather, 8 for x lengths of
   // 256 and more, 4 below
@@ -372,6 +386,12 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
 #pragma unroll
    for (int u = 0; u < kXU; ++u)
      pvs[u] = idxs[u] >= 0 ? p[((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u]] : typename Io<C>::t{};
+   [[maybe_unused]] float2 rvs[MODE == kFuseRV ? kXU : 1];
+   if constexpr (MODE == kFuseRV) {
+#pragma unroll
+     for (int u = 0; u < kXU; ++u)
+       rvs[u] = idxs[u] >= 0 ? kf->rhat[((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u]] : make_float2(0.f, 0.f);
+   }
 #pragma unroll
    for (int u = 0; u < kXU; ++u) {
     const int32_t idx = idxs[u];
@@ -401,17 +421,17 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
     }
     ap[o] = io_put<C>(conj ? conjc(res) : res);
     if constexpr (MODE == kFuseRV) {
-      kred::acc_cdot(re, im, kf->rhat[o], res);  // <rhat, v>
+      kred::acc_cdot(dot, rvs[u], res);  // <rhat, v>
     } else if constexpr (MODE == kFuseTS) {
-      kred::acc_cdot(re, im, res, kf->s[o]);     // <t, s>
-      kred::acc_nrm(tt, res);                    // |t|^2
+      kred::acc_cdot(dot, res, pv);      // <t, s>: the product's input is s
+      kred::acc_nrm(tt, res);            // |t|^2
     }
    }
   }
   if constexpr (MODE == kFuseRV) {
-    double acc[2] = {re.get(), im.get()};
+    float ah[2] = {dot.hi.x, dot.hi.y}, al[2] = {dot.lo.x, dot.lo.y};
     double tot[2];
-    if (kred::last_cta_totals<2>(acc, rbx->part, rbx->count, b, x_slot<NC>(), x_slots<NC>(), tot) &&
+    if (kred::last_cta_totals<2>(ah, al, rbx->part, rbx->count, b, x_slot<NC>(), x_slots<NC>(), tot) &&
         threadIdx.x == 0) {
       KState& k = ksw[b];
       if (!k.done) {
@@ -422,9 +442,10 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
       }
     }
   } else if constexpr (MODE == kFuseTS) {
-    double acc[3] = {re.get(), im.get(), tt.get()};
+    float ah[3] = {dot.hi.x, dot.hi.y, tt.hi.x}, al[3] = {dot.lo.x, dot.lo.y, tt.lo.x};
+    kred::pair_add(ah[2], al[2], tt.hi.y, tt.lo.y);
     double tot[3];
-    if (kred::last_cta_totals<3>(acc, rbx->part, rbx->count, b, x_slot<NC>(), x_slots<NC>(), tot) &&
+    if (kred::last_cta_totals<3>(ah, al, rbx->part, rbx->count, b, x_slot<NC>(), x_slots<NC>(), tot) &&
         threadIdx.x == 0) {
       KState& k = ksw[b];
       if (!k.done) {
