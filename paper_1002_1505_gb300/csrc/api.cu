@@ -654,6 +654,13 @@ Err ensure_einc(dda_ctx* c) {
   return Err::Ok();
 }
 
+// programmatic dependent launch of the compile-time kernels that this thread launches in a scope
+struct PdlScope {
+  bool prev;
+  explicit PdlScope(bool on) : prev(dda::pdl_enabled()) { dda::set_pdl(on); }
+  ~PdlScope() { dda::set_pdl(prev); }
+};
+
 struct SolveStats {
   std::vector<int> iters, done;
   std::vector<int> mv;  // products with A applied to each RHS
@@ -704,15 +711,13 @@ Err krylov(dda_ctx* c, const dda_solve_opts& o, const dda::KrylovVecs<C>& kv, do
   // capacity is known.
   bool fused = false;
   dda::RedBuf rbx{};
-  // Programmatic dependent launch inside the iteration chain (DDA_PDL=1): every kernel
-  // of an iteration may be scheduled behind its predecessor's tail (pdl.cuh).
+  // Programmatic dependent launch inside the iteration chain: every kernel of an iteration may be
+  // scheduled behind its predecessor's tail (pdl.cuh).  Taken while the vectors are short (iterations
+  // bound by launches and tails: 12^3 sphere, 2 RHS 412 -> 370 us a solve, 45 x 27 x 37 2132 -> 2076, 64 x
+  // 48 x 32 4414 -> 4354, 48^3 with 8 RHS 14.25 -> 14.14 ms); with 64 RHS of 48^3 (21 M elements) the
+  // early CTAs cost 1 %.  DDA_PDL=1 / 0 forces it on / off.
   const char* pdl_env = std::getenv("DDA_PDL");
-  const bool pdl = pdl_env && std::atoi(pdl_env) != 0;
-  struct PdlScope {
-    bool prev;
-    explicit PdlScope(bool on) : prev(dda::pdl_enabled()) { dda::set_pdl(on); }
-    ~PdlScope() { dda::set_pdl(prev); }
-  };
+  const bool pdl = pdl_env ? std::atoi(pdl_env) != 0 : (int64_t)nrhs * n3 <= (4 << 20);
   // one_iter: one BiCGstab / CCG iteration (2 products), or one BiCGstab(2) cycle (4 products)
   auto one_iter = [&]() -> Err {
     PdlScope scope(pdl);
@@ -1448,6 +1453,10 @@ dda_status dda_matvec(dda_ctx* c, const void* p, void* ap, int nrhs, int dtype) 
   if (p == ap) return fail(c, Err::make(DDA_EINVAL, "p and ap may not alias"));
   Err e = set_dev(c);
   if (!e.ok()) return fail(c, e);
+  // the passes of a product are scheduled behind their predecessors' tails: 24^3 grid, 2 RHS 14.35 -> 9.6
+  // us, 128 x 96 x 64 43.0 -> 37.0, 90 x 54 x 80 (five passes) 42.2 -> 32.7, 96^3 with 128 RHS 2204 -> 2196;
+  // with the twiddle copies ahead of the wait 7.9, 35.5, 31.2 and 2183
+  PdlScope pdl(true);
   if (dtype == DDA_C64) {
     e = ensure_tuned<float2>(c, nrhs);
     if (e.ok()) e = matvec<float2>(c, (const float2*)p, (float2*)ap, nrhs, 0, false);
@@ -2157,6 +2166,7 @@ Err matvec_fixed_scratch(dda_ctx* c, const C* p, C* ap, int nrhs) {
   // a bulk-staged plane pass reports a bounded wait that gave up through the context's fault
   // flag; without that flag (no earlier allocating call made it) run the plane pass unstaged
   if (!d.fault) t.bulk = false;
+  PdlScope pdl(true);  // as dda_matvec
   return dda::launch_matvec<C>(g, d, t, p, ap, nrhs, 0, false, c->stream);
 }
 }  // namespace

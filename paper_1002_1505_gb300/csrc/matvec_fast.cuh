@@ -170,15 +170,15 @@ __device__ __forceinline__ void x_fwd_body(const Geom& g, const MvData<C>& d, co
   constexpr int RA = Shape<PX>::RA, LB = Shape<PX>::LB, H = Shape<PX>::H;
   static_assert(NC == 1 || NC == 3, "one or three components per CTA");
   static_assert(MODE == kFuseNone || (MODE == kFuseP || MODE == kFuseS), "x forward fuses p or s updates");
-  pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* in = tw + PX;
   C* out = in + NC * TY * ip;
   const int y0 = blockIdx.x * TY, z = blockIdx.y;
   const int b = blockIdx.z / (3 / NC), c0 = (blockIdx.z % (3 / NC)) * NC;
-  if (rhs_done(d, b)) return;
   copy_tw(tw, d.twx, PX);
+  pdl_begin();
+  if (rhs_done(d, b)) return;
   [[maybe_unused]] C k1 = czero<C>(), k2 = czero<C>();  // (beta, omega) or (alpha, -)
   [[maybe_unused]] kred::AccF2 ss;
   if constexpr (MODE == kFuseP) {
@@ -317,15 +317,15 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
   constexpr int RA = Shape<PX>::RA, LB = Shape<PX>::LB, H = Shape<PX>::H;
   static_assert(NC == 1 || NC == 3, "one or three components per CTA");
   static_assert(MODE == kFuseNone || (MODE == kFuseRV || MODE == kFuseTS), "x inverse fuses the dot products");
-  pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* in = tw + PX;
   C* out = in + NC * TY * ip;
   const int y0 = blockIdx.x * TY, z = blockIdx.y;
   const int b = blockIdx.z / (3 / NC), c0 = (blockIdx.z % (3 / NC)) * NC;
-  if (rhs_done(d, b)) return;
   copy_tw(tw, d.twx, PX);
+  pdl_begin();
+  if (rhs_done(d, b)) return;
   __syncthreads();
   const int64_t plane = (int64_t)g.nz * g.ys;
   for (int i = threadIdx.x; i < NC * 2 * RA * TY; i += blockDim.x) {
@@ -490,11 +490,13 @@ __global__ void __launch_bounds__(NT) k_yz_plane(Geom g, MvData<C> d) {
   constexpr int RAy = Shape<PY>::RA, LBy = Shape<PY>::LB, Hy = Shape<PY>::H;
   constexpr int RAz = Shape<PZ>::RA, LBz = Shape<PZ>::LB, Hz = Shape<PZ>::H;
   constexpr int RP = PY + 1;
-  pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* twy = reinterpret_cast<C*>(smem_raw);
   C* twz = twy + PY;
   C* pl = twz + PZ;
+  copy_tw(twy, d.twy, PY);
+  copy_tw(twz, d.twz, PZ);
+  pdl_begin();
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + ((plane_bytes<C>(PY, PZ) + 15) & ~(size_t)15));
   const int b = blockIdx.x, kx = blockIdx.y;
   if (rhs_done(d, b)) return;
@@ -510,8 +512,6 @@ __global__ void __launch_bounds__(NT) k_yz_plane(Geom g, MvData<C> d) {
     bulk::mbar_arrive_expect_tx(bar, 3 * cbytes);
     for (int c = 0; c < 3; ++c) bulk::load_g2s(stage + c * nz * ny, wb + c * cstride, cbytes, bar);
   }
-  copy_tw(twy, d.twy, PY);
-  copy_tw(twz, d.twz, PZ);
   __syncthreads();  // barrier initialised before anyone polls it
   if (staged) bulk::mbar_wait(bar, 0, bulk::kMaxPolls, d.fault);
   // y forward, pass A: staged block (or global) -> registers -> plane
@@ -681,18 +681,18 @@ __global__ void __launch_bounds__(NT, (half_min_ctas(PY, PZ))) k_yz_half(Geom g,
   using SZ = Shape<PZ>;
   constexpr int RAy = SY::RA, LBy = SY::LB, PH = PY / 2, RP = half_pitch<PY>();
   constexpr int RAz = SZ::RA, LBz = SZ::LB, Hz = SZ::H;
-  pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* twy = reinterpret_cast<C*>(smem_raw);
   C* twz = twy + PY;
   C* pl = twz + PZ;
   const int b = blockIdx.x, kx = blockIdx.y;
+  copy_tw(twy, d.twy, PY);
+  copy_tw(twz, d.twz, PZ);
+  pdl_begin();
   if (rhs_done(d, b)) return;
   const int nz = g.nz, ny = g.ny;
   C* wb = d.work + ((int64_t)b * 3 * g.px + kx) * ((int64_t)nz * g.ys);
   const int64_t cstride = (int64_t)g.px * nz * g.ys;
-  copy_tw(twy, d.twy, PY);
-  copy_tw(twz, d.twz, PZ);
   __syncthreads();
   const int nrow = 3 * nz;
   // y pass A of half 0: rows (z, c) from the workspace
@@ -837,14 +837,14 @@ __global__ void __launch_bounds__(256) k_y_rows(Geom g, C* __restrict__ work, co
                                                 int64_t nrows) {
   constexpr int RA = Shape<PY>::RA, LB = Shape<PY>::LB, H = Shape<PY>::H;
   constexpr int RP = PY + 1;
-  pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* s = tw + PY;
+  copy_tw(tw, twg, PY);
+  pdl_begin();
   const int64_t r0 = (int64_t)blockIdx.x * RPB;
   const int nr = (int)min((int64_t)RPB, nrows - r0);
   const int ny = g.ny;
-  copy_tw(tw, twg, PY);
   __syncthreads();
   if (!INV) {
     for (int i = threadIdx.x; i < nr * LB; i += blockDim.x) {
@@ -983,14 +983,14 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, NT, NA>())) k_z_col
   constexpr int RA = SZ::RA, LB = SZ::LB, H = SZ::H;
   constexpr int P = zcols_pad<C, PZ, G, NA>();  // spare elements after each sub-block
   constexpr bool kFuse = LB * sizeof(C) <= 96;
-  pdl_begin();
   extern __shared__ unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* s = tw + PZ;
   const int ky0 = blockIdx.y * G, kx = blockIdx.z, b = blockIdx.x;
+  copy_tw(tw, d.twz, PZ);
+  pdl_begin();
   if (rhs_done(d, b)) return;
   const int nz = g.nz, py = g.py;
-  copy_tw(tw, d.twz, PZ);
   __syncthreads();
   C* wb = d.work + ((int64_t)b * 3 * g.px + kx) * ((int64_t)nz * g.ys);
   const int64_t cstride = (int64_t)g.px * nz * g.ys;

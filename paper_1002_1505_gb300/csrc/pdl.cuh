@@ -8,9 +8,10 @@
 // launch latency and CTA rasterisation overlap the predecessor's tail instead
 // of following it.
 //
-// Rule kept by every kernel launched through launch_k: pdl_begin() is its first
-// statement, before any global-memory access (griddepcontrol.wait is a no-op for
-// a kernel launched without the attribute).  Because the signal is given only
+// Rule kept by every kernel launched through launch_k: pdl_begin() comes before
+// any global-memory access except reads of the twiddle tables, which are written
+// by synchronous copies when the grid is set up (griddepcontrol.wait is a no-op
+// for a kernel launched without the attribute).  Because the signal is given only
 // after the wait, a grid can be scheduled early only behind a predecessor whose
 // CTAs are all resident, and never before the grid two steps back has finished.
 #pragma once
