@@ -44,7 +44,7 @@ struct dda_ctx {
   double* d_origin = nullptr;
   int tw_len[3] = {0, 0, 0};          // padded lengths the twiddle tables were built for
   int32_t* d_gperm = nullptr;         // storage <-> natural frequency tables of the Green build
-  int gperm_key[2] = {0, 0};          // (px, py) they were built for
+  int gperm_key[3] = {0, 0, 0};       // (px, py, pz) they were built for
 
   // incident
   bool have_inc = false;
@@ -1271,15 +1271,15 @@ dda_status dda_build_green_fft(dda_ctx* c, const int32_t pad[3]) {
     const bool want_df = c->t128.fast && !c->t128.plane && dda::df_lengths(c->g128);
     if (e.ok() && want_df) e = grow(c, &c->d_ghatdf, sizeof(dda::dfp::dfc) * 6 * M);
     if (!e.ok()) return fail(c, e);
-    // frequency-order tables of the Green build (kept while px, py stay the same)
-    if (e.ok() && (c->gperm_key[0] != g.px || c->gperm_key[1] != g.py || !c->d_gperm)) {
+    // frequency-order tables of the Green build (kept while the lengths stay the same)
+    if (e.ok() && (c->gperm_key[0] != g.px || c->gperm_key[1] != g.py || c->gperm_key[2] != g.pz || !c->d_gperm)) {
       std::vector<int32_t> tab;
       dda::green_perm_tables(g64, &tab);
       e = grow(c, &c->d_gperm, sizeof(int32_t) * tab.size());
       if (e.ok() && cudaMemcpy(c->d_gperm, tab.data(), sizeof(int32_t) * tab.size(), cudaMemcpyHostToDevice) !=
                         cudaSuccess)
         e = Err::make(DDA_ECUDA, "Green-table upload failed");
-      if (e.ok()) { c->gperm_key[0] = g.px; c->gperm_key[1] = g.py; }
+      if (e.ok()) { c->gperm_key[0] = g.px; c->gperm_key[1] = g.py; c->gperm_key[2] = g.pz; }
     }
     if (!e.ok()) return fail(c, e);
     if (c->periodic) {

@@ -211,7 +211,7 @@ constexpr size_t kNoAllocScratchBytes = 32ull << 20;
 Err noalloc_scratch(int device, void** out);
 
 // Green tensor: fill + FP64 FFT + pack into ghat128 / ghat64 / ghatdf (double-float, may be null).
-// storage <-> natural frequency tables the Green build needs (natx[px] | naty[py] | stx[px/2+1] | sty[py/2+1])
+// storage <-> natural frequency tables the Green build needs: stx[px] | sty[py] | stz[pz] | naty[py]
 void green_perm_tables(const Geom& g, std::vector<int32_t>* out);
 Err build_green(const Geom& g, double kd, const double2* twx, const double2* twy, const double2* twz,
                 const int32_t* perm, double2* gw, double2* ghat128, float2* ghat64, dfp::dfc* ghatdf,

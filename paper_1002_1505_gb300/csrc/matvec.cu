@@ -320,33 +320,39 @@ __global__ void k_fft_strided(C* data, int64_t estride, int64_t ninner, int64_t 
 // The interaction tensor of a lattice offset n, component c (xx, xy, xz, yy, yz, zz), is even
 // or odd in each of n_x, n_y, n_z: xy is odd in x and y, xz in x and z, yz in y and z, the
 // diagonal components even in all three.  Its zero-padded DFT inherits the same parity per
-// axis, so the FP64 build fills and transforms only what the parities do not determine:
-// the x transforms run on the rows with y <= Py/2, z <= Pz/2, the y transforms on the
-// planes z <= Pz/2 for natural kx <= Px/2, the z transforms on natural kx <= Px/2,
-// ky <= Py/2, and the missing parts are mirrored in between and in the final pack (1/4 of
-// the FFT work and of the fill of a plain 3-D transform).
+// axis, so the FP64 build (bound by the FP64 pipe) uses the parities twice.  It fills and transforms
+// only what they do not determine: offsets n_x >= 0 are evaluated, the x transforms run on the rows
+// with y <= Py/2, z <= Pz/2, the y transforms on the planes z <= Pz/2 for natural kx <= Px/2, the z
+// transforms on natural kx <= Px/2, ky <= Py/2, and the missing parts are mirrored in between and in
+// the final pack.  And along each axis an even and an odd component go through one transform: of the
+// sum s = a + b, A(k) = (S(k) + S(-k))/2 and B(k) = (S(k) - S(-k))/2, so six components take four
+// transforms per axis:
+//   x: S1 = xx + xy, S2 = yy + xz, S3 = yz, S4 = zz
+//   y: T1 = xx + xy, T2 = yy + yz, T3 = xz, T4 = zz
+//   z: F1 = xx + xz, F2 = yy + yz, F3 = xy, F4 = zz
+// Measured on 128 x 96 x 64 (one component per transform before, each value converted at each use):
+// fill 54 -> 30 us, transforms 227 -> 165, expansions 18 -> 17, pack 105 -> 47.
+
 __device__ __forceinline__ bool odd_in(int c, int axis) {
   // bit a of the mask = odd in axis a (0 = x, 1 = y, 2 = z)
   const int mask[6] = {0, 3, 5, 0, 6, 0};
   return (mask[c] >> axis) & 1;
 }
 
-// q[c][zq][yq][x] for zq <= Pz/2, yq <= Py/2 and all x (offsets wrapped along x)
+// q[j][zq][yq][x], j = S1 .. S4, for zq <= Pz/2, yq <= Py/2 and all x (offsets wrapped along x): a thread
+// evaluates one offset n_x >= 0 and writes it and its mirror image
 __global__ void k_green_fill_q(Geom g, double kd, double2* q) {
-  const int hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
-  const int64_t Q = (int64_t)g.px * hy1 * hz1;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < Q; i += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % g.px);
-    const int64_t rest = i / g.px;
+  const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
+  const int64_t Q = (int64_t)g.px * hy1 * hz1, N = (int64_t)hx1 * hy1 * hz1;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    const int x = (int)(i % hx1);
+    const int64_t rest = i / hx1;
     const int y = (int)(rest % hy1), z = (int)(rest / hy1);
-    int ox = 0;
-    bool ok = y < g.ny && z < g.nz;
-    if (x < g.nx) ox = x; else if (x > g.px - g.nx) ox = x - g.px; else ok = false;
-    if (ox == 0 && y == 0 && z == 0) ok = false;
+    const bool ok = x < g.nx && y < g.ny && z < g.nz && (x | y | z) != 0;
     double2 out[6];
     for (int c = 0; c < 6; ++c) out[c] = make_double2(0.0, 0.0);
     if (ok) {
-      const double rx = ox, ry = y, rz = z;
+      const double rx = x, ry = y, rz = z;
       const double r2 = rx * rx + ry * ry + rz * rz;
       const double r = sqrt(r2);
       const double inv_r = 1.0 / r;
@@ -366,51 +372,66 @@ __global__ void k_green_fill_q(Geom g, double kd, double2* q) {
         out[c] = make_double2(pref.x * inner.x - pref.y * inner.y, pref.x * inner.y + pref.y * inner.x);
       }
     }
-    for (int c = 0; c < 6; ++c) q[(int64_t)c * Q + i] = out[c];
+    double2* row = q + rest * g.px;
+    row[x] = cadd(out[0], out[1]);
+    row[Q + x] = cadd(out[3], out[2]);
+    row[2 * Q + x] = out[4];
+    row[3 * Q + x] = out[5];
+    const int xm = x ? g.px - x : 0;
+    if (xm != x) {
+      row[xm] = csub(out[0], out[1]);
+      row[Q + xm] = csub(out[3], out[2]);
+      row[2 * Q + xm] = out[4];
+      row[3 * Q + xm] = out[5];
+    }
   }
 }
 
-// After the x transform only the natural frequencies kx <= Px/2 are carried on (the others
-// follow by the x parity); the spectra are in the engine's digit-reversed storage order, so
-// the host passes the storage position stx[k] of natural frequency k and, for the final
-// pack, the natural frequency natx[s] of storage position s (likewise for y).
-// t[c][zq][y][k] (all y, k <= Px/2) from q[c][zq][yq][stx[k]]: rows y > Py/2 mirror Py - y
+__device__ __forceinline__ double2 half_sum(double2 a, double2 b) { return make_double2(0.5 * (a.x + b.x), 0.5 * (a.y + b.y)); }
+__device__ __forceinline__ double2 half_diff(double2 a, double2 b) { return make_double2(0.5 * (a.x - b.x), 0.5 * (a.y - b.y)); }
+
+// After the x transform only the natural frequencies kx <= Px/2 are carried on; the spectra are in the
+// engine's digit-reversed storage order, st*[k] = storage position of natural frequency k.
+// t[j][zq][y][k], j = T1 .. T4 (all y, k <= Px/2), from q[j][zq][yq][storage]: rows y > Py/2 mirror Py - y
 __global__ void k_green_expand_y(Geom g, const int32_t* __restrict__ stx, const double2* __restrict__ q,
                                  double2* __restrict__ t) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
   const int64_t Q = (int64_t)g.px * hy1 * hz1, T = (int64_t)hx1 * g.py * hz1;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < 6 * T; o += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(o / T);
-    const int64_t i = o - c * T;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < T; i += (int64_t)gridDim.x * blockDim.x) {
     const int k = (int)(i % hx1);
     const int64_t rest = i / hx1;
     const int y = (int)(rest % g.py), z = (int)(rest / g.py);
     const bool mir = y > g.py / 2;
-    const int ys = mir ? g.py - y : y;
-    double2 v = q[(int64_t)c * Q + ((int64_t)z * hy1 + ys) * g.px + stx[k]];
-    if (mir && odd_in(c, 1)) v = make_double2(-v.x, -v.y);
-    t[o] = v;
+    const double2* row = q + ((int64_t)z * hy1 + (mir ? g.py - y : y)) * g.px;
+    const int p = stx[k], m = stx[k ? g.px - k : 0];
+    const double2 s2 = row[Q + p], s2m = row[Q + m], yz = row[2 * Q + p];
+    const double2 yy = half_sum(s2, s2m);
+    t[i] = row[mir ? m : p];  // xx + xy, or xx - xy
+    t[T + i] = mir ? csub(yy, yz) : cadd(yy, yz);
+    t[2 * T + i] = half_diff(s2, s2m);
+    t[3 * T + i] = row[3 * Q + p];
   }
 }
 
-// f[c][z][kx][ky] (all z; natural kx <= Px/2, ky <= Py/2) from t[c][zq][sty[ky]][kx]:
-// planes z > Pz/2 mirror Pz - z with the z parity.  ky runs fastest because the pack below reads
-// every element four times with consecutive ky (in storage order) per warp.
+// f[j][z][kx][ky], j = F1 .. F4 (all z; natural kx <= Px/2, ky <= Py/2), from t[j][zq][storage][kx]: planes
+// z > Pz/2 mirror Pz - z.  ky runs fastest, for the pack below.
 __global__ void k_green_expand_z(Geom g, const int32_t* __restrict__ sty, const double2* __restrict__ t,
                                  double2* __restrict__ f) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
   const int64_t T = (int64_t)hx1 * g.py * hz1, P = (int64_t)hx1 * hy1, F = P * g.pz;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < 6 * F; o += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(o / F);
-    const int64_t i = o - c * F;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < F; i += (int64_t)gridDim.x * blockDim.x) {
     const int z = (int)(i / P);
     const int64_t r = i - (int64_t)z * P;
     const int kx = (int)(r / hy1), ky = (int)(r - (int64_t)kx * hy1);
     const bool mir = z > g.pz / 2;
-    const int zs = mir ? g.pz - z : z;
-    double2 v = t[(int64_t)c * T + ((int64_t)zs * g.py + sty[ky]) * hx1 + kx];
-    if (mir && odd_in(c, 2)) v = make_double2(-v.x, -v.y);
-    f[o] = v;
+    const double2* pl = t + (int64_t)(mir ? g.pz - z : z) * g.py * hx1 + kx;
+    const int64_t p = (int64_t)sty[ky] * hx1, m = (int64_t)sty[ky ? g.py - ky : 0] * hx1;
+    const double2 t1 = pl[p], t1m = pl[m], xz = pl[2 * T + p];
+    const double2 xx = half_sum(t1, t1m);
+    f[i] = mir ? csub(xx, xz) : cadd(xx, xz);
+    f[F + i] = pl[T + (mir ? m : p)];  // yy + yz, or yy - yz
+    f[2 * F + i] = half_diff(t1, t1m);
+    f[3 * F + i] = pl[3 * T + p];
   }
 }
 
@@ -432,31 +453,71 @@ __device__ __forceinline__ void ghat_put(const double2 (&w)[6], int kx, int kz, 
   }
 }
 
-// Ghat (storage positions) = f[c][kz][kx'][ky'] / M, with kx', ky' the natural frequencies folded
-// into [0, P/2] and the sign of the parities of the folds.  One thread per spectral point, ky
-// fastest; grid (ceil(py / blockDim), pz, px).  Bound by the three tensors it writes (240 bytes a
-// point).
-__global__ void k_green_pack(Geom g, const int32_t* __restrict__ natx, const int32_t* __restrict__ naty,
-                             const double2* __restrict__ f, double2* __restrict__ g128, float2* __restrict__ g64,
-                             dfp::dfc* __restrict__ gdf) {
-  const int ky = blockIdx.x * blockDim.x + threadIdx.x, kz = blockIdx.y, kx = blockIdx.z;
-  if (ky >= g.py) return;
-  const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1;
+// xx .. zz at natural kx <= Px/2, ky <= Py/2 and storage positions (kzs, kzm) of (kz, -kz), times inv
+__device__ __forceinline__ void green_parts(const double2* __restrict__ f, int64_t F, int64_t P, int64_t at, int kzs,
+                                            int kzm, double inv, double2 (&w)[6]) {
+  const double2 a = f[kzs * P + at], am = f[kzm * P + at], b = f[F + kzs * P + at], bm = f[F + kzm * P + at];
+  w[0] = half_sum(a, am);
+  w[1] = f[2 * F + kzs * P + at];
+  w[2] = half_diff(a, am);
+  w[3] = half_sum(b, bm);
+  w[4] = half_diff(b, bm);
+  w[5] = f[3 * F + kzs * P + at];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) w[c] = make_double2(w[c].x * inv, w[c].y * inv);
+}
+
+// Ghat (storage positions) from f.  A CTA takes one natural (kx <= Px/2, kz <= Pz/2): it forms and converts
+// every value of the ky row once, in shared memory (the conversions to float pairs are FP64 instructions:
+// converted at every use they were three quarters of the pack), and writes the rows of +-kx, +-kz with the
+// signs of the parities, ky in storage order.  Bound by the tensors it writes (240 bytes a point).
+// grid (Pz/2 + 1, Px/2 + 1); smem: hy1 x 6 double2, then float4 (x.hi, x.lo, y.hi, y.lo)
+__global__ void __launch_bounds__(128) k_green_pack(Geom g, const int32_t* __restrict__ naty,
+                                                    const int32_t* __restrict__ stx, const int32_t* __restrict__ stz,
+                                                    const double2* __restrict__ f, double2* __restrict__ g128,
+                                                    float2* __restrict__ g64, dfp::dfc* __restrict__ gdf) {
+  extern __shared__ double2 sg[];
+  const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, py = g.py;
+  float4* sf = reinterpret_cast<float4*>(sg + 6 * hy1);
+  const int kz = blockIdx.x, kx = blockIdx.y;
+  const int kzm = kz ? g.pz - kz : 0, kxm = kx ? g.px - kx : 0;
   const int64_t P = (int64_t)hx1 * hy1, F = P * g.pz;
   const double inv = 1.0 / ((double)g.px * g.py * g.pz);
-  int nx = natx[kx], ny = naty[ky];
-  const bool fx = nx > g.px / 2, fy = ny > g.py / 2;
-  if (fx) nx = g.px - nx;
-  if (fy) ny = g.py - ny;
-  const double2* src = f + (int64_t)kz * P + (int64_t)nx * hy1 + ny;
-  double2 w[6];
+  for (int ky = threadIdx.x; ky < hy1; ky += blockDim.x) {
+    double2 w[6];
+    green_parts(f, F, P, (int64_t)kx * hy1 + ky, stz[kz], stz[kzm], inv, w);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const double2 v = src[(int64_t)c * F];
-    const double sc = (fx && odd_in(c, 0)) != (fy && odd_in(c, 1)) ? -inv : inv;
-    w[c] = make_double2(v.x * sc, v.y * sc);
+    for (int c = 0; c < 6; ++c) {
+      sg[c * hy1 + ky] = w[c];
+      const dfp::dfc v = dfp::from_c128(w[c]);
+      sf[c * hy1 + ky] = make_float4(v.x.hi, v.x.lo, v.y.hi, v.y.lo);
+    }
   }
-  ghat_put(w, kx, kz, ky, g.pz, g.py, g128, g64, gdf);
+  __syncthreads();
+  for (int v = 0; v < 4; ++v) {
+    const bool mx = v & 1, mz = v & 2;
+    if ((mx && kxm == kx) || (mz && kzm == kz)) continue;
+    const int sx = stx[mx ? kxm : kx], sz = stz[mz ? kzm : kz];
+    const int64_t a16 = ghat_at<double2>(sx, sz, 0, g.pz, py), a8 = ghat_at<float2>(sx, sz, 0, g.pz, py);
+    for (int k = threadIdx.x; k < py; k += blockDim.x) {
+      const int n = naty[k];
+      const bool fy = n > py / 2;
+      const int at = fy ? py - n : n;
+      float4 h[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const bool neg = ((mx && odd_in(c, 0)) != (fy && odd_in(c, 1))) != (mz && odd_in(c, 2));
+        const double2 w = sg[c * hy1 + at];
+        h[c] = sf[c * hy1 + at];
+        if (neg) h[c] = make_float4(-h[c].x, -h[c].y, -h[c].z, -h[c].w);
+        g128[a16 + (int64_t)c * py + k] = neg ? make_double2(-w.x, -w.y) : w;
+        if (gdf) *reinterpret_cast<float4*>(gdf + a16 + (int64_t)c * py + k) = h[c];
+      }
+      float4* q = reinterpret_cast<float4*>(g64) + a8 + k;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) q[(int64_t)c * py] = make_float4(h[2 * c].x, h[2 * c].z, h[2 * c + 1].x, h[2 * c + 1].z);
+    }
+  }
 }
 
 // natural frequency of storage position p of an in-place DIF transform with this plan:
@@ -645,6 +706,7 @@ void init_kernel_attrs() {
   optin(k_zconv<float2>); optin(k_zconv<double2>);
   optin(k_fft_rows<float2>); optin(k_fft_rows<double2>);
   optin(k_fft_strided<float2>); optin(k_fft_strided<double2>);
+  optin(k_green_pack);
   fast_optin_c64(v);
   cluster_optin_c64(v);
   plane_bulk_optin_c64(v);
@@ -654,19 +716,18 @@ void init_kernel_attrs() {
 }
 
 void green_perm_tables(const Geom& g, std::vector<int32_t>* out) {
-  const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1;
-  out->assign((size_t)g.px + g.py + hx1 + hy1, 0);
-  int32_t* natx = out->data();
-  int32_t* naty = natx + g.px;
-  int32_t* stx = naty + g.py;
-  int32_t* sty = stx + hx1;
-  for (int p = 0; p < g.px; ++p) {
-    natx[p] = natural_index(g.plx, p);
-    if (natx[p] <= g.px / 2) stx[natx[p]] = p;
-  }
-  for (int p = 0; p < g.py; ++p) {
-    naty[p] = natural_index(g.ply, p);
-    if (naty[p] <= g.py / 2) sty[naty[p]] = p;
+  const FftPlan* pl[3] = {&g.plx, &g.ply, &g.plz};
+  const int len[3] = {g.px, g.py, g.pz};
+  const size_t all = (size_t)g.px + g.py + g.pz;
+  out->assign(all + g.py, 0);
+  int32_t* st = out->data();
+  for (int a = 0; a < 3; ++a) {
+    for (int p = 0; p < len[a]; ++p) {
+      const int n = natural_index(*pl[a], p);
+      st[n] = p;
+      if (a == 1) (*out)[all + p] = n;
+    }
+    st += len[a];
   }
 }
 
@@ -674,38 +735,32 @@ Err build_green(const Geom& g, double kd, const double2* twx, const double2* twy
                 const int32_t* perm, double2* gw, double2* ghat128, float2* ghat64, dfp::dfc* ghatdf,
                 cudaStream_t st) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
-  const int64_t Q = (int64_t)g.px * hy1 * hz1, T = (int64_t)hx1 * g.py * hz1, F = (int64_t)hx1 * hy1 * g.pz;
+  const int64_t T = (int64_t)hx1 * g.py * hz1, F = (int64_t)hx1 * hy1 * g.pz;
   auto nblk = [](int64_t n) { return (int)std::min<int64_t>((n + 255) / 256, 152 * 16); };
   Err e = Err::Ok();
-  // perm (green_perm_tables): natx[px] | naty[py] | stx[hx1] | sty[hy1]
-  const int32_t* d_natx = perm;
-  const int32_t* d_naty = d_natx + g.px;
-  const int32_t* d_stx = d_naty + g.py;
-  const int32_t* d_sty = d_stx + hx1;
+  const int32_t *stx = perm, *sty = stx + g.px, *stz = sty + g.py, *naty = stz + g.pz;  // green_perm_tables
   // q (in gw): the quarter y <= Py/2, z <= Pz/2 of the wrapped tensor; x rows transformed in place
   double2* q = gw;
-  if (e.ok()) {
-    k_green_fill_q<<<nblk(Q), 256, 0, st>>>(g, kd, q);
-    if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green fill failed");
-  }
-  if (e.ok()) e = fft_rows<double2>(q, 6 * (int64_t)hy1 * hz1, g.px, g.plx, twx, g.px, g.px, false, st);
+  k_green_fill_q<<<nblk((int64_t)hx1 * hy1 * hz1), 256, 0, st>>>(g, kd, q);
+  if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green fill failed");
+  if (e.ok()) e = fft_rows<double2>(q, 4 * (int64_t)hy1 * hz1, g.px, g.plx, twx, g.px, g.px, false, st);
   // t (in the ghat128 buffer, free until the pack): planes z <= Pz/2, all y, natural kx <= Px/2
   double2* t = ghat128;
   if (e.ok()) {
-    k_green_expand_y<<<nblk(6 * T), 256, 0, st>>>(g, d_stx, q, t);
+    k_green_expand_y<<<nblk(T), 256, 0, st>>>(g, stx, q, t);
     if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green expand (y) failed");
   }
-  if (e.ok()) e = fft_strided<double2>(t, g.py, hx1, hx1, 6 * (int64_t)hz1, (int64_t)hx1 * g.py, g.ply, twy, false, st);
+  if (e.ok()) e = fft_strided<double2>(t, g.py, hx1, hx1, 4 * (int64_t)hz1, (int64_t)hx1 * g.py, g.ply, twy, false, st);
   // f (in gw): all z, natural ky <= Py/2, kx <= Px/2; z columns transformed
   if (e.ok()) {
-    k_green_expand_z<<<nblk(6 * F), 256, 0, st>>>(g, d_sty, t, gw);
+    k_green_expand_z<<<nblk(F), 256, 0, st>>>(g, sty, t, gw);
     if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green expand (z) failed");
   }
   if (e.ok())
-    e = fft_strided<double2>(gw, g.pz, (int64_t)hx1 * hy1, (int64_t)hx1 * hy1, 6, F, g.plz, twz, false, st);
+    e = fft_strided<double2>(gw, g.pz, (int64_t)hx1 * hy1, (int64_t)hx1 * hy1, 4, F, g.plz, twz, false, st);
   if (e.ok()) {
-    k_green_pack<<<dim3((g.py + 127) / 128, g.pz, g.px), std::min(128, (g.py + 31) / 32 * 32), 0, st>>>(
-        g, d_natx, d_naty, gw, ghat128, ghat64, ghatdf);
+    const size_t sm = (size_t)hy1 * 6 * (sizeof(double2) + sizeof(float4));  // < the y transforms' 272 py bytes
+    k_green_pack<<<dim3(hz1, hx1), 128, sm, st>>>(g, naty, stx, stz, gw, ghat128, ghat64, ghatdf);
     if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green pack failed");
   }
   g_launches += 4;
