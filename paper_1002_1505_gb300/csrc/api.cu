@@ -506,6 +506,13 @@ Err apply_tune(dda_ctx* c, const dda::MvTune& t) {
   return Err::Ok();
 }
 
+// programmatic dependent launch of the compile-time kernels that this thread launches in a scope
+struct PdlScope {
+  bool prev;
+  explicit PdlScope(bool on) : prev(dda::pdl_enabled()) { dda::set_pdl(on); }
+  ~PdlScope() { dda::set_pdl(prev); }
+};
+
 template <typename C>
 Err ensure_tuned(dda_ctx* c, int nrhs) {
   const int idx = (sizeof(C) == sizeof(float2)) ? 0 : 1;
@@ -560,6 +567,7 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
   cand.push_back(t5);
   dda::MvTune best = cand[0];
   {
+    PdlScope pdl(true);  // as the products are launched, whoever calls first
     const size_t bytes = sizeof(C) * (size_t)nrhs * 3 * c->n;
     DDA_TRY(grow(c, (char**)&c->d_tunebuf, 2 * bytes));
     C* p = (C*)c->d_tunebuf;
@@ -602,23 +610,24 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
           }
     }
     // then the x passes' tile height for the chosen schedule (short tiles give small batches more CTAs)
+    // and one component per CTA (smaller tiles in shared memory, longer rows per store); short products
+    // again in three rounds (64 x 48 x 32, 2 RHS: the shapes take 34.6 to 40 us, and one round picked
+    // the 39 us one in some runs)
     if (err.ok()) {
-      const dda::MvTune chosen = best;
+      std::vector<dda::MvTune> shapes;
       for (int ty : {4, 8}) {
         if (!dda::x_tile_height_ok(sizeof(C), g0.px, ty) || ty == dda::x_tile_height_default(sizeof(C), g0.px))
           continue;
-        dda::MvTune t = chosen;
-        t.xty = ty;
-        time_one(t);
-        if (!err.ok()) break;
+        shapes.push_back(best);
+        shapes.back().xty = ty;
       }
-    }
-    // one component per x-pass CTA (smaller tiles in shared memory, longer rows per store)
-    if (err.ok()) {
-      dda::MvTune t = best;
-      t.xnc = 1;
-      t.xty = 0;
-      time_one(t);
+      shapes.push_back(best);
+      shapes.back().xnc = 1;
+      shapes.back().xty = 0;
+      const bool brief = best_ms < 0.2f;
+      if (brief) shapes.push_back(best);
+      for (int round = 0; round < (brief ? 3 : 1); ++round)
+        for (size_t i = 0; i < shapes.size() && err.ok(); ++i) time_one(shapes[i], brief ? 5 : 3);
     }
     // the 5-pass z columns with their middle stages fused in registers (long pass-B sub-blocks)
     if (err.ok() && sizeof(C) == sizeof(float2) && !best.plane && dda::zcols_rfuse_available_c64(g0)) {
@@ -653,13 +662,6 @@ Err ensure_einc(dda_ctx* c) {
   c->einc_valid = true;
   return Err::Ok();
 }
-
-// programmatic dependent launch of the compile-time kernels that this thread launches in a scope
-struct PdlScope {
-  bool prev;
-  explicit PdlScope(bool on) : prev(dda::pdl_enabled()) { dda::set_pdl(on); }
-  ~PdlScope() { dda::set_pdl(prev); }
-};
 
 struct SolveStats {
   std::vector<int> iters, done;
@@ -776,7 +778,7 @@ Err krylov(dda_ctx* c, const dda_solve_opts& o, const dda::KrylovVecs<C>& kv, do
       fused = !(fe && std::atoi(fe) == 0) && !ccg && !b2 && !cocg && !qmr && c->t64.fast && cap >= nrhs;
       if (fused) {
         // the folded reductions' table follows the vector kernels' table in the same buffer
-        const int nx = dda::x_ctas_per_rhs_c64(Sel<float2>::geom(c), c->t64);
+        const int nx = dda::x_ctas_per_rhs_c64(Sel<float2>::geom(c), c->t64, nrhs);
         DDA_TRY(ensure_part(c, sizeof(double) * ((size_t)rb.nblk + nx) * nrhs * dda::kRedSlots));
         rb.part = c->d_part;
         rbx.part = c->d_part + (size_t)rb.nblk * nrhs * dda::kRedSlots;
@@ -1243,13 +1245,14 @@ dda_status dda_build_green_fft(dda_ctx* c, const int32_t pad[3]) {
       if (std::atoi(f) == 1) {
         if (t64.fast) t64.xnc = 1;
         if (t128.fast) t128.xnc = 1;
+        t64.xpin = true;
       }
       c->forced_schedule = true;
     }
     // DDA_XTILE pins the x passes' tile height (y rows per CTA: 4, 8 or 16 where instantiated)
     if (const char* f = std::getenv("DDA_XTILE")) {
       const int ty = std::atoi(f);
-      if (t64.fast && dda::x_tile_height_ok(sizeof(float2), g.px, ty)) t64.xty = ty;
+      if (t64.fast && dda::x_tile_height_ok(sizeof(float2), g.px, ty)) t64.xty = ty, t64.xpin = true;
       if (t128.fast && dda::x_tile_height_ok(sizeof(double2), g.px, ty)) t128.xty = ty;
       c->forced_schedule = true;
     }

@@ -132,6 +132,7 @@ struct MvTune {
   int clus = 0;           // plane pass split over a cluster of this many CTAs (0: one CTA per plane)
   int xty = 0;            // y rows per CTA of the compile-time x passes (0: the length's default)
   int xnc = 0;            // components per CTA of the x passes (0 or 3: all three; 1: one)
+  bool xpin = false;      // xty and xnc were asked for: the folded solver passes keep to them too
   bool bulk = false;      // plane pass stages its HBM blocks with bulk copies
   int half = 0;           // plane pass half by half with this many threads (0: whole planes)
   int zr = 0;             // 5-pass z columns with pass B, Ghat and inverse pass B fused in registers
@@ -331,7 +332,7 @@ template <typename C> Err ccg_beta_update(const KrylovVecs<C>& kv, KState* ks, R
 // reduction table of x_ctas_per_rhs_c64 slots per RHS and zeroed per-RHS counters.
 Err launch_bicg_half_c64(const Geom& g, const MvData<float2>& d, const MvTune& t, const KrylovVecs<float2>& kv,
                          KState* ks, const RedBuf& rbx, int nrhs, int half, cudaStream_t st);
-int x_ctas_per_rhs_c64(const Geom& g, const MvTune& t);
+int x_ctas_per_rhs_c64(const Geom& g, const MvTune& t, int nrhs);
 // its x passes for the other lengths; mode: 1 p update, 2 s update (forward), 3 <rhat, v>, 4 <t, s> (inverse)
 Err more_x_fused(int mode, const Geom& g, const MvData<float2>& d, const MvTune& t, const KrylovVecs<float2>& kv,
                  KState* ks, const RedBuf& rbx, int nrhs, cudaStream_t st);

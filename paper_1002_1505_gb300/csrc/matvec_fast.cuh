@@ -132,20 +132,30 @@ __device__ __forceinline__ int x_slots() {
   return (int)(gridDim.x * gridDim.y * (3 / NC));
 }
 
-// The gather and the scatter walk the tile's (component, y) rows with 8, 16 or 32 lanes to a row (the
-// width that leaves the fewest lanes idle at this nx, the wider one on a tie) and step along x, so a
-// position costs no division; with a flat index decoded by nx the integer divisions were most of the
+// The gather and the scatter walk the tile's y rows with a group of lanes to a row and step along x, so
+// a position costs no division; with a flat index decoded by nx the integer divisions were most of the
 // instructions of an x pass (256 x 256 x 320, 32 RHS: forward 2.13 -> 1.38 ms, inverse 1.96 -> 1.81;
-// 96^3, 128 RHS: 0.38 -> 0.26 and 0.41 -> 0.36).
+// 96^3, 128 RHS: 0.38 -> 0.26 and 0.41 -> 0.36).  A group has 8, 16 or 32 lanes, whichever leaves
+// the fewest idle at this nx (the wider one on a tie), but no fewer than give all threads a row.  A
+// position stands for the NC components of its site: they share the map entry and the address.
+template <int ROWS>
 struct RowWalk {
+  static constexpr int min_lg() {
+    int l = 3;
+    while ((256 >> l) > ROWS) ++l;
+    return l;
+  }
   int lg, x, r;          // log2 of the lanes per row; current position
   int x0, step, rstep;
   __device__ __forceinline__ explicit RowWalk(int nx) {
-    const int w32 = (nx + 31) & ~31, w16 = (nx + 15) & ~15, w8 = (nx + 7) & ~7;
-    int best = w32;
-    lg = 5;
-    if (w16 < best) { best = w16; lg = 4; }
-    if (w8 * 8 <= best * 7) lg = 3;
+    constexpr int kMin = min_lg();
+    lg = kMin > 5 ? kMin : 5;
+    if constexpr (kMin <= 4) {
+      const int w32 = (nx + 31) & ~31, w16 = (nx + 15) & ~15, w8 = (nx + 7) & ~7;
+      int best = w32;
+      if (w16 < best) { best = w16; lg = 4; }
+      if (kMin <= 3 && w8 * 8 <= best * 7) lg = 3;
+    }
     step = 1 << lg;
     x0 = x = threadIdx.x & (step - 1);
     r = threadIdx.x >> lg;
@@ -159,6 +169,17 @@ struct RowWalk {
     }
   }
 };
+
+// Sites per thread and round of the gather and the scatter: their map entries are loaded first and their
+// values next, so a thread has NC x (vectors read) x x_sites independent loads in flight.  Three components:
+// 4 sites of one 8-byte vector (96^3, 128 RHS forward / inverse: 2 sites 0.207 / 0.292 ms, 4 0.184 / 0.288,
+// 6 0.211 / 0.303; with a map entry read for every component 0.258 / 0.333), 2 where the registers hold
+// the vectors of a folded solver update (solve of 48^3, 64 RHS: 1 site 88.7 ms, 2 86.9, 4 90.5) or
+// 16-byte values.  One component: 8 for x lengths of 256 and more, 4 below.
+template <int PX, int NC, bool FUSED, int BYTES>
+constexpr int x_sites() {
+  return NC == 1 ? (PX >= 256 ? 8 : 4) : (FUSED || BYTES > 8 ? 2 : 4);
+}
 
 // ------------------------------------------------------------------ x forward
 // grid (ceil(ny/TY), nz, nrhs * 3/NC): NC components (1 or 3) of TY y rows per CTA.
@@ -189,64 +210,69 @@ __device__ __forceinline__ void x_fwd_body(const Geom& g, const MvData<C>& d, co
     const KState k = ksw[b];
     k1 = mk((float)k.alpha.x, (float)k.alpha.y);
   }
-  // gather: kXU elements per thread per round, their site indices (map) loaded first and their
-  // values next, so that a thread has kXU independent loads in flight at each of the two steps;
-  // 8 for x lengths of 256 and more (measured 4 % faster on a 256 x 256 x 320 grid), 4 below
-  // (8 was slower on 128 x 96 x 64)
-  constexpr int kXU = PX >= 256 ? 8 : 4;
-  for (RowWalk w(g.nx); w.r < NC * TY;) {
+  const int64_t vec = ((int64_t)b * 3 + c0) * g.n;  // component c of a site: vec + c n + idx
+  // one composition: the Jacobi scale of an axis is the same for every site
+  [[maybe_unused]] C sc0[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) sc0[c] = (d.sc && !d.comp) ? d.sc[((int64_t)b * g.ncomp) * 3 + c0 + c] : czero<C>();
+  constexpr int kXU = x_sites<PX, NC, MODE != kFuseNone, sizeof(typename Io<C>::t)>();
+  for (RowWalk<TY> w(g.nx); w.r < TY;) {
     int32_t idxs[kXU];
     int rs[kXU], xs[kXU];
 #pragma unroll
     for (int u = 0; u < kXU; ++u) {
       rs[u] = w.r;
       xs[u] = w.x;
-      const int y = y0 + w.r % TY;
-      idxs[u] = (w.r < NC * TY && w.x < g.nx && y < g.ny) ? __ldg(d.map + ((int64_t)z * g.ny + y) * g.nx + w.x) : -1;
+      const int y = y0 + w.r;
+      idxs[u] = (w.r < TY && w.x < g.nx && y < g.ny) ? __ldg(d.map + ((int64_t)z * g.ny + y) * g.nx + w.x) : -1;
       w.next(g.nx);
     }
-    C vals[kXU];
-    // the vectors' values first: the stores below would otherwise order every element's loads behind
+    // every vector's values first: the stores below would otherwise order every element's loads behind
     // the previous element's store
-    [[maybe_unused]] C ra[MODE == kFuseNone ? 1 : kXU], va[MODE == kFuseNone ? 1 : kXU], pa[MODE == kFuseP ? kXU : 1];
-    if constexpr (MODE != kFuseNone) {
+    typename Io<C>::t pv[MODE == kFuseNone ? kXU : 1][NC];
+    [[maybe_unused]] C ra[MODE == kFuseNone ? 1 : kXU][NC], va[MODE == kFuseNone ? 1 : kXU][NC],
+        pa[MODE == kFuseP ? kXU : 1][NC];
 #pragma unroll
-      for (int u = 0; u < kXU; ++u) {
-        const int64_t o = ((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u];
+    for (int u = 0; u < kXU; ++u) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const int64_t o = vec + (int64_t)c * g.n + idxs[u];
         const bool in_target = idxs[u] >= 0;
-        ra[u] = in_target ? kf->r[o] : czero<C>();
-        va[u] = in_target ? kf->v[o] : czero<C>();
-        if constexpr (MODE == kFuseP) pa[u] = in_target ? kf->p[o] : czero<C>();
+        if constexpr (MODE == kFuseNone) {
+          pv[u][c] = in_target ? p[o] : typename Io<C>::t{};
+        } else {
+          ra[u][c] = in_target ? kf->r[o] : czero<C>();
+          va[u][c] = in_target ? kf->v[o] : czero<C>();
+          if constexpr (MODE == kFuseP) pa[u][c] = in_target ? kf->p[o] : czero<C>();
+        }
       }
     }
 #pragma unroll
     for (int u = 0; u < kXU; ++u) {
-      const int cl = rs[u] / TY;
+      if (rs[u] >= TY || xs[u] >= g.nx) continue;
       const int32_t idx = idxs[u];
-      C v = czero<C>();
-      if (idx >= 0) {
-        const int64_t o = ((int64_t)b * 3 + c0 + cl) * g.n + idx;
-        if constexpr (MODE == kFuseNone) {
-          v = io_get<C>(p[o]);
-          if (conj) v = conjc(v);
-        } else if constexpr (MODE == kFuseP) {
-          v = cadd(ra[u], cmul(k1, csub(pa[u], cmul(k2, va[u]))));
-          kf->p[o] = v;
-        } else {
-          v = csub(ra[u], cmul(k1, va[u]));
-          kf->s[o] = v;
-          kred::acc_nrm(ss, v);
-        }
-        if (d.sc) {  // Jacobi scaling: transform s * v
-          const int c = c0 + cl;
-          v = cmul(v, d.sc[((int64_t)b * g.ncomp + (d.comp ? d.comp[3 * idx + c] : 0)) * 3 + c]);
-        }
-      }
-      vals[u] = v;
-    }
 #pragma unroll
-    for (int u = 0; u < kXU; ++u)
-      if (rs[u] < NC * TY && xs[u] < g.nx) in[rs[u] * ip + xs[u]] = vals[u];
+      for (int c = 0; c < NC; ++c) {
+        C v = czero<C>();
+        if (idx >= 0) {
+          const int64_t o = vec + (int64_t)c * g.n + idx;
+          if constexpr (MODE == kFuseNone) {
+            v = io_get<C>(pv[u][c]);
+            if (conj) v = conjc(v);
+          } else if constexpr (MODE == kFuseP) {
+            v = cadd(ra[u][c], cmul(k1, csub(pa[u][c], cmul(k2, va[u][c]))));
+            kf->p[o] = v;
+          } else {
+            v = csub(ra[u][c], cmul(k1, va[u][c]));
+            kf->s[o] = v;
+            kred::acc_nrm(ss, v);
+          }
+          if (d.sc)  // Jacobi scaling: transform s * v
+            v = cmul(v, d.comp ? d.sc[((int64_t)b * g.ncomp + d.comp[3 * idx + c0 + c]) * 3 + c0 + c] : sc0[c]);
+        }
+        in[(c * TY + rs[u]) * ip + xs[u]] = v;
+      }
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < NC * TY * LB; i += blockDim.x) {
@@ -367,66 +393,71 @@ __device__ __forceinline__ void x_inv_body(const Geom& g, const MvData<C>& d, co
   __syncthreads();
   const C* ia = d.ia + (int64_t)(rhs0 + b) * g.ncomp * 3;
   [[maybe_unused]] kred::AccF2 dot, tt;
-  // kXU elements per thread per round, site indices first, then the input values (independent loads
-  // in flight: 256 x 256 x 320, 32 RHS 1.81 -> 1.69 ms); as in the forward gather, 8 for x lengths of
-  // 256 and more, 4 below
-  constexpr int kXU = PX >= 256 ? 8 : 4;
-  for (RowWalk w(g.nx); w.r < NC * TY;) {
-   int32_t idxs[kXU];
-   int rs[kXU], xs[kXU];
-   typename Io<C>::t pvs[kXU];
+  const int64_t vec = ((int64_t)b * 3 + c0) * g.n;  // component c of a site: vec + c n + idx
+  // one composition: alpha^{-1} (or the Jacobi scale) of an axis is the same for every site
+  C tab0[NC];
 #pragma unroll
-   for (int u = 0; u < kXU; ++u) {
-     rs[u] = w.r;
-     xs[u] = w.x;
-     const int y = y0 + w.r % TY;
-     idxs[u] = (w.r < NC * TY && w.x < g.nx && y < g.ny) ? __ldg(d.map + ((int64_t)z * g.ny + y) * g.nx + w.x) : -1;
-     w.next(g.nx);
-   }
+  for (int c = 0; c < NC; ++c)
+    tab0[c] = (d.comp || d.iat) ? czero<C>() : (d.sc ? d.sc[((int64_t)b * g.ncomp) * 3 + c0 + c] : ia[c0 + c]);
+  constexpr int kXU = x_sites<PX, NC, MODE != kFuseNone, sizeof(typename Io<C>::t)>();
+  for (RowWalk<TY> w(g.nx); w.r < TY;) {
+    int32_t idxs[kXU];
+    int rs[kXU], xs[kXU];
+    typename Io<C>::t pvs[kXU][NC];
+    [[maybe_unused]] float2 rvs[MODE == kFuseRV ? kXU : 1][NC];
 #pragma unroll
-   for (int u = 0; u < kXU; ++u)
-     pvs[u] = idxs[u] >= 0 ? p[((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u]] : typename Io<C>::t{};
-   [[maybe_unused]] float2 rvs[MODE == kFuseRV ? kXU : 1];
-   if constexpr (MODE == kFuseRV) {
+    for (int u = 0; u < kXU; ++u) {
+      rs[u] = w.r;
+      xs[u] = w.x;
+      const int y = y0 + w.r;
+      idxs[u] = (w.r < TY && w.x < g.nx && y < g.ny) ? __ldg(d.map + ((int64_t)z * g.ny + y) * g.nx + w.x) : -1;
+      w.next(g.nx);
+    }
 #pragma unroll
-     for (int u = 0; u < kXU; ++u)
-       rvs[u] = idxs[u] >= 0 ? kf->rhat[((int64_t)b * 3 + c0 + rs[u] / TY) * g.n + idxs[u]] : make_float2(0.f, 0.f);
-   }
+    for (int u = 0; u < kXU; ++u) {
 #pragma unroll
-   for (int u = 0; u < kXU; ++u) {
-    const int32_t idx = idxs[u];
-    if (idx < 0) continue;
-    const int cl = rs[u] / TY;
-    const C conv = in[rs[u] * ip + xs[u]];
-    const int c = c0 + cl;
-    const int64_t o = ((int64_t)b * 3 + c) * g.n + idx;
-    const int cc = d.comp ? d.comp[3 * idx + c] : 0;  // composition of axis c
-    C pv = io_get<C>(pvs[u]);
-    if (conj) pv = conjc(pv);
-    C res;
-    if (d.iat) {  // rotated dielectric frame: row c of the full symmetric alpha^{-1} of this site
-      const C* m6 = d.iat + ((int64_t)(rhs0 + b) * g.n + idx) * 6;
-      const int64_t oc = ((int64_t)b * 3) * g.n + idx;
-      res = conv;
-#pragma unroll
-      for (int c2 = 0; c2 < 3; ++c2) {
-        C q = io_get<C>(p[oc + (int64_t)c2 * g.n]);
-        if (conj) q = conjc(q);
-        const int lo = c < c2 ? c : c2, hi = c < c2 ? c2 : c;
-        res = cadd(res, cmul(m6[lo == 0 ? hi : (lo == 1 ? 2 + hi : 5)], q));
+      for (int c = 0; c < NC; ++c) {
+        const int64_t o = vec + (int64_t)c * g.n + idxs[u];
+        pvs[u][c] = idxs[u] >= 0 ? p[o] : typename Io<C>::t{};
+        if constexpr (MODE == kFuseRV) rvs[u][c] = idxs[u] >= 0 ? kf->rhat[o] : make_float2(0.f, 0.f);
       }
-    } else {
-      res = d.sc ? cadd(cmul(d.sc[((int64_t)b * g.ncomp + cc) * 3 + c], conv), pv)
-                 : cadd(conv, cmul(ia[cc * 3 + c], pv));
     }
-    ap[o] = io_put<C>(conj ? conjc(res) : res);
-    if constexpr (MODE == kFuseRV) {
-      kred::acc_cdot(dot, rvs[u], res);  // <rhat, v>
-    } else if constexpr (MODE == kFuseTS) {
-      kred::acc_cdot(dot, res, pv);      // <t, s>: the product's input is s
-      kred::acc_nrm(tt, res);            // |t|^2
+#pragma unroll
+    for (int u = 0; u < kXU; ++u) {
+      const int32_t idx = idxs[u];
+      if (idx < 0) continue;
+#pragma unroll
+      for (int cl = 0; cl < NC; ++cl) {
+        const C conv = in[(cl * TY + rs[u]) * ip + xs[u]];
+        const int c = c0 + cl;
+        C pv = io_get<C>(pvs[u][cl]);
+        if (conj) pv = conjc(pv);
+        C res;
+        if (d.iat) {  // rotated dielectric frame: row c of the full symmetric alpha^{-1} of this site
+          const C* m6 = d.iat + ((int64_t)(rhs0 + b) * g.n + idx) * 6;
+          const int64_t oc = ((int64_t)b * 3) * g.n + idx;
+          res = conv;
+#pragma unroll
+          for (int c2 = 0; c2 < 3; ++c2) {
+            C q = io_get<C>(p[oc + (int64_t)c2 * g.n]);
+            if (conj) q = conjc(q);
+            const int lo = c < c2 ? c : c2, hi = c < c2 ? c2 : c;
+            res = cadd(res, cmul(m6[lo == 0 ? hi : (lo == 1 ? 2 + hi : 5)], q));
+          }
+        } else {
+          const int cc = d.comp ? d.comp[3 * idx + c] : 0;  // composition of axis c
+          const C tb = !d.comp ? tab0[cl] : (d.sc ? d.sc[((int64_t)b * g.ncomp + cc) * 3 + c] : ia[cc * 3 + c]);
+          res = d.sc ? cadd(cmul(tb, conv), pv) : cadd(conv, cmul(tb, pv));
+        }
+        ap[vec + (int64_t)cl * g.n + idx] = io_put<C>(conj ? conjc(res) : res);
+        if constexpr (MODE == kFuseRV) {
+          kred::acc_cdot(dot, rvs[u][cl], res);  // <rhat, v>
+        } else if constexpr (MODE == kFuseTS) {
+          kred::acc_cdot(dot, res, pv);          // <t, s>: the product's input is s
+          kred::acc_nrm(tt, res);                // |t|^2
+        }
+      }
     }
-   }
   }
   if constexpr (MODE == kFuseRV) {
     float ah[2] = {dot.hi.x, dot.hi.y}, al[2] = {dot.lo.x, dot.lo.y};
@@ -1216,6 +1247,19 @@ inline int x_ty_pick(const MvTune& t, size_t csize, int px) {
   return (t.xty > 0 && x_ty_valid(csize, px, t.xty)) ? t.xty : x_ty_rt(csize, px);
 }
 
+// Tile of the x passes with folded solver updates.  Three components per CTA whatever the plain product
+// was tuned to: the folded vectors share each site's map entry and address, and a dot product is reduced
+// over a third of the CTAs (solves, one component -> three: 64 x 48 x 32, 2 RHS 2.97 -> 2.79 ms, 48^3,
+// 8 RHS 14.9 -> 13.6, 48^3, 32 RHS 50.9 -> 45.4, 64^3, 4 RHS 7.85 -> 7.43).  The default tile of 16 rows
+// where it gives two CTAs per SM or more, else 8 (16 -> 8 rows: 64 x 48 x 32, 192 -> 384 CTAs, 3.11 ->
+// 2.79 ms; 40^3, 240 -> 400, 1.92 -> 1.82; 32 x 64 x 64, 512 -> 1024, 2.55 -> 2.72).
+inline int xf_nc_pick(const MvTune& t, int px) { return t.xpin ? x_nc_pick(t, px) : (more_length(px) ? 1 : 3); }
+inline int xf_ty_pick(const Geom& g, const MvTune& t, int nrhs) {
+  if (t.xpin || more_length(g.px)) return x_ty_pick(t, sizeof(float2), g.px);
+  const int ty = x_ty_rt(sizeof(float2), g.px);
+  return ty > 8 && (int64_t)((g.ny + ty - 1) / ty) * g.nz * nrhs < 2 * 152 ? 8 : ty;
+}
+
 // z columns per CTA of the 5-pass z kernel: widest tile under ~110 KB of shared memory
 constexpr int zcols_g_rt(size_t csize, int pz) {
   return (size_t)pz * 3 * 32 * csize <= 110 * 1024 ? 32 : ((size_t)pz * 3 * 16 * csize <= 110 * 1024 ? 16 : 8);
@@ -1537,17 +1581,17 @@ Err launch_matvec_fast(const Geom& g, const MvData<C>& d, const MvTune& t, const
 
 // ------------------------------------------------------------------ BiCGstab half-iterations, folded (complex64)
 // x-pass CTAs per RHS of the schedule t (the reduction slots of the folded dot products)
-inline int x_ctas_per_rhs(const Geom& g, const MvTune& t) {
-  const int NC = x_nc_pick(t, g.px);
-  const int TY = x_ty_pick(t, sizeof(float2), g.px);
+inline int x_ctas_per_rhs(const Geom& g, const MvTune& t, int nrhs) {
+  const int NC = xf_nc_pick(t, g.px);
+  const int TY = xf_ty_pick(g, t, nrhs);
   return ((g.ny + TY - 1) / TY) * g.nz * (3 / NC);
 }
 
 template <int MODE, bool FWD>
 Err launch_x_fused(const Geom& g, const MvData<float2>& d, const MvTune& t, const KrylovVecs<float2>& kv, KState* ks,
                    const RedBuf& rbx, int nrhs, cudaStream_t st) {
-  const int NC = x_nc_pick(t, g.px);
-  const int TY = x_ty_pick(t, sizeof(float2), g.px);
+  const int NC = xf_nc_pick(t, g.px);
+  const int TY = xf_ty_pick(g, t, nrhs);
   const size_t sm = x_fast_smem<float2>(g, TY, NC);
   const dim3 grid((g.ny + TY - 1) / TY, g.nz, nrhs * (3 / NC));
   const int ip = odd_pitch(g.nx);
