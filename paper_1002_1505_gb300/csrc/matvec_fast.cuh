@@ -1044,6 +1044,22 @@ __global__ void __launch_bounds__(NT, (zcols_min_ctas<C, PZ, NT, NA>())) k_z_col
         xa[it][j] = (ok && zz < nz) ? wb[c * cstride + (int64_t)zz * g.ys + ky0 + gg] : czero<C>();
       }
     }
+    // Meanwhile the input of the CTA one per SM further on starts on its way from HBM to L2, so that
+    // its own loads meet L2 latency (256^3, 16 RHS 3.17 -> 2.98 ms, 192^3 1.31 -> 1.24, 160^3 0.717 ->
+    // 0.705; distances of 64 to 400 CTAs alike).  Not for 8-column tiles, whose rows are half a line
+    // (256 x 256 x 320, 32 RHS 7.11 -> 7.30).  A hint only: rows and columns of d.work, nothing is written.
+    if constexpr (G >= 16) {
+      const unsigned lin = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z) + 152;
+      const unsigned q = lin / gridDim.x, b2 = lin - q * gridDim.x;
+      const unsigned kx2 = q / gridDim.y, ky2 = (q - kx2 * gridDim.y) * G;
+      if (kx2 < gridDim.z) {
+        const C* w2 = d.work + ((int64_t)b2 * 3 * g.px + kx2) * ((int64_t)nz * g.ys) + ky2;
+        for (int i = threadIdx.x; i < 3 * nz; i += NT) {
+          const int c = (i >= nz) + (i >= 2 * nz), zz = i - c * nz;
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(w2 + c * cstride + (int64_t)zz * g.ys));
+        }
+      }
+    }
 #pragma unroll
     for (int it = 0; it < kItA; ++it) {
       const int i = threadIdx.x + it * NT;
