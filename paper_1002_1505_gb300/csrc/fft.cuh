@@ -223,6 +223,11 @@ __device__ __forceinline__ void dif_stage(C* s, const Batch& b, int L, int Ls, c
     for (int j = 0; j < R; ++j) v[j] = base[j * m * b.estride];
     Dft<R, -1, C>::run(v);
     base[0] = v[0];
+    if (m == 1) {  // sub-blocks of R: every twiddle is 1 (in FP64 the products are a third of the stage)
+#pragma unroll
+      for (int k = 1; k < R; ++k) base[k * b.estride] = v[k];
+      continue;
+    }
 #pragma unroll
     for (int k = 1; k < R; ++k) base[k * m * b.estride] = cmul(v[k], tw[n1 * k * tws]);
   }
@@ -243,8 +248,13 @@ __device__ __forceinline__ void dit_stage(C* s, const Batch& b, int L, int Ls, c
     C* base = s + p * b.pstride + (blk * Ls + n1) * b.estride;
     C v[R];
     v[0] = base[0];
+    if (m == 1) {
 #pragma unroll
-    for (int k = 1; k < R; ++k) v[k] = cmulc(base[k * m * b.estride], tw[n1 * k * tws]);
+      for (int k = 1; k < R; ++k) v[k] = base[k * b.estride];
+    } else {
+#pragma unroll
+      for (int k = 1; k < R; ++k) v[k] = cmulc(base[k * m * b.estride], tw[n1 * k * tws]);
+    }
     Dft<R, 1, C>::run(v);
 #pragma unroll
     for (int j = 0; j < R; ++j) base[j * m * b.estride] = v[j];

@@ -305,7 +305,7 @@ __global__ void k_fft_strided(C* data, int64_t estride, int64_t ninner, int64_t 
     s[e * ti + ii] = (ii < ni) ? base[e * estride + ii] : czero<C>();
   }
   __syncthreads();
-  const Batch bt{ti, 1, ti, true};
+  const Batch bt{ni, 1, ti, true};  // the pencils that exist: Px/2 + 1 of them leave one in the last tile
   if (inverse) fft_inverse(s, bt, pl, L, tw);
   else fft_forward(s, bt, pl, L, tw);
   for (int i = threadIdx.x; i < L * ti; i += blockDim.x) {
@@ -331,7 +331,8 @@ __global__ void k_fft_strided(C* data, int64_t estride, int64_t ninner, int64_t 
 //   y: T1 = xx + xy, T2 = yy + yz, T3 = xz, T4 = zz
 //   z: F1 = xx + xz, F2 = yy + yz, F3 = xy, F4 = zz
 // Measured on 128 x 96 x 64 (one component per transform before, each value converted at each use):
-// fill 54 -> 30 us, transforms 227 -> 165, expansions 18 -> 17, pack 105 -> 47.
+// fill 54 -> 30 us, transforms 227 -> 165 (135 with the launch sizes of fft_threads, no products by 1
+// in the last stage and no empty pencils), expansions 18 -> 17, pack 105 -> 47.
 
 __device__ __forceinline__ bool odd_in(int c, int axis) {
   // bit a of the mask = odd in axis a (0 = x, 1 = y, 2 = z)
@@ -668,6 +669,11 @@ unsigned long long launches() { return g_launches.load(); }
 void add_launches(unsigned long long n) { g_launches += n; }
 void sub_launches(unsigned long long n) { g_launches -= n; }
 
+// Threads for a tile of `elems` elements in the FP64 transforms of the Green tensor: one radix-8
+// butterfly each.  The stages wait on FP64 latency, and at 66 to 74 registers a 256-thread CTA of which
+// 64 have work leaves an SM with six busy warps; small CTAs fill it.
+static int fft_threads(size_t elems) { return (int)std::min<size_t>(256, std::max<size_t>(64, (elems / 8 + 31) / 32 * 32)); }
+
 template <typename C>
 Err fft_rows(C* data, int64_t nrows, int64_t row_stride, const FftPlan& pl, const C* tw, int nin, int nout,
              bool inverse, cudaStream_t st) {
@@ -675,7 +681,7 @@ Err fft_rows(C* data, int64_t nrows, int64_t row_stride, const FftPlan& pl, cons
   const size_t sr = sizeof(C) * ((size_t)pl.L + (size_t)rpb * (pl.L + 1));
   DDA_TRY(set_smem(sr));
   const unsigned nb = (unsigned)((nrows + rpb - 1) / rpb);
-  k_fft_rows<C><<<nb, 256, sr, st>>>(data, nrows, row_stride, pl, tw, nin, nout, rpb, inverse);
+  k_fft_rows<C><<<nb, fft_threads((size_t)rpb * pl.L), sr, st>>>(data, nrows, row_stride, pl, tw, nin, nout, rpb, inverse);
   DDA_CU(cudaGetLastError());
   g_launches += 1;
   return Err::Ok();
@@ -688,7 +694,7 @@ Err fft_strided(C* data, int L, int64_t estride, int64_t ninner, int64_t nouter,
   const size_t sm = sizeof(C) * ((size_t)L + (size_t)L * ti);
   DDA_TRY(set_smem(sm));
   dim3 grid((unsigned)((ninner + ti - 1) / ti), (unsigned)nouter);
-  k_fft_strided<C><<<grid, 256, sm, st>>>(data, estride, ninner, outer_stride, pl, tw, ti, inverse);
+  k_fft_strided<C><<<grid, fft_threads((size_t)ti * L), sm, st>>>(data, estride, ninner, outer_stride, pl, tw, ti, inverse);
   DDA_CU(cudaGetLastError());
   g_launches += 1;
   return Err::Ok();
