@@ -266,7 +266,8 @@ DDA_API dda_status dda_matvec(dda_ctx *ctx, const void *p_dev, void *ap_dev, int
  * library holds those 32 MiB until the process exits.  Requests whose scratch
  * (sizeof(complex) x 3 x Px x Nz x Ys per RHS, Ys = Ny on the 3-pass schedule,
  * Py on the 5-pass one) exceeds 32 MiB return DDA_EINVAL with the sizes in the
- * message.  The call makes no cudaMalloc, cudaFree or other allocating call.
+ * message (a grid whose only compile-time schedule has 5 passes falls back to the
+ * general 3-pass kernel first, where that fits).  The call makes no cudaMalloc, cudaFree or other allocating call.
  * The array's device address is looked up once per device, with that device
  * current, by the first dda_build_green_fft on the device (a prerequisite of
  * this call; the array sits in the same device module as the Green-tensor
@@ -407,7 +408,7 @@ DDA_API dda_status dda_profile_matvec(dda_ctx *ctx, int nrhs, int dtype, int ite
  * first product for a given RHS count times the candidate schedules and keeps
  * the fastest) or pinned by the DDA_SCHEDULE environment variable at
  * dda_build_green_fft time ("generic", "fast5", "plane512", "plane768",
- * "cluster2", "cluster4"; DDA_XTILE = 4, 8 or 16 pins the x passes' tile
+ * "cluster2", "cluster4", "half256", "half384"; DDA_XTILE = 4, 8 or 16 pins the x passes' tile
  * height; DDA_BULK = 1 or 0 pins bulk-copy staging of the plane pass;
  * DDA_XCOMP = 1 runs the x passes with one field component per CTA).
  * info[0] = passes (3 = fused y-z plane, 5 = split), info[1] = 1 when the
@@ -419,7 +420,7 @@ DDA_API dda_status dda_profile_matvec(dda_ctx *ctx, int nrhs, int dtype, int ite
  * HBM blocks with bulk copies (TMA), info[7] = field components per CTA of the
  * x passes (3 or 1; 0 for the generic engine), info[8] = 1 when the 5-pass z
  * columns run pass B, the Ghat multiply and the inverse pass B of the three
- * components in registers (a tuner candidate for long z transforms); info[9..11]
+ * components in registers on 8 columns per CTA (a tuner candidate for Pz = 160); info[9..11]
  * are reserved (0). */
 DDA_API dda_status dda_schedule_info(dda_ctx *ctx, int dtype, int32_t info[12]);
 
