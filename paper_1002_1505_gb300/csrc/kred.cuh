@@ -45,7 +45,9 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2)
 
 // Block sum of NS pairs, blockDim.x = 256: the warps' sums stay in pairs (an FP64 shuffle tree of three
 // values costs a CTA of eight warps 1900 issue cycles at 1/64 of the FP32 rate, this one 300), then one
-// warp adds the eight warps' sums of all values in FP64; result in out (doubles, NS <= 4).
+// warp adds the eight warps' sums of all values in FP64; result in out (doubles, NS <= 4).  Lanes 0, 8, ..
+// of that warp store a value each; its closing __syncwarp orders their stores before whatever thread 0 does
+// next, so that a fence and a release by thread 0 alone publish all of them.
 template <int NS>
 __device__ __forceinline__ void block_sum_pairs(float (&h)[NS], float (&l)[NS], double* out) {
   __shared__ double red[NS * 8];
@@ -62,6 +64,7 @@ __device__ __forceinline__ void block_sum_pairs(float (&h)[NS], float (&l)[NS], 
     double x = threadIdx.x < NS * 8 ? red[threadIdx.x] : 0.0;
     for (int o = 4; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o, 8);
     if (threadIdx.x % 8 == 0 && threadIdx.x < NS * 8) out[threadIdx.x / 8] = x;
+    __syncwarp();
   }
 }
 
