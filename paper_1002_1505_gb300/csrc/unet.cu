@@ -29,7 +29,6 @@
 
 #include <algorithm>
 #include <array>
-#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -986,6 +985,7 @@ struct dda_unet {
   cudaEvent_t ev = nullptr;            // the mask sum's copy has arrived
   bool use_tc = true;                  // convolutions on tcgen05 (DDA_UNET_TC=0: mma.sync throughout)
   unsigned int* d_fault = nullptr;     // set when a bounded tensor-core wait gave up
+  uint32_t opted = 0;                  // kernels opted in to large shared memory on this device (smem_optin)
   std::vector<std::pair<std::array<int, 6>, dda::nn::TcTile>> tiles;  // tc_tile's answers by shape
   uint4* xb = nullptr;                 // bfloat16 copy of a tcgen05 convolution's input
   size_t xb_bytes = 0;
@@ -1127,14 +1127,13 @@ Err encode_act_map(CUtensorMap* m, const void* base, int cpad, const dda::nn::Di
   return Err::Ok();
 }
 
-// opt k_conv_tc<NP> in to the full 227 KB of dynamic shared memory (once per instantiation)
-template <int NP>
-Err tc_smem_optin() {
-  static bool done = false;
-  if (!done) {
-    DDA_CU(cudaFuncSetAttribute(dda::nn::k_conv_tc<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    done = true;
-  }
+// Opt a kernel in to `bytes` of dynamic shared memory.  The attribute belongs to the current device, so it
+// is kept with the network (which has one device) and not with the process; bit says which kernel.
+template <typename K>
+Err smem_optin(dda_unet* n, K* kern, int bytes, uint32_t bit) {
+  if (n->opted & bit) return Err::Ok();
+  DDA_CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  n->opted |= bit;
   return Err::Ok();
 }
 
@@ -1152,7 +1151,7 @@ Err conv_planes(dda_unet* n, const dda_unet::Layer& L, const uint4* xp, const dd
   switch (np16(cout)) {
 #define CASE(NP)                                                                                                    \
   case NP:                                                                                                          \
-    DDA_TRY(tc_smem_optin<NP>());                                                                                   \
+    DDA_TRY(smem_optin(n, dda::nn::k_conv_tc<NP>, 227 * 1024, 1u << (NP / 16)));                                    \
     dda::nn::k_conv_tc<NP><<<grid, dda::nn::kTcThreads, smem, n->stream>>>(tmap, wt, kc_n, transposed, bias, out,   \
                                                                            cout, relu, d, tl, n->d_fault);          \
     break;
@@ -1281,11 +1280,7 @@ Err wgrad(dda_unet* n, const dda_unet::Layer& L, const float* x, int xs, const u
   switch (L.nt_n) {
 #define CASE(NT)                                                                                                     \
   case NT: {                                                                                                         \
-    static std::atomic<bool> done{false};                                                                            \
-    if (!done) {                                                                                                     \
-      DDA_CU(cudaFuncSetAttribute(dda::nn::k_wgrad<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024));   \
-      done = true;                                                                                                   \
-    }                                                                                                                \
+    DDA_TRY(smem_optin(n, dda::nn::k_wgrad<NT>, 112 * 1024, 1u << (16 + NT)));                                       \
     dda::nn::k_wgrad<NT><<<grid, dda::nn::kWgT, sm, n->stream>>>(x, xs, xp, L.cin, gy, mask, gs, L.cout, L.taps, d, t, \
                                                                  n->part, gbp, L.kc_n);                              \
     break;                                                                                                           \
