@@ -342,12 +342,26 @@ dda::RedBuf redbuf(dda_ctx* c, int nrhs, int64_t n3) {
 }
 
 // The far-field buffers: nrd (RHS, direction) pairs of directions and sums, scratch, phase tables, in one
-// allocation of at least 8 MB, so that a context's first observables usually need one cudaMalloc.
+// allocation of at least 8 MB, so that a context's first observables usually need one cudaMalloc.  The
+// context keeps up to kFarKept of it; more goes back at the end of the call (FarHold).
+constexpr size_t kFarKept = (size_t)64 << 20;
+struct FarHold {
+  dda_ctx* c;
+  ~FarHold() {
+    size_t& cap = cap_of(c, (void**)&c->d_far);
+    if (cap <= kFarKept) return;
+    cudaFree(c->d_far);  // waits for the work that uses it
+    c->d_far = nullptr;
+    cap = 0;
+  }
+};
 Err far_buffers(dda_ctx* c, size_t nrd, size_t scratch_doubles, size_t tab_bytes) {
   auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t nh = al(sizeof(double) * 3 * nrd), F = al(sizeof(double2) * 3 * nrd);
   const size_t part = al(sizeof(double) * scratch_doubles);
+  const auto gen = c->gen;
   DDA_TRY(grow(c, &c->d_far, std::max<size_t>(nh + F + part + al(tab_bytes), (size_t)8 << 20)));
+  c->gen = gen;  // no captured iteration holds this buffer
   c->d_nh = reinterpret_cast<double*>(c->d_far);
   c->d_F = reinterpret_cast<double2*>(c->d_far + nh);
   c->d_fpart = reinterpret_cast<double*>(c->d_far + nh + F);
@@ -1926,7 +1940,8 @@ dda_status dda_cross_sections(dda_ctx* c, const void* p_dev, double* q_out, cons
       }
       const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
       const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
-      e = far_buffers(c, (size_t)nrhs * ndir, dda::farfield_scratch(nrhs, ndir, c->n, box, nblk), 0);
+      FarHold hold{c};
+      e = far_buffers(c, (size_t)nrhs * ndir, dda::farfield_scratch(nrhs, c->iorth, ndir, c->n, box, nblk), 0);
       double2* d_F = c->d_F;
       if (e.ok()) {
         e = cuda_ok(cudaMemcpy(c->d_nh, nh.data(), sizeof(double) * nh.size(), cudaMemcpyHostToDevice),
@@ -2035,7 +2050,8 @@ dda_status dda_periodic_scattering(dda_ctx* c, const void* p_dev, int n_spec, co
     for (int b = 0; b < nrhs; ++b) std::copy(nd.begin(), nd.end(), nh.begin() + (size_t)b * ndir * 3);
     const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>((c->n + 2047) / 2048, 64));
     const int box[3] = {c->tgt.box[0], c->tgt.box[1], c->tgt.box[2]};
-    e = far_buffers(c, (size_t)nrhs * ndir, dda::farfield_scratch(nrhs, ndir, c->n, box, nblk), 0);
+    FarHold hold{c};
+    e = far_buffers(c, (size_t)nrhs * ndir, dda::farfield_scratch(nrhs, c->iorth, ndir, c->n, box, nblk), 0);
     if (e.ok())
       e = cuda_ok(cudaMemcpy(c->d_nh, nh.data(), sizeof(double) * nh.size(), cudaMemcpyHostToDevice),
                   "direction upload");
@@ -2302,6 +2318,7 @@ dda_status dda_angular_averages(dda_ctx* c, const void* p_dev, double eta, doubl
       nl[3 * d + 1] = std::sin(t) * std::cos(f);
       nl[3 * d + 2] = std::sin(t) * std::sin(f);
     }
+    FarHold hold{c};
     e = far_buffers(c, (size_t)per * ndir, plan.part_doubles, plan.tab_bytes);
     std::vector<double> nh((size_t)per * ndir * 3);
     std::vector<double2> F((size_t)per * ndir * 3);

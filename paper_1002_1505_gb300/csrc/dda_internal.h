@@ -367,7 +367,7 @@ Err qsums(const uint8_t* comp, const double2* einc /*[nrhs][3][N]*/, const doubl
 // F[rhs][dir][3] = sum_j P_j exp(-i kd n_dir . r_j), FP64; ndir directions per RHS (nhat
 // [nrhs][ndir][3] in TF, the same for the iorth RHS of an orientation); map: box -> site;
 // scratch: farfield_scratch doubles.
-size_t farfield_scratch(int nrhs, int ndir, int64_t n, const int box[3], int nblk);
+size_t farfield_scratch(int nrhs, int iorth, int ndir, int64_t n, const int box[3], int nblk);
 Err farfield(const int32_t* ijk, const int32_t* map, const double* origin3, const double* nhat, double kd,
              const double2* p, int nrhs, int iorth, int ndir, int64_t n, const int box[3], double2* out,
              double* scratch, int nblk, cudaStream_t st);

@@ -156,16 +156,17 @@ __global__ void k_far(const int32_t* ijk, const double* org, const double* nhat,
   bred<6>(acc, part + (((int64_t)b * ndir + d) * gridDim.x + blockIdx.x) * 6);
 }
 
-__global__ void k_far_fin(const double* part, int nblk, double2* out) {
-  const int o = blockIdx.x;  // rhs * ndir + dir
+// out[rhs][d0 + d] = the block partials of directions d0 .. d0 + nd - 1 in order; grid nrhs * nd
+__global__ void k_far_fin(const double* part, int nblk, int nd, int ndir, int d0, double2* out) {
+  const int64_t o = blockIdx.x, b = o / nd;  // rhs * nd + dir
   double v[6] = {0, 0, 0, 0, 0, 0};
   for (int i = threadIdx.x; i < nblk; i += blockDim.x)
-    for (int s = 0; s < 6; ++s) v[s] += part[((int64_t)o * nblk + i) * 6 + s];
+    for (int s = 0; s < 6; ++s) v[s] += part[(o * nblk + i) * 6 + s];
   __shared__ double res[6];
   bred<6>(v, res);
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int c = 0; c < 3; ++c) out[(int64_t)o * 3 + c] = make_double2(res[2 * c], res[2 * c + 1]);
+    for (int c = 0; c < 3; ++c) out[(b * ndir + d0 + o - b * nd) * 3 + c] = make_double2(res[2 * c], res[2 * c + 1]);
 }
 
 // ------------------------------------------------------------------ many scattering directions
@@ -928,15 +929,26 @@ Err qsums_tensor(const double2* einc, const double2* iat, double kd, const doubl
   return Err::Ok();
 }
 
-// row blocks of the row-wise far field, and the doubles of scratch `farfield` needs (phase tables of
-// the row-wise path, then the partials)
+// row blocks of the row-wise far field
 static int far_row_blocks(const int box[3]) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)box[1] * box[2] + kFarT - 1) / kFarT, 512));
 }
-size_t farfield_scratch(int nrhs, int ndir, int64_t n, const int box[3], int nblk) {
-  if (!far_by_rows(n, box, kRowsMost64)) return (size_t)6 * nrhs * ndir * nblk;
-  const size_t nt = (size_t)(box[0] + 1) / 2 + box[1] + box[2];
-  return (size_t)2 * nrhs * ndir * nt + (size_t)6 * nrhs * ndir * far_row_blocks(box);
+static bool far_rows64(int nrhs, int64_t n, const int box[3]) { return far_by_rows(n, box, kRowsMost64) && nrhs <= 65535; }
+// Its scratch for one direction: a column of the phase tables of each direction set, and the row blocks'
+// partials of each RHS.  Directions beyond kFarScratch's worth take further passes, in whole direction
+// groups: a pass of 64 MiB is thousands of CTAs, and with 32 RHS, 2000 directions and a 111 x 128 x 160 box
+// the scratch of a single pass was 0.84 GB.
+static size_t far_rows64_doubles(int nrhs, int iorth, const int box[3]) {
+  return (size_t)2 * (nrhs / iorth) * ((box[0] + 1) / 2 + box[1] + box[2]) + (size_t)6 * nrhs * far_row_blocks(box);
+}
+constexpr size_t kFarScratch = (size_t)64 << 20;
+static int far_rows64_dirs(int nrhs, int iorth, int ndir, const int box[3]) {
+  const size_t fit = kFarScratch / sizeof(double) / far_rows64_doubles(nrhs, iorth, box);
+  return (int)std::min<size_t>({(size_t)ndir, std::max<size_t>(1, fit / kFarDirs) * kFarDirs, (size_t)65535 * kFarDirs});
+}
+size_t farfield_scratch(int nrhs, int iorth, int ndir, int64_t n, const int box[3], int nblk) {
+  if (!far_rows64(nrhs, n, box)) return (size_t)6 * nrhs * ndir * nblk;
+  return far_rows64_doubles(nrhs, iorth, box) * far_rows64_dirs(nrhs, iorth, ndir, box);
 }
 
 Err farfield(const int32_t* ijk, const int32_t* map, const double* origin3, const double* nhat, double kd,
@@ -944,26 +956,29 @@ Err farfield(const int32_t* ijk, const int32_t* map, const double* origin3, cons
              double* scratch, int nblk, cudaStream_t st) {
   const size_t sm = sizeof(double2) * (size_t)(box[0] + box[1] + box[2]);
   if (sm > 48 * 1024) return Err::make(DDA_EUNSUPPORTED, "target box too long for the far-field phase tables");
-  if (far_by_rows(n, box, kRowsMost64) && ndir <= 65535 * kFarDirs && nrhs <= 65535) {
+  if (far_rows64(nrhs, n, box)) {
     const int nx = box[0], ny = box[1], nz = box[2], U = (nx + 1) / 2, sets = nrhs / iorth;
-    const int nrb = far_row_blocks(box);
-    double2* tab = reinterpret_cast<double2*>(scratch);
-    double* part = scratch + 2 * (size_t)sets * ndir * (U + ny + nz);
+    const int nrb = far_row_blocks(box), per = far_rows64_dirs(nrhs, iorth, ndir, box);
     auto runs = [](int v) { return (v + kRun64 - 1) / kRun64; };
-    k_row_tables<double2, kRun64><<<dim3((unsigned)((ndir + 31) / 32), runs(U) + runs(ny) + runs(nz), sets), 32, 0, st>>>(
-        nhat, iorth, ndir, ndir, origin3, kd, nx, ny, nz, tab);
-    DDA_CU(cudaGetLastError());
-    k_far_rows64<<<dim3(nrb, (ndir + kFarDirs - 1) / kFarDirs, nrhs), kFarT, sizeof(double2) * U * kFarDirs, st>>>(
-        map, p, n, nx, ny, nz, ndir, iorth, tab, part);
-    DDA_CU(cudaGetLastError());
-    k_far_fin<<<nrhs * ndir, kT, 0, st>>>(part, nrb, out);
-    DDA_CU(cudaGetLastError());
-    add_launches(3);
+    for (int d0 = 0; d0 < ndir; d0 += per) {
+      const int nd = std::min(per, ndir - d0);
+      double2* tab = reinterpret_cast<double2*>(scratch);
+      double* part = scratch + 2 * (size_t)sets * nd * (U + ny + nz);
+      k_row_tables<double2, kRun64><<<dim3((unsigned)((nd + 31) / 32), runs(U) + runs(ny) + runs(nz), sets), 32, 0, st>>>(
+          nhat + (size_t)3 * d0, iorth, ndir, nd, origin3, kd, nx, ny, nz, tab);
+      DDA_CU(cudaGetLastError());
+      k_far_rows64<<<dim3(nrb, (nd + kFarDirs - 1) / kFarDirs, nrhs), kFarT, sizeof(double2) * U * kFarDirs, st>>>(
+          map, p, n, nx, ny, nz, nd, iorth, tab, part);
+      DDA_CU(cudaGetLastError());
+      k_far_fin<<<(unsigned)(nrhs * (int64_t)nd), kT, 0, st>>>(part, nrb, nd, ndir, d0, out);
+      DDA_CU(cudaGetLastError());
+      add_launches(3);
+    }
     return Err::Ok();
   }
   k_far<<<dim3(nblk, ndir, nrhs), kT, sm, st>>>(ijk, origin3, nhat, kd, p, ndir, n, box[0], box[1], box[2], scratch);
   DDA_CU(cudaGetLastError());
-  k_far_fin<<<nrhs * ndir, kT, 0, st>>>(scratch, nblk, out);
+  k_far_fin<<<nrhs * ndir, kT, 0, st>>>(scratch, nblk, ndir, ndir, 0, out);
   DDA_CU(cudaGetLastError());
   add_launches(2);
   return Err::Ok();
