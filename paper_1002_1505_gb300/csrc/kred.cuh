@@ -2,14 +2,16 @@
 // rather than by a vector loop: each CTA reduces its products into one slot of
 // a partial-sum table, and the last CTA of a right-hand side to arrive (a
 // device-scope counter) sums that RHS's slots in a fixed order.  The scheme and
-// the double-float product accumulation are those of the Krylov vector kernels
-// (krylov.cu), so fused and unfused iterations reduce alike.
+// the double-float product accumulation of a thread are those of the Krylov
+// vector kernels (krylov.cu); across a warp those add in FP64 and the folded
+// passes in three floats (sum3.cuh), so the two differ in the last bits of FP64.
 #pragma once
 
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "dda_internal.h"
+#include "sum3.cuh"
 
 namespace dda {
 namespace kred {
@@ -43,25 +45,28 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float h2, float l2)
   h = s;
 }
 
-// Block sum of NS pairs, blockDim.x = 256: the warps' sums stay in pairs (an FP64 shuffle tree of three
-// values costs a CTA of eight warps 1900 issue cycles at 1/64 of the FP32 rate, this one 300), then one
-// warp adds the eight warps' sums of all values in FP64; result in out (doubles, NS <= 4).  Lanes 0, 8, ..
-// of that warp store a value each; its closing __syncwarp orders their stores before whatever thread 0 does
-// next, so that a fence and a release by thread 0 alone publish all of them.
+// Block sum of NS pairs, blockDim.x = 256.  The warps' sums are carried in three floats (Sum3), which keep
+// more than the FP64 shuffle tree that they stand for: that tree runs at 1/64 of the FP32 rate and costs a
+// CTA 1900 issue cycles for three values of eight warps.  (A tree of pairs keeps fewer bits than FP64, and
+// three floats cost next to nothing more: a 64 x 48 x 32 solve takes 4.169 ms with them, 4.163 with pairs.)
+// Then one warp turns the eight warps' sums of all values into FP64 and adds them; result in out (doubles,
+// NS <= 4).  Lanes 0, 8, .. of that warp store a value each; its closing __syncwarp orders their stores
+// before whatever thread 0 does next, so that a fence and a release by thread 0 alone publish all of them.
 template <int NS>
 __device__ __forceinline__ void block_sum_pairs(float (&h)[NS], float (&l)[NS], double* out) {
-  __shared__ double red[NS * 8];
-#pragma unroll
-  for (int s = 0; s < NS; ++s)
-    for (int o = 16; o > 0; o >>= 1)
-      pair_add(h[s], l[s], __shfl_down_sync(0xffffffffu, h[s], o), __shfl_down_sync(0xffffffffu, l[s], o));
+  __shared__ Sum3 red[NS * 8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0)
 #pragma unroll
-    for (int s = 0; s < NS; ++s) red[s * 8 + w] = (double)h[s] + (double)l[s];
+  for (int s = 0; s < NS; ++s) {
+    Sum3 v{h[s], l[s], 0.f};
+    for (int o = 16; o > 0; o >>= 1)
+      v.add(Sum3{__shfl_down_sync(0xffffffffu, v.h, o), __shfl_down_sync(0xffffffffu, v.l, o),
+                 __shfl_down_sync(0xffffffffu, v.t, o)});
+    if (lane == 0) red[s * 8 + w] = v;
+  }
   __syncthreads();
   if (threadIdx.x < 32) {
-    double x = threadIdx.x < NS * 8 ? red[threadIdx.x] : 0.0;
+    double x = threadIdx.x < NS * 8 ? red[threadIdx.x].get() : 0.0;
     for (int o = 4; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o, 8);
     if (threadIdx.x % 8 == 0 && threadIdx.x < NS * 8) out[threadIdx.x / 8] = x;
     __syncwarp();

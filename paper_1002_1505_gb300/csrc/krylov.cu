@@ -47,7 +47,9 @@ __device__ __forceinline__ double nrm_acc(double acc, double2 a) { return acc + 
 // vectors: a double-float pair (Dekker/Knuth): each product is split exactly
 // into p + pe with one FMA, added with the two-sum, so a thread's partial keeps
 // about 48 bits using FP32 instructions only (the FP64 pipe of this GPU is too
-// slow to keep up with memory); partials are combined in FP64 from the warp up.
+// slow to keep up with memory); partials are combined in FP64 from the warp up
+// (in the folded passes and k_bicg_xr of complex64 in three floats across a warp,
+// kred.cuh, then in FP64).
 template <typename C> struct Acc;
 template <> struct Acc<double2> {
   double v = 0.0;

@@ -1,5 +1,6 @@
 """The device reductions run on the host, thread by thread (tests/native): what a CTA announces to the
-others has to be stored by then, in any order in which its threads may have run."""
+others has to be stored by then, in any order in which its threads may have run, and a sum that FP64
+adds exactly has to come out exactly."""
 import os
 import shutil
 import subprocess
@@ -26,6 +27,11 @@ def run_native(name, tmp_path):
     res = subprocess.run(cmd, capture_output=True, text=True)
     assert res.returncode == 0, res.stderr[-3000:]
     return subprocess.run([exe], capture_output=True, text=True, timeout=120)
+
+
+def test_sums_keep_the_bits_of_fp64(tmp_path):
+    res = run_native("reduction_bits", tmp_path)
+    assert res.returncode == 0, res.stdout
 
 
 def test_slot_is_stored_before_it_is_announced(tmp_path):
