@@ -324,15 +324,21 @@ __global__ void k_fft_strided(C* data, int64_t estride, int64_t ninner, int64_t 
 // only what they do not determine: offsets n_x >= 0 are evaluated, the x transforms run on the rows
 // with y <= Py/2, z <= Pz/2, the y transforms on the planes z <= Pz/2 for natural kx <= Px/2, the z
 // transforms on natural kx <= Px/2, ky <= Py/2, and the missing parts are mirrored in between and in
-// the final pack.  And along each axis an even and an odd component go through one transform: of the
-// sum s = a + b, A(k) = (S(k) + S(-k))/2 and B(k) = (S(k) - S(-k))/2, so six components take four
+// the final pack.  And along each axis an even and an odd off-diagonal component go through one transform:
+// of the sum s = a + b, A(k) = (S(k) + S(-k))/2 and B(k) = (S(k) - S(-k))/2, so six components take five
 // transforms per axis:
-//   x: S1 = xx + xy, S2 = yy + xz, S3 = yz, S4 = zz
-//   y: T1 = xx + xy, T2 = yy + yz, T3 = xz, T4 = zz
-//   z: F1 = xx + xz, F2 = yy + yz, F3 = xy, F4 = zz
-// Measured on 128 x 96 x 64 (one component per transform before, each value converted at each use):
-// fill 54 -> 30 us, transforms 227 -> 165 (135 with the launch sizes of fft_threads, no products by 1
-// in the last stage and no empty pencils), expansions 18 -> 17, pack 105 -> 47.
+//   x: S1 = yz + xy, S2 = xz, then xx, yy, zz
+//   y: T1 = xz + xy, T2 = yz, then xx, yy, zz
+//   z: F1 = xy + xz, F2 = yz, then xx, yy, zz
+// Each half carries the rounding of the whole, so only components of one size are paired: an off-diagonal
+// one with a diagonal one (four transforms) raises the tensor's error by a tenth, as the diagonal ones of
+// the nearest sites are several times larger.
+// Measured on 128 x 96 x 64 (one component per transform before, each value converted at each use): incidence,
+// tensor, alpha, field and a first product 541 -> 376 us (351 with four transforms).  Error of complex128
+// products on 90 x 54 x 80, three draws: 3.7, 4.3, 4.0e-16 with a transform per component (and the general
+// engine's product), 4.4, 4.9, 4.7e-16 with diagonal and off-diagonal pairs, 3.8, 4.2, 3.8e-16 like this.
+// Components that vanish for boxes of one layer are packed as zeros: such a box's in-plane and normal
+// dipoles do not act on each other.
 
 __device__ __forceinline__ bool odd_in(int c, int axis) {
   // bit a of the mask = odd in axis a (0 = x, 1 = y, 2 = z)
@@ -340,8 +346,8 @@ __device__ __forceinline__ bool odd_in(int c, int axis) {
   return (mask[c] >> axis) & 1;
 }
 
-// q[j][zq][yq][x], j = S1 .. S4, for zq <= Pz/2, yq <= Py/2 and all x (offsets wrapped along x): a thread
-// evaluates one offset n_x >= 0 and writes it and its mirror image
+// q[j][zq][yq][x], j = S1, S2, xx, yy, zz, for zq <= Pz/2, yq <= Py/2 and all x (offsets wrapped along x): a
+// thread evaluates one offset n_x >= 0 and writes it and its mirror image
 __global__ void k_green_fill_q(Geom g, double kd, double2* q) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
   const int64_t Q = (int64_t)g.px * hy1 * hz1, N = (int64_t)hx1 * hy1 * hz1;
@@ -374,16 +380,18 @@ __global__ void k_green_fill_q(Geom g, double kd, double2* q) {
       }
     }
     double2* row = q + rest * g.px;
-    row[x] = cadd(out[0], out[1]);
-    row[Q + x] = cadd(out[3], out[2]);
-    row[2 * Q + x] = out[4];
-    row[3 * Q + x] = out[5];
+    row[x] = cadd(out[4], out[1]);
+    row[Q + x] = out[2];
+    row[2 * Q + x] = out[0];
+    row[3 * Q + x] = out[3];
+    row[4 * Q + x] = out[5];
     const int xm = x ? g.px - x : 0;
     if (xm != x) {
-      row[xm] = csub(out[0], out[1]);
-      row[Q + xm] = csub(out[3], out[2]);
-      row[2 * Q + xm] = out[4];
-      row[3 * Q + xm] = out[5];
+      row[xm] = csub(out[4], out[1]);
+      row[Q + xm] = make_double2(-out[2].x, -out[2].y);
+      row[2 * Q + xm] = out[0];
+      row[3 * Q + xm] = out[3];
+      row[4 * Q + xm] = out[5];
     }
   }
 }
@@ -393,7 +401,7 @@ __device__ __forceinline__ double2 half_diff(double2 a, double2 b) { return make
 
 // After the x transform only the natural frequencies kx <= Px/2 are carried on; the spectra are in the
 // engine's digit-reversed storage order, st*[k] = storage position of natural frequency k.
-// t[j][zq][y][k], j = T1 .. T4 (all y, k <= Px/2), from q[j][zq][yq][storage]: rows y > Py/2 mirror Py - y
+// t[j][zq][y][k], j = T1, T2, xx, yy, zz (all y, k <= Px/2), from q[j][zq][yq][storage]: rows y > Py/2 mirror Py - y
 __global__ void k_green_expand_y(Geom g, const int32_t* __restrict__ stx, const double2* __restrict__ q,
                                  double2* __restrict__ t) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
@@ -405,17 +413,18 @@ __global__ void k_green_expand_y(Geom g, const int32_t* __restrict__ stx, const 
     const bool mir = y > g.py / 2;
     const double2* row = q + ((int64_t)z * hy1 + (mir ? g.py - y : y)) * g.px;
     const int p = stx[k], m = stx[k ? g.px - k : 0];
-    const double2 s2 = row[Q + p], s2m = row[Q + m], yz = row[2 * Q + p];
-    const double2 yy = half_sum(s2, s2m);
-    t[i] = row[mir ? m : p];  // xx + xy, or xx - xy
-    t[T + i] = mir ? csub(yy, yz) : cadd(yy, yz);
-    t[2 * T + i] = half_diff(s2, s2m);
+    const double2 s1 = row[p], s1m = row[m], xz = row[Q + p];
+    const double2 yz = half_sum(s1, s1m), xy = half_diff(s1, s1m);
+    t[i] = mir ? csub(xz, xy) : cadd(xz, xy);
+    t[T + i] = mir ? make_double2(-yz.x, -yz.y) : yz;
+    t[2 * T + i] = row[2 * Q + p];
     t[3 * T + i] = row[3 * Q + p];
+    t[4 * T + i] = row[4 * Q + p];
   }
 }
 
-// f[j][z][kx][ky], j = F1 .. F4 (all z; natural kx <= Px/2, ky <= Py/2), from t[j][zq][storage][kx]: planes
-// z > Pz/2 mirror Pz - z.  ky runs fastest, for the pack below.
+// f[j][z][kx][ky], j = F1, F2, xx, yy, zz (all z; natural kx <= Px/2, ky <= Py/2), from t[j][zq][storage][kx]:
+// planes z > Pz/2 mirror Pz - z.  ky runs fastest, for the pack below.
 __global__ void k_green_expand_z(Geom g, const int32_t* __restrict__ sty, const double2* __restrict__ t,
                                  double2* __restrict__ f) {
   const int hx1 = g.px / 2 + 1, hy1 = g.py / 2 + 1, hz1 = g.pz / 2 + 1;
@@ -427,12 +436,13 @@ __global__ void k_green_expand_z(Geom g, const int32_t* __restrict__ sty, const 
     const bool mir = z > g.pz / 2;
     const double2* pl = t + (int64_t)(mir ? g.pz - z : z) * g.py * hx1 + kx;
     const int64_t p = (int64_t)sty[ky] * hx1, m = (int64_t)sty[ky ? g.py - ky : 0] * hx1;
-    const double2 t1 = pl[p], t1m = pl[m], xz = pl[2 * T + p];
-    const double2 xx = half_sum(t1, t1m);
-    f[i] = mir ? csub(xx, xz) : cadd(xx, xz);
-    f[F + i] = pl[T + (mir ? m : p)];  // yy + yz, or yy - yz
-    f[2 * F + i] = half_diff(t1, t1m);
+    const double2 t1 = pl[p], t1m = pl[m], yz = pl[T + p];
+    const double2 xz = half_sum(t1, t1m), xy = half_diff(t1, t1m);
+    f[i] = mir ? csub(xy, xz) : cadd(xy, xz);
+    f[F + i] = mir ? make_double2(-yz.x, -yz.y) : yz;
+    f[2 * F + i] = pl[2 * T + p];
     f[3 * F + i] = pl[3 * T + p];
+    f[4 * F + i] = pl[4 * T + p];
   }
 }
 
@@ -455,15 +465,17 @@ __device__ __forceinline__ void ghat_put(const double2 (&w)[6], int kx, int kz, 
 }
 
 // xx .. zz at natural kx <= Px/2, ky <= Py/2 and storage positions (kzs, kzm) of (kz, -kz), times inv
-__device__ __forceinline__ void green_parts(const double2* __restrict__ f, int64_t F, int64_t P, int64_t at, int kzs,
-                                            int kzm, double inv, double2 (&w)[6]) {
-  const double2 a = f[kzs * P + at], am = f[kzm * P + at], b = f[F + kzs * P + at], bm = f[F + kzm * P + at];
-  w[0] = half_sum(a, am);
-  w[1] = f[2 * F + kzs * P + at];
-  w[2] = half_diff(a, am);
-  w[3] = half_sum(b, bm);
-  w[4] = half_diff(b, bm);
-  w[5] = f[3 * F + kzs * P + at];
+__device__ __forceinline__ void green_parts(const Geom& g, const double2* __restrict__ f, int64_t F, int64_t P,
+                                            int64_t at, int kzs, int kzm, double inv, double2 (&w)[6]) {
+  const double2 a = f[kzs * P + at], am = f[kzm * P + at];
+  const double2 zero = make_double2(0.0, 0.0);
+  const bool x1 = g.nx == 1, y1 = g.ny == 1, z1 = g.nz == 1;
+  w[0] = f[2 * F + kzs * P + at];
+  w[1] = x1 || y1 ? zero : half_sum(a, am);
+  w[2] = x1 || z1 ? zero : half_diff(a, am);
+  w[3] = f[3 * F + kzs * P + at];
+  w[4] = y1 || z1 ? zero : f[F + kzs * P + at];
+  w[5] = f[4 * F + kzs * P + at];
 #pragma unroll
   for (int c = 0; c < 6; ++c) w[c] = make_double2(w[c].x * inv, w[c].y * inv);
 }
@@ -486,7 +498,7 @@ __global__ void __launch_bounds__(128) k_green_pack(Geom g, const int32_t* __res
   const double inv = 1.0 / ((double)g.px * g.py * g.pz);
   for (int ky = threadIdx.x; ky < hy1; ky += blockDim.x) {
     double2 w[6];
-    green_parts(f, F, P, (int64_t)kx * hy1 + ky, stz[kz], stz[kzm], inv, w);
+    green_parts(g, f, F, P, (int64_t)kx * hy1 + ky, stz[kz], stz[kzm], inv, w);
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       sg[c * hy1 + ky] = w[c];
@@ -749,21 +761,21 @@ Err build_green(const Geom& g, double kd, const double2* twx, const double2* twy
   double2* q = gw;
   k_green_fill_q<<<nblk((int64_t)hx1 * hy1 * hz1), 256, 0, st>>>(g, kd, q);
   if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green fill failed");
-  if (e.ok()) e = fft_rows<double2>(q, 4 * (int64_t)hy1 * hz1, g.px, g.plx, twx, g.px, g.px, false, st);
+  if (e.ok()) e = fft_rows<double2>(q, 5 * (int64_t)hy1 * hz1, g.px, g.plx, twx, g.px, g.px, false, st);
   // t (in the ghat128 buffer, free until the pack): planes z <= Pz/2, all y, natural kx <= Px/2
   double2* t = ghat128;
   if (e.ok()) {
     k_green_expand_y<<<nblk(T), 256, 0, st>>>(g, stx, q, t);
     if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green expand (y) failed");
   }
-  if (e.ok()) e = fft_strided<double2>(t, g.py, hx1, hx1, 4 * (int64_t)hz1, (int64_t)hx1 * g.py, g.ply, twy, false, st);
+  if (e.ok()) e = fft_strided<double2>(t, g.py, hx1, hx1, 5 * (int64_t)hz1, (int64_t)hx1 * g.py, g.ply, twy, false, st);
   // f (in gw): all z, natural ky <= Py/2, kx <= Px/2; z columns transformed
   if (e.ok()) {
     k_green_expand_z<<<nblk(F), 256, 0, st>>>(g, sty, t, gw);
     if (cudaGetLastError() != cudaSuccess) e = Err::make(DDA_ECUDA, "Green expand (z) failed");
   }
   if (e.ok())
-    e = fft_strided<double2>(gw, g.pz, (int64_t)hx1 * hy1, (int64_t)hx1 * hy1, 4, F, g.plz, twz, false, st);
+    e = fft_strided<double2>(gw, g.pz, (int64_t)hx1 * hy1, (int64_t)hx1 * hy1, 5, F, g.plz, twz, false, st);
   if (e.ok()) {
     const size_t sm = (size_t)hy1 * 6 * (sizeof(double2) + sizeof(float4));  // < the y transforms' 272 py bytes
     k_green_pack<<<dim3(hz1, hx1), 128, sm, st>>>(g, naty, stx, stz, gw, ghat128, ghat64, ghatdf);
