@@ -23,7 +23,7 @@ def run_native(name, tmp_path):
     exe = os.path.join(tmp_path, name)
     src = os.path.join(ROOT, "tests", "native", name + ".cpp")
     inc = [os.path.join(ROOT, "paper_1002_1505_gb300", "csrc"), os.path.join(ROOT, "include"), cuda_include()]
-    cmd = ["g++", "-std=c++17", "-O1", "-ffp-contract=off", "-w", "-o", exe, src] + ["-I" + i for i in inc]
+    cmd = ["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-w", "-o", exe, src] + ["-I" + i for i in inc]
     res = subprocess.run(cmd, capture_output=True, text=True)
     assert res.returncode == 0, res.stderr[-3000:]
     return subprocess.run([exe], capture_output=True, text=True, timeout=120)
