@@ -39,6 +39,7 @@
 
 #include "bulk.cuh"
 #include "dda_internal.h"
+#include "sum3.cuh"
 
 namespace dda {
 namespace nn {
@@ -459,7 +460,7 @@ __global__ void k_pack_tc(const float* __restrict__ w, int taps, int cin, int co
 // voxels a warp loads the gradient's fragments once (ldmatrix, transposed: voxels are the K axis of
 // both operands) and one input fragment per tap.  Rows are padded so that eight rows 16 bytes wide fall
 // on different banks.  part[tile][tap][kc*16 + row][NT*8]; the chunk-0 CTAs also sum the unrounded
-// gradient per channel (pair sums, then FP64): gbp[tile][NT*8].  Latency and staging bound; one CTA per
+// gradient per channel (in three floats, which hold more than FP64, then FP64): gbp[tile][NT*8].  Latency and staging bound; one CTA per
 // (4096 voxels, tap) with gathers straight from memory took 1.5 of the 2.6 ms of a training pass of 16
 // 16^3 samples and the channel sums 0.35, these kernels and their sums
 // about 0.25.
@@ -472,7 +473,7 @@ constexpr int kWgXS = 48;  // bytes per staged input row: 16 channels and a pad 
 __host__ __device__ constexpr int wg_gs(int NT) { return (NT % 2 ? NT : NT + 1) * 16; }
 __host__ inline size_t wg_smem(const WgTile& t, int NT) {
   const size_t main = (size_t)t.rows * kWgXS + (size_t)t.Kpad * wg_gs(NT) + (size_t)t.Kpad * 4;
-  const size_t red = sizeof(double) * (size_t)kWgT * 8 + sizeof(float) * 9 * 16 * NT * 8;
+  const size_t red = sizeof(float) * (3 * (size_t)kWgT * 8 + 9 * 16 * NT * 8);
   return (main > red ? main : red) + 16;
 }
 __device__ __forceinline__ void ldsm_x4t(uint32_t (&r)[4], uint32_t addr) {
@@ -546,9 +547,9 @@ __global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int
                   (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
   constexpr int NG = kWgT / NT;
   const int nt0 = tid % NT, vg = tid / NT;
-  float bh[8], bl[8];
+  Sum3 bs[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) bh[j] = bl[j] = 0.f;
+  for (int j = 0; j < 8; ++j) bs[j] = Sum3{0.f, 0.f, 0.f};
   if (vg < NG)
     for (int k = vg; k < tl.Kpad; k += NG) {
       const int xx = k % tl.Tx, q = k / tl.Tx;
@@ -568,11 +569,7 @@ __global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int
       // padding voxels (zero gradient) take the first voxel's rows, so that shifted rows stay in the tile
       if (nt0 == 0) off[k] = k < tl.K ? ((zz + hal) * sy + yy + hal) * sx + xx + hal : (hal * sy + hal) * sx + hal;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float s = __fadd_rn(bh[j], f[j]), w = __fsub_rn(s, bh[j]);
-        bl[j] = __fadd_rn(bl[j], __fadd_rn(__fsub_rn(bh[j], __fsub_rn(s, w)), __fsub_rn(f[j], w)));
-        bh[j] = s;
-      }
+      for (int j = 0; j < 8; ++j) bs[j].add(f[j]);
     }
   __syncthreads();
   const uint32_t xa = tc_saddr(xt) + ((lane >> 3) & 1) * 16, ga = tc_saddr(gt);
@@ -620,8 +617,8 @@ __global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int
     }
   }
   __syncthreads();  // the staged tiles are read; their memory holds the reductions now
-  double* red = reinterpret_cast<double*>(sm_wg);  // [NG][NT * 8]
-  float* wred = reinterpret_cast<float*>(red + kWgT * 8);
+  float* red = reinterpret_cast<float*>(sm_wg);  // the bias sums: [3][NG][NT * 8]
+  float* wred = red + 3 * kWgT * 8;
   if (!hal) {
 #pragma unroll
     for (int n = 0; n < NT; ++n)
@@ -631,7 +628,12 @@ __global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int
   }
   if (kc == 0 && vg < NG) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) red[vg * (NT * 8) + nt0 * 8 + j] = (double)bh[j] + (double)bl[j];
+    for (int j = 0; j < 8; ++j) {
+      float* r = red + vg * (NT * 8) + nt0 * 8 + j;
+      r[0] = bs[j].h;
+      r[NG * NT * 8] = bs[j].l;
+      r[2 * NG * NT * 8] = bs[j].t;
+    }
   }
   __syncthreads();
   if (!hal) {
@@ -645,8 +647,12 @@ __global__ void __launch_bounds__(kWgT) k_wgrad(const float* __restrict__ x, int
   if (kc == 0) {
     for (int i = tid; i < NT * 64; i += kWgT) {  // eight lanes per channel
       const int c = i >> 3;
-      double v = 0.0;
-      for (int k = i & 7; k < NG; k += 8) v += red[k * (NT * 8) + c];
+      Sum3 b{0.f, 0.f, 0.f};
+      for (int k = i & 7; k < NG; k += 8) {
+        const float* r = red + k * (NT * 8) + c;
+        b.add(Sum3{r[0], r[NG * NT * 8], r[2 * NG * NT * 8]});
+      }
+      double v = isfinite(b.h) ? b.get() : (double)b.h;  // an overflow's rounding errors are not numbers
       for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
       if ((i & 7) == 0) gbp[(int64_t)tile * (NT * 8) + c] = v;
     }
