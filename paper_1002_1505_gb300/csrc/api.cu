@@ -592,12 +592,9 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
     DDA_CU(cudaEventCreate(&e1));
     float best_ms = 1e30f, last_ms = 1e30f;
     Err err = Err::Ok();
-    // one warm-up product, then `reps` timed between events on the context's stream
-    auto time_one = [&](const dda::MvTune& t, int reps = 3) {
+    // `reps` products between events on the context's stream, the mean in last_ms
+    auto products = [&](int reps) {
       last_ms = 1e30f;
-      apply_tune<C>(c, t);
-      err = matvec<C>(c, p, ap, nrhs, 0, false);
-      if (!err.ok()) return;
       cudaEventRecord(e0, c->stream);
       for (int r = 0; r < reps && err.ok(); ++r) err = matvec<C>(c, p, ap, nrhs, 0, false);
       cudaEventRecord(e1, c->stream);
@@ -605,28 +602,47 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
       cudaEventSynchronize(e1);
       cudaEventElapsedTime(&last_ms, e0, e1);
       last_ms /= reps;
+    };
+    auto keep = [&](const dda::MvTune& t) {
       if (last_ms < best_ms) { best_ms = last_ms; best = t; }
     };
-    std::vector<float> ms(cand.size(), 1e30f);
-    for (size_t i = 0; i < cand.size() && err.ok(); ++i) {
-      time_one(cand[i]);
-      ms[i] = last_ms;
-    }
-    // short products differ by less than three of them show: the candidates within 15 % of the best are
-    // timed twice more, and the least time of each counts
-    if (err.ok() && best_ms < 0.2f) {
-      const float line = 1.15f * best_ms;
-      for (int round = 0; round < 2; ++round)
-        for (size_t i = 0; i < cand.size() && err.ok(); ++i)
+    // One warm-up product (it loads the kernels), one timed, which rules out what is far from the best, and two
+    // more.  The first starts on an idle stream, which a short product shows and a long one does not.
+    auto time_one = [&](const dda::MvTune& t) {
+      last_ms = 1e30f;
+      apply_tune<C>(c, t);
+      err = matvec<C>(c, p, ap, nrhs, 0, false);
+      if (!err.ok()) return;
+      products(1);
+      if (!err.ok() || last_ms > 1.3f * best_ms) return;
+      const float one = last_ms;
+      products(2);
+      if (err.ok() && one >= 0.2f) last_ms = (one + 2 * last_ms) / 3;
+      keep(t);
+    };
+    // Short products differ by less than a few of them show, so those within 8 % of the best are timed again,
+    // up to three times where launches are most of a product, and the least time of each counts.  The first
+    // product of a grid pays for all this: 64 x 48 x 32 with 2 RHS 3.1 ms, a sphere of 12 1.1 (8.2 and 1.6 with
+    // up to three rounds of six products; the schedules picked are as fast).
+    auto time_all = [&](const std::vector<dda::MvTune>& list) {
+      std::vector<float> ms(list.size(), 1e30f);
+      for (size_t i = 0; i < list.size() && err.ok(); ++i) {
+        time_one(list[i]);
+        ms[i] = last_ms;
+      }
+      const float line = 1.08f * best_ms;
+      for (int round = best_ms < 0.02f ? 3 : (best_ms < 0.2f ? 1 : 0); round > 0; --round)
+        for (size_t i = 0; i < list.size() && err.ok(); ++i)
           if (ms[i] <= line) {
-            time_one(cand[i], 5);
-            ms[i] = std::min(ms[i], last_ms);
+            apply_tune<C>(c, list[i]);
+            products(3);
+            keep(list[i]);
           }
-    }
+    };
+    time_all(cand);
     // then the x passes' tile height for the chosen schedule (short tiles give small batches more CTAs)
-    // and one component per CTA (smaller tiles in shared memory, longer rows per store); short products
-    // again in three rounds (64 x 48 x 32, 2 RHS: the shapes take 34.6 to 40 us, and one round picked
-    // the 39 us one in some runs)
+    // and one component per CTA (smaller tiles in shared memory, longer rows per store); 64 x 48 x 32,
+    // 2 RHS: the shapes take 34.6 to 40 us
     if (err.ok()) {
       std::vector<dda::MvTune> shapes;
       for (int ty : {4, 8}) {
@@ -638,10 +654,7 @@ Err ensure_tuned(dda_ctx* c, int nrhs) {
       shapes.push_back(best);
       shapes.back().xnc = 1;
       shapes.back().xty = 0;
-      const bool brief = best_ms < 0.2f;
-      if (brief) shapes.push_back(best);
-      for (int round = 0; round < (brief ? 3 : 1); ++round)
-        for (size_t i = 0; i < shapes.size() && err.ok(); ++i) time_one(shapes[i], brief ? 5 : 3);
+      time_all(shapes);
     }
     // the 5-pass z columns with their middle stages fused in registers (long pass-B sub-blocks)
     if (err.ok() && sizeof(C) == sizeof(float2) && !best.plane && dda::zcols_rfuse_available_c64(g0)) {

@@ -460,10 +460,9 @@ __global__ void k_pack_tc(const float* __restrict__ w, int taps, int cin, int co
 // voxels a warp loads the gradient's fragments once (ldmatrix, transposed: voxels are the K axis of
 // both operands) and one input fragment per tap.  Rows are padded so that eight rows 16 bytes wide fall
 // on different banks.  part[tile][tap][kc*16 + row][NT*8]; the chunk-0 CTAs also sum the unrounded
-// gradient per channel (in three floats, which hold more than FP64, then FP64): gbp[tile][NT*8].  Latency and staging bound; one CTA per
-// (4096 voxels, tap) with gathers straight from memory took 1.5 of the 2.6 ms of a training pass of 16
-// 16^3 samples and the channel sums 0.35, these kernels and their sums
-// about 0.25.
+// gradient per channel (in three floats, which hold more than FP64, then FP64): gbp[tile][NT*8].  Latency
+// and staging bound; one CTA per (4096 voxels, tap) with gathers straight from memory took 1.5 of the 2.6 ms
+// of a training pass of 16 16^3 samples and the channel sums 0.35, these kernels and their sums about 0.25.
 constexpr int kWgT = 288;
 struct WgTile {
   int Tx, Ty, Tz, ntx, nty, ntz;
