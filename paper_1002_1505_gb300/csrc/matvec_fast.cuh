@@ -28,7 +28,7 @@
 // include this header.  Everything length-dependent then lives in namespace fast_more instead of fast.
 // Grids with a length of the second set run the 5-pass schedule with one component per x-pass CTA,
 // nothing to tune; on the general engine a 90 x 54 x 80 grid with 2 RHS took 109 us in complex64 and
-// 901 us in complex128, here 44 and 508.
+// 901 us in complex128, here 33.7 and 498.
 #define DDA_CORE_LENGTHS(X) X(16) X(24) X(32) X(40) X(48) X(64) X(80) X(96) X(128) X(160) X(192) X(256) X(320)
 #define DDA_MORE_LENGTHS(X) \
   X(18) X(20) X(30) X(36) X(50) X(54) X(60) X(72) X(90) X(100) X(108) X(120) X(144) X(150) X(162) X(180) X(200) X(216) X(240) X(288)
@@ -54,7 +54,7 @@ using f2::Shape;
 template <typename C>
 __device__ __forceinline__ C conjc(C a) { a.y = -a.y; return a; }
 
-// one Ghat record (GhatAt, dda_internal.h): the six components sit in 16-byte pieces one row of ky
+// one Ghat record (ghat_at, dda_internal.h): the six components sit in 16-byte pieces one row of ky
 // apart, so that consecutive ky load consecutive 16-byte words
 template <typename C>
 __device__ __forceinline__ void load6(const C* __restrict__ gh, int64_t at, int py, C (&g)[6]) {
@@ -977,7 +977,8 @@ __global__ void __launch_bounds__(256) k_y_rows(Geom g, C* __restrict__ work, co
 // (kFuse) where the sub-blocks are short enough; else pass B and the multiply go through shared
 // memory.  NA = 2 takes two stages after the radix 2 into pass A (radix 16), which shortens the
 // sub-blocks of the long transforms to 8 and 10 elements so that they fuse (256 x 256 x 320, 32 RHS:
-// 8.40 -> 7.87 ms; with the coalesced Ghat pieces 7.62 ms).
+// 8.40 -> 7.87 ms; with the coalesced Ghat pieces 7.62, with packed FP32 sums 7.11, with both parts of the
+// twiddles (twc, fft2.cuh) 7.44).
 template <typename C, int PZ, int G, int NA>
 constexpr int zcols_pad() {
   // complex64: a warp's column group spans 2G words; when that is under the 32 banks, place

@@ -322,9 +322,10 @@ struct PairSum {
 // Many directions, FP32 products.  A thread owns two directions, a CTA 2 kRowT directions of one set
 // and a run of rows, staged in shared memory as P+ and P- pairs that every thread reads by broadcast;
 // a row's sum is FP32 (at most half the box's x length of terms), rows are added in pair sums.
-// Bound by FP32 issue and the broadcasts (48 FMAs per 6 LDS.128): 131,072 sites x 2292 directions x 2
-// polarizations in 0.28 ms, where the site kernel took 7.66 ms (three table lookups and two complex
-// products per site and direction, and 48 FP64 block sums per CTA at 1/64 of the FP32 rate).
+// No one unit bounds it: issue 59 %, FMA 44 %, load write-back (the broadcasts) 46 % with 15 warps per SM.
+// 131,072 sites x 2292 directions x 2 polarizations in 0.28 ms, where the site kernel took 7.66 ms (three
+// table lookups and two complex products per site and direction, and 48 FP64 block sums per CTA at 1/64 of
+// the FP32 rate).
 // grid (nblk, ndp / (2 kRowT), nsets); part[set][blk][nb * 6][ndp].
 constexpr int kRowT = 128;
 template <int NB>
@@ -867,7 +868,7 @@ Err farfield_many(const int32_t* ijk, const int32_t* map, const double* origin3,
     k_row_tables<float2, kRun><<<dim3((unsigned)((f.ndp + 127) / 128), runs(U) + runs(ny) + runs(nz), sets), 128, 0, st>>>(
         nhat, f.nb, ndir, (int)f.ndp, origin3, kd, nx, ny, nz, tab);
     DDA_CU(cudaGetLastError());
-    // rows staged at a time: about 24 KB (one row of the longest box, 384 pairs, takes 36 KB)
+    // rows staged at a time: about 24 KB (one row of the longest box, 350 pairs, takes 33.6 KB)
     const size_t row_bytes = sizeof(float4) * (size_t)U * f.nb * 3;
     const int rb = (int)std::max<size_t>(1, std::min<size_t>(32, 24576 / row_bytes));
     const size_t sm = rb * row_bytes + sizeof(int) * rb;
